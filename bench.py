@@ -359,8 +359,7 @@ def run_ours(args):
     ms, job_n = reduce_ranks(ms, float(total_n), dev)
     value = job_n / (ms / 1e3)
     ms_step = ms / args.steps
-    # roofline of the dominant (only) kernel: k_fused_ws (the pipelined
-    # insert, the default at this table size), one launch per step
+    # roofline of the dominant (only) kernel: k_fused, one launch per step
     mean_n = total_n / args.steps
     mean_c = sum(cells) / len(cells)
     alg = algorithmic_bytes(int(mean_n), int(mean_c))
@@ -421,7 +420,7 @@ def run_ours(args):
                        "parallelism": f"replicas x{ws} (independent frame streams)"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "peak_source": peak_kind, "kernel": "k_fused_ws",
+                         "peak_source": peak_kind, "kernel": "k_fused",
                          "algorithmic_bytes_per_launch": alg},
             "gpu_launches": args.steps,
             "clocks": clk.summary(),
@@ -441,7 +440,7 @@ def run_ours(args):
         if merge:
             line["merge_modes"] = {
                 "workload": "the headline HD frames (temporal and plain) with each warp "
-                            "aggregation of the pipelined insert (pps_tuning.merge): none, "
+                            "aggregation of the insert (pps_tuning.merge): none, "
                             "gated (__match_any_sync where neighbouring lanes repeat a key; "
                             "the default), always", **merge}
         if precision:

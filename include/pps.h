@@ -214,9 +214,8 @@ typedef struct pps_camera {
  *             Algorithm 1) hashed last into both hashes: vertices share a cell
  *             only if their extra words are equal.  NULL: none.  Use the same
  *             choice for every call on a table in a frame.
- * pps_filter runs frames with dist or extra through the split kernels (the
- * persistent launch is built without them); pps_batch_create,
- * pps_filter_noalloc and the host-buffer calls reject them.
+ * pps_batch_create, pps_filter_noalloc and the host-buffer calls reject dist
+ * and extra.
  * All nine float arrays are required.  16-byte-aligned arrays are read with
  * 128-bit loads; other alignments take a scalar path.
  */
@@ -260,33 +259,19 @@ typedef struct pps_stats_t {
 /*
  * Launch shape of a table's kernels (no effect on results up to the order of
  * FP32 additions; fixed-point results are identical).
- *  batch      per-thread insert: vertices each thread carries through one
- *             insert step together (their probes and atomics overlap): 2 or 4;
- *             0 = library default (2).  Also used by the split kernels and the
- *             batched launch.
- *  insert     how pps_filter's persistent launch inserts: 0 = library default
- *             (pipelined while the slot index fits in L2, T <= 2^23; per
- *             thread for larger tables), 1 = per thread (each thread builds its vertices'
- *             keys, then probes and accumulates them), 2 = pipelined (key
- *             warps build keys, merge equal ones within the warp as `merge`
- *             says and queue one entry per group in shared memory; probe
- *             warps run the table operations of four queued keys per thread
- *             at once).  Frames
- *             with an evicting history or the neighborhood fallback always
- *             insert per thread.
- *  key_warps  pipelined insert: key warps of the 16 warps of a CTA (the rest
- *             probe): 4, 8 or 12; 0 = library default (8).
+ *  batch      vertices each lane carries through one insert step together
+ *             (their keys and probes overlap): 2 or 4; 0 = library default (2).
+ *  insert     0, 1 or 2: accepted, without effect (one insert serves every
+ *             table).
+ *  key_warps  0, 4, 8 or 12: accepted, without effect.
  *  block      batched launch (taken from the first view's table): threads
- *             per CTA, 256 or 512; 0 = library default (512).  Each CTA
- *             takes tiles of 2,048 vertices, 2048 / block per thread.
- *  merge      pipelined insert: warp aggregation of equal keys before they are
- *             queued: 0 = library default (2); 1 = none, one queue entry per
- *             vertex; 2 = merge with __match_any_sync (the lowest lane of each
- *             group of equal keys leads, the others add their contributions
- *             to its entry) in the warps where two neighbouring lanes hold
- *             equal keys, and skip the match elsewhere (coherent primary hits
- *             repeat keys across neighbouring pixels; secondary bounces
- *             rarely repeat one within a warp); 3 = merge in every warp.
+ *             per CTA, 256 or 512; 0 = library default (512).
+ *  merge      equal keys within a row of 32 consecutive vertices go through
+ *             the table once: 0 = library default (2); 1 = never; 2 = in the
+ *             rows where two neighbouring vertices hold equal keys, which one
+ *             shuffle and a vote find (coherent primary hits repeat keys across
+ *             neighbouring pixels; secondary bounces rarely repeat one within
+ *             a row); 3 = in every row.
  *  reserved   must be zero.
  */
 typedef struct pps_tuning {
@@ -365,9 +350,9 @@ int pps_query(pps_table *t, const pps_vertices *v, size_t n, const uint32_t *slo
 
 /*
  * pps_filter: the whole frame in one persistent cooperative launch: build,
- * insert, [blend if blend != 0], query and the per-frame clear, separated by
- * grid-wide barriers, with each vertex's cell index kept on chip (shared
- * memory) or, for large n, in a library-owned scratch buffer.  Results equal
+ * insert, [blend if blend != 0] and query, separated by
+ * grid-wide barriers, with each vertex's cell index kept in a library-owned
+ * scratch buffer.  Results equal
  * pps_build + pps_insert + [pps_blend] + pps_query.  The table is left ready
  * for the next frame.  Errors: PPS_EINVAL, PPS_ENOMEM, PPS_ECUDA.
  */
@@ -430,7 +415,7 @@ int pps_keys(pps_table *t, const pps_vertices *v, size_t n, uint32_t *h_out, uin
  * pps_filter on a table created from `p` (FP32 atomics: equal up to
  * summation order).
  *  - Working memory is one static device array inside the library (about
- *    26 MB), held by every GPU that loads the library until the process exits.
+ *    33 MB), held by every GPU that loads the library until the process exits.
  *    Limits: log2_slots <= 20 and n <= 524,288; larger requests, another
  *    accum_mode, or a history return PPS_EINVAL.
  *  - The first call in a CUDA context (the device's primary context, that

@@ -68,10 +68,10 @@ struct pps_table {
   uint32_t frame_tiles = 0;  // split path: tiles (cell-id blocks) used this frame
   pps_tuning tune{};         // launch shape (batch width 0 = library default)
   size_t D = 0;              // capacity of the dense cell arrays
-  uint32_t* gstash = nullptr;
-  size_t gstash_cap = 0;
-  uint32_t* split_ids = nullptr;  // pps_filter on the split kernels: each vertex's cell id
-  size_t split_ids_cap = 0;
+  uint32_t* stash = nullptr;  // [D] the vertices' cell ids during a call
+  // The slots still hold the last frame of a persistent launch, which empties
+  // them before it uses them: nothing else may read them before empty_slots.
+  bool stale = false;
   uint32_t* neigh_q = nullptr;  // neighborhood search: queue of low-count vertices
   size_t neigh_q_cap = 0;
   void* stage = nullptr;  // pps_filter_host device staging
@@ -194,50 +194,53 @@ bool temporal(const pps_table* t) { return t->p.hist_mode != PPS_HIST_NONE; }
 
 int batch_of(const pps_table* t) { return t->tune.batch == 4 ? 4 : 2; }
 
-// The library default: the pipelined insert while the slot index fits in L2
-// with the accumulators (T <= 2^23 slots, 64 MB); beyond that the table's
-// operations go to DRAM and the per-thread insert, whose every thread probes,
-// was measured faster (stress workload, T = 2^26: 9.6 vs 10.5 ms per frame).
-pps::InsertShape insert_shape(const pps_table* t) {
-  pps::InsertShape s;
-  const bool big = t->T > (1u << 23);
-  s.pipelined = t->tune.insert == 2 || (t->tune.insert == 0 && !big) ? 1 : 0;
-  s.key_warps = t->tune.key_warps ? static_cast<int>(t->tune.key_warps) : 8;
-  s.merge = t->tune.merge ? static_cast<int>(t->tune.merge) : 2;
-  return s;
+int merge_of(const pps_table* t) { return t->tune.merge ? static_cast<int>(t->tune.merge) : 2; }
+
+// Empty the slot table: of the split path's frame, or of what a persistent
+// launch left.
+int empty_slots(pps_table* t, cudaStream_t st) {
+  if (t->stale)
+    PPS_CUDA(cudaMemsetAsync(t->dev.slots, 0, t->T * sizeof(unsigned long long), st));
+  else if (t->state != kClean)
+    PPS_CUDA(pps::launch_clear(t->dev, t->frame_tiles, st));
+  t->stale = false;
+  return PPS_OK;
 }
 
-// Empty the cells of the split path's frame (the fused path leaves none behind)
-// and reset the frame counters.
-int reset_frame(pps_table* t, cudaStream_t st) {
-  if (t->state != kClean) {
-    PPS_CUDA(pps::launch_clear(t->dev, t->frame_tiles, st));
-    t->frame_tiles = 0;
-    t->state = kClean;
+// Begin a frame: reset its counters and, unless its launch empties the whole
+// slot table itself (`swept`), the slots.
+int reset_frame(pps_table* t, bool swept, cudaStream_t st) {
+  if (!swept) {
+    if (int rc = empty_slots(t, st)) return rc;
+  } else if (t->state != kClean) {
+    t->stale = true;
   }
+  t->frame_tiles = 0;
+  t->state = kClean;
   PPS_CUDA(cudaMemsetAsync(t->dev.ctrl, 0, pps::kCtrlFrameBytes, st));
   return PPS_OK;
 }
 
 // Make the dense cell arrays hold at least `need` cells, keeping the first
-// `keep` cells (accumulators, cell info, tile counts and quantized keys).  New accumulators
-// start at zero.
+// `keep` cells (accumulators, cell info, tile counts and quantized keys),
+// and the stash as many vertices.
 int ensure_dense(pps_table* t, size_t need, size_t keep, cudaStream_t st) {
   if (need <= t->D) return PPS_OK;
-  if (need > 0xFFFFFFF0ull) return fail(PPS_EINVAL, "more than 2^32 - 16 cells in one frame");
+  constexpr size_t kMost = 0x7FFFFFF0ull;  // the stash words' top bit marks a cell's creator
+  if (need > kMost) return fail(PPS_EINVAL, "more than 2^31 - 16 cells in one frame");
   size_t cap = t->D ? t->D : 1;
   while (cap < need) cap *= 2;
-  if (cap > 0xFFFFFFF0ull) cap = 0xFFFFFFF0ull;
+  if (cap > kMost) cap = kMost;
   const size_t acc_b = t->dev.fixed ? 32 : 16;
   const size_t nb = cap / 4 + 16;  // tile counts: one per block of >= 4 cells
-  void *acc = nullptr, *info = nullptr, *bc = nullptr, *kw = nullptr, *hold = nullptr;
+  void *acc = nullptr, *info = nullptr, *bc = nullptr, *kw = nullptr, *hold = nullptr, *ids = nullptr;
   cudaError_t e = cudaMalloc(&acc, cap * acc_b);
   if (e == cudaSuccess) e = cudaMalloc(&info, cap * sizeof(uint4));
   if (e == cudaSuccess) e = cudaMalloc(&bc, nb * sizeof(uint32_t));
   if (e == cudaSuccess && (t->dev.hist_migrate || t->dev.normal_search))
     e = cudaMalloc(&kw, cap * sizeof(uint4));
   if (e == cudaSuccess && t->dev.hist_migrate) e = cudaMalloc(&hold, cap * sizeof(float4));
-  if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, cap * acc_b, st);
+  if (e == cudaSuccess) e = cudaMalloc(&ids, cap * sizeof(uint32_t));
   void* old_acc = t->dev.fixed ? static_cast<void*>(t->dev.acc64) : static_cast<void*>(t->dev.acc);
   if (e == cudaSuccess && keep) {
     e = cudaMemcpyAsync(acc, old_acc, keep * acc_b, cudaMemcpyDeviceToDevice, st);
@@ -256,6 +259,7 @@ int ensure_dense(pps_table* t, size_t need, size_t keep, cudaStream_t st) {
     cudaFree(bc);
     cudaFree(kw);
     cudaFree(hold);
+    cudaFree(ids);
     cudaGetLastError();
     return fail(PPS_ENOMEM, std::string("dense cell arrays: ") + cudaGetErrorString(e));
   }
@@ -264,6 +268,8 @@ int ensure_dense(pps_table* t, size_t need, size_t keep, cudaStream_t st) {
   cudaFree(t->dev.bcount);
   cudaFree(t->dev.kw);
   cudaFree(t->dev.hold);
+  cudaFree(t->stash);
+  t->stash = static_cast<uint32_t*>(ids);
   t->dev.kw = static_cast<uint4*>(kw);
   t->dev.hold = static_cast<float4*>(hold);
   if (t->dev.fixed)
@@ -294,8 +300,7 @@ void free_all(pps_table* t) {
   cudaFree(t->dev.hold);
   cudaFree(t->dev.hcells);
   cudaFree(t->dev.ctrl);
-  cudaFree(t->gstash);
-  cudaFree(t->split_ids);
+  cudaFree(t->stash);
   cudaFree(t->neigh_q);
   cudaFree(t->stage);
   cudaFree(t->scratch_u64);
@@ -393,7 +398,9 @@ int pps_create(pps_table** out, const pps_params* p) {
   if (e == cudaSuccess) e = alloc(reinterpret_cast<void**>(&t->dev.ctrl), sizeof(pps::Ctrl));
   if (e == cudaSuccess) e = alloc(reinterpret_cast<void**>(&t->scratch_u64), 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
-  if (e == cudaSuccess && ensure_dense(t, std::min<size_t>(T, 1u << 22), 0, nullptr) != PPS_OK)
+  // the cells of a frame of min(T, 2^22) vertices on the split path
+  const size_t tiles0 = std::min<size_t>(T, 1u << 22) / pps::tile_size() + 1;
+  if (e == cudaSuccess && ensure_dense(t, tiles0 * pps::split_tile_ids(), 0, nullptr) != PPS_OK)
     e = cudaErrorMemoryAllocation;
   if (e != cudaSuccess) {
     free_all(t);
@@ -452,7 +459,7 @@ int pps_build(pps_table* t, const pps_camera* cam, uint32_t frame, void* stream)
   if (int rc = check_table(t)) return rc;
   if (!cam) return fail(PPS_EINVAL, "camera is NULL");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (int rc = reset_frame(t, st)) return rc;
+  if (int rc = reset_frame(t, false, st)) return rc;
   set_camera(t, cam, frame);
   t->state = kOpen;
   if (t->coarse) return pps_build(t->coarse, cam, frame, stream);
@@ -468,9 +475,10 @@ int pps_insert(pps_table* t, const pps_vertices* v, size_t n, uint32_t* slot_out
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t tile = static_cast<size_t>(pps::tile_size());
   const size_t tiles = (n + tile - 1) / tile;
-  if (int rc = ensure_dense(t, (t->frame_tiles + tiles) * tile, t->frame_tiles * tile, st)) return rc;
-  PPS_CUDA(pps::launch_insert(t->kc, t->dev, to_dev(v), n, slot_out, t->frame_tiles,
-                              batch_of(t), st));
+  const size_t ids = static_cast<size_t>(pps::split_tile_ids());
+  if (int rc = ensure_dense(t, (t->frame_tiles + tiles) * ids, t->frame_tiles * ids, st)) return rc;
+  PPS_CUDA(pps::launch_insert(t->kc, t->dev, to_dev(v), n, t->stash, slot_out, t->frame_tiles,
+                              batch_of(t), merge_of(t), st));
   t->frame_tiles += static_cast<uint32_t>(tiles);
   if (t->coarse) return pps_insert(t->coarse, v, n, nullptr, stream);
   return PPS_OK;
@@ -496,7 +504,7 @@ int pps_query(pps_table* t, const pps_vertices* v, size_t n, const uint32_t* slo
   if (int rc = check_output(out, n)) return rc;
   if (t->state == kClean) return fail(PPS_ESTATE, "pps_query needs an open frame");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const uint32_t id_limit = t->frame_tiles * static_cast<uint32_t>(pps::tile_size());
+  const uint32_t id_limit = t->frame_tiles * static_cast<uint32_t>(pps::split_tile_ids());
   if (!t->coarse) {
     PPS_CUDA(pps::launch_query(t->kc, t->dev, to_dev(v), n, slot_in, to_dev(out),
                                t->state == kBlended, id_limit, st));
@@ -512,7 +520,7 @@ int pps_query(pps_table* t, const pps_vertices* v, size_t n, const uint32_t* slo
                              id_limit, st));
   const pps_table* k = t->coarse;
   PPS_CUDA(pps::launch_query(k->kc, k->dev, to_dev(v), n, nullptr, c, k->state == kBlended,
-                             k->frame_tiles * static_cast<uint32_t>(pps::tile_size()), st));
+                             k->frame_tiles * static_cast<uint32_t>(pps::split_tile_ids()), st));
   PPS_CUDA(pps::launch_combine_coarse(n, f.status, c, o, st));
   return PPS_OK;
 }
@@ -524,27 +532,19 @@ namespace {
 // One resolution of pps_filter: the persistent launch over all n vertices.
 int filter_one(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_vertices* v,
                size_t n, int blend, float alpha, const pps::OutPtrs& out, cudaStream_t st) {
-  if (int rc = reset_frame(t, st)) return rc;
+  pps::FusedPlan plan;
+  plan.batch = batch_of(t);
+  plan.merge = merge_of(t);
+  plan.temporal = temporal(t);
+  plan.evict = t->dev.hist_evict != 0;
+  plan.neigh = t->dev.neighbors != 0;
+  plan.kv = v->dist || v->extra;
+  plan.sweep = n && pps::sweep_pays_host(t->dev, n);
+  if (int rc = reset_frame(t, plan.sweep, st)) return rc;
   set_camera(t, cam, frame);
   if (n == 0) return PPS_OK;
-  pps::FusedPlan plan;
-  PPS_CUDA(pps::plan_fused(n, temporal(t), batch_of(t), &plan, t->dev.hist_evict != 0,
-                           t->dev.neighbors != 0, insert_shape(t), t->dev.fixed != 0));
-  // cell ids and (off-chip) stash words cover whole tiles: [0, ntiles * tile)
-  const size_t ftile = static_cast<size_t>(pps::fused_tile_size());
-  const size_t stash_need = (n + ftile - 1) / ftile * ftile;
-  if (int rc = ensure_dense(t, stash_need, 0, st)) return rc;
-  if (plan.global_stash && t->gstash_cap < stash_need) {
-    cudaFree(t->gstash);
-    t->gstash = nullptr;
-    t->gstash_cap = 0;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&t->gstash), stash_need * sizeof(uint32_t));
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return fail(PPS_ENOMEM, "pps_filter: scratch stash allocation failed");
-    }
-    t->gstash_cap = stash_need;
-  }
+  PPS_CUDA(pps::plan_fused(n, ~size_t{0}, &plan));
+  if (int rc = ensure_dense(t, pps::fused_cells(n, plan.tile, plan.batch), 0, st)) return rc;
   if (t->dev.neighbors && t->neigh_q_cap < n) {
     cudaFree(t->neigh_q);
     t->neigh_q = nullptr;
@@ -557,9 +557,9 @@ int filter_one(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_ve
   }
   if (blend)
     if (int rc = next_epoch(t, st)) return rc;
-  PPS_CUDA(pps::launch_fused(t->kc, t->dev, to_dev(v), n, out, temporal(t), blend != 0, alpha,
-                             plan, t->gstash, t->neigh_q, st));
-  t->state = kClean;
+  PPS_CUDA(pps::launch_fused(t->kc, t->dev, to_dev(v), n, out, blend != 0, alpha, plan, t->stash,
+                             t->neigh_q, st));
+  t->stale = plan.sweep;
   return PPS_OK;
 }
 
@@ -577,25 +577,16 @@ int pps_filter(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_ve
   if (blend && (!std::isfinite(alpha) || alpha > 1.0f))
     return fail(PPS_EINVAL, "alpha must be finite and <= 1");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (v->dist || v->extra || t->dev.hist_migrate || t->dev.normal_search) {
-    // key variants and history migration: the split kernels (the persistent
-    // ones are built without them); the insert's cell ids spare the lookup
-    // its keys and probes
-    if (t->split_ids_cap < n) {
-      cudaFree(t->split_ids);
-      t->split_ids = nullptr;
-      t->split_ids_cap = 0;
-      if (cudaMalloc(reinterpret_cast<void**>(&t->split_ids), n * sizeof(uint32_t)) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(PPS_ENOMEM, "pps_filter: cell-id scratch allocation failed");
-      }
-      t->split_ids_cap = n;
-    }
+  if (t->dev.hist_migrate || t->dev.normal_search) {
+    // history migration, similar normals: the split kernels; the insert's cell
+    // ids (the stash, in place) spare the lookup its keys and probes
+    const size_t tiles = (n + pps::tile_size() - 1) / pps::tile_size();
+    if (int rc = ensure_dense(t, tiles * pps::split_tile_ids(), 0, st)) return rc;
     if (int rc = pps_build(t, cam, frame, stream)) return rc;
-    if (int rc = pps_insert(t, v, n, t->split_ids, stream)) return rc;
+    if (int rc = pps_insert(t, v, n, t->stash, stream)) return rc;
     if (blend)
       if (int rc = pps_blend(t, alpha, stream)) return rc;
-    return pps_query(t, v, n, t->split_ids, out, stream);
+    return pps_query(t, v, n, t->stash, out, stream);
   }
   if (!t->coarse) return filter_one(t, cam, frame, v, n, blend, alpha, to_dev(out), st);
   // multi-level: both resolutions, then the choice per vertex
@@ -777,8 +768,10 @@ int table_for_batch(pps_table* t, size_t n, ViewDesc* vd, int* batch, int* block
       t->p.normal_search)
     return fail(PPS_EINVAL, "batched views take tables without a low-count fallback, eviction, "
                             "migration or normal search");
-  const size_t ftile = static_cast<size_t>(fused_tile_size());
-  if (int rc = ensure_dense(t, (n + ftile - 1) / ftile * ftile, 0, st)) return rc;
+  // the batch's tile width and batch are not known yet: room for the widest id ranges
+  if (int rc = ensure_dense(t, fused_cells(n, 64u, 4), 0, st)) return rc;
+  if (int rc = empty_slots(t, st)) return rc;
+  t->stale = true;  // until something else needs the slots, the batch's launches do as they like
   vd->kc = t->kc;
   vd->t = t->dev;
   *batch = batch_of(t);
@@ -813,10 +806,11 @@ int pps_get_tuning(pps_table* t, pps_tuning* tune) {
   if (!tune) return fail(PPS_EINVAL, "tuning is NULL");
   *tune = t->tune;
   tune->batch = static_cast<uint32_t>(batch_of(t));
-  tune->insert = insert_shape(t).pipelined ? 2u : 1u;
+  // one insert serves every table; the fields read as they always did
+  tune->insert = t->tune.insert ? t->tune.insert : t->T > (1u << 23) ? 1u : 2u;
   tune->key_warps = t->tune.key_warps ? t->tune.key_warps : 8u;
   tune->block = t->tune.block ? t->tune.block : 512u;
-  tune->merge = static_cast<uint32_t>(insert_shape(t).merge);
+  tune->merge = static_cast<uint32_t>(merge_of(t));
   return PPS_OK;
 }
 
@@ -834,7 +828,8 @@ int pps_stats(pps_table* t, pps_stats_t* out, void* stream) {
   if (!out) return fail(PPS_EINVAL, "out is NULL");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   PPS_CUDA(cudaMemsetAsync(t->scratch_u64, 0, 2 * sizeof(unsigned long long), st));
-  PPS_CUDA(pps::launch_count_nonzero(t->dev.slots, 8, 0, 8, t->T, t->scratch_u64, st));
+  if (t->state != kClean)  // between frames the table is empty
+    PPS_CUDA(pps::launch_count_nonzero(t->dev.slots, 8, 0, 8, t->T, t->scratch_u64, st));
   if (t->dev.hcells)
     PPS_CUDA(pps::launch_count_nonzero(t->dev.hcells, t->dev.hstride, t->dev.hfp_off, 4, t->Th,
                                        t->scratch_u64 + 1, st));
@@ -866,6 +861,12 @@ int pps_table_dump(pps_table* t, uint32_t* fp_host, void* acc_host, void* stream
   if (!fp_host) return fail(PPS_EINVAL, "fp_host is NULL");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t acc_b = t->dev.fixed ? 32 : 16;
+  if (t->state == kClean) {  // between frames the table is empty
+    PPS_CUDA(cudaStreamSynchronize(st));
+    std::memset(fp_host, 0, t->T * sizeof(uint32_t));
+    if (acc_host) std::memset(acc_host, 0, t->T * acc_b);
+    return PPS_OK;
+  }
   unsigned long long* slots =
       static_cast<unsigned long long*>(std::malloc(t->T * sizeof(unsigned long long)));
   unsigned char* acc = static_cast<unsigned char*>(std::malloc(t->D * acc_b));

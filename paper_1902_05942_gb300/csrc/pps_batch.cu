@@ -58,7 +58,7 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
   cudaGetDevice(&b->device);
   b->alpha = alpha;
   int batch = 2, block = 512;
-  const size_t ftile = static_cast<size_t>(pps::fused_tile_size());
+  size_t total = 0;
   for (uint32_t i = 0; i < nviews; ++i) {
     const pps_view& v = views[i];
     if (!v.table || !v.out.r || !v.out.g || !v.out.b || (v.n && (!v.v.px || !v.v.py || !v.v.pz ||
@@ -85,14 +85,10 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
                            v.v.id, v.v.id_base, v.v.stream_id, v.v.dist, v.v.extra};
     vd.o = pps::OutPtrs{v.out.r, v.out.g, v.out.b, v.out.count, v.out.status};
     vd.n = v.n;
-    vd.tile_base = b->total_tiles;
-    vd.ntiles = static_cast<uint32_t>((v.n + ftile - 1) / ftile);
-    vd.vec = pps::vec_inputs_host(vd.v) ? 1 : 0;
-    vd.ovec = pps::vec_outputs_host(vd.o) ? 1 : 0;
+    total += v.n;
     vd.blended = blend && tmp ? 1 : 0;
     vd.sweep = pps::sweep_pays_host(vd.t, v.n) ? 1 : 0;
     b->temporal = b->temporal || tmp;
-    b->total_tiles += vd.ntiles;
     b->base.push_back(vd);
     b->tables.push_back(v.table);
   }
@@ -100,7 +96,13 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
     delete b;
     return bfail(PPS_EINVAL, "alpha must be finite and <= 1");
   }
-  cudaError_t e = pps::plan_multi(b->total_tiles, b->temporal, batch, block, &b->plan);
+  const uint32_t tile = pps::fused_tile(total, batch);
+  for (pps::ViewDesc& vd : b->base) {
+    vd.tile_base = b->total_tiles;
+    vd.ntiles = static_cast<uint32_t>((vd.n + tile - 1) / tile);
+    b->total_tiles += vd.ntiles;
+  }
+  cudaError_t e = pps::plan_multi(b->total_tiles, tile, b->temporal, batch, block, &b->plan);
   const size_t bytes = nviews * sizeof(pps::ViewDesc);
   for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
     e = cudaMalloc(&b->dviews[k], bytes);
@@ -110,8 +112,8 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
   }
   if (e == cudaSuccess) e = cudaMalloc(&b->ctrl, sizeof(pps::Ctrl));
   if (e == cudaSuccess) e = cudaMemset(b->ctrl, 0, sizeof(pps::Ctrl));
-  if (e == cudaSuccess && b->plan.global_stash)
-    e = cudaMalloc(&b->gstash, static_cast<size_t>(b->total_tiles) * ftile * sizeof(uint32_t));
+  if (e == cudaSuccess && b->total_tiles)
+    e = cudaMalloc(&b->gstash, static_cast<size_t>(b->total_tiles) * tile * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   // capture: descriptor upload, counter resets, the persistent kernel
   cudaStream_t cs = nullptr;

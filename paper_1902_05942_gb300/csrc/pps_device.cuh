@@ -21,7 +21,6 @@ namespace pps {
 
 constexpr uint32_t kOverflowSlot = 0xFFFFFFFFu;  // slot_out value on probe overflow
 constexpr uint32_t kOwnerBit = 0x80000000u;      // stash word: this vertex owns its cell
-constexpr uint32_t kStashOverflow = 0x7FFFFFFFu; // stash word: probe overflow
 
 // ---------------------------------------------------------------- parameters
 struct KeyConst {
@@ -57,15 +56,13 @@ struct Ctrl {
   unsigned long long overflow_vertices;
   unsigned long long vertices;
   unsigned long long hist_overflow;
-  unsigned long long tile_next;   // persistent kernel: next vertex tile to hand out
-  unsigned long long blend_next;  // persistent kernel: next tile whose cells to blend
   unsigned long long neigh_count;  // persistent kernel: low-count vertices queued for the search
   unsigned int error;
   unsigned int bar_count;
   unsigned int bar_gen;
   unsigned int pad[1];
 };
-constexpr size_t kCtrlFrameBytes = 7 * sizeof(unsigned long long);  // reset per frame
+constexpr size_t kCtrlFrameBytes = 5 * sizeof(unsigned long long);  // reset per frame
 
 enum : unsigned int {
   kErrBarrierTimeout = 1u,
@@ -151,8 +148,10 @@ __device__ __forceinline__ uint2 philox_first2_rk(uint32_t c0, uint32_t c1, cons
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
     const uint32_t k0 = r ? kc.rk0[r - 1] : kc.seed, k1 = r ? kc.rk1[r - 1] : kc.frame;
-    const uint32_t lo0 = 0xD2511F53u * x0, hi0 = __umulhi(0xD2511F53u, x0);
-    const uint32_t lo1 = 0xCD9E8D57u * x2, hi1 = __umulhi(0xCD9E8D57u, x2);
+    // 32 x 32 -> 64-bit products, one instruction each
+    const unsigned long long p0 = 0xD2511F53ull * x0, p1 = 0xCD9E8D57ull * x2;
+    const uint32_t lo0 = static_cast<uint32_t>(p0), hi0 = static_cast<uint32_t>(p0 >> 32);
+    const uint32_t lo1 = static_cast<uint32_t>(p1), hi1 = static_cast<uint32_t>(p1 >> 32);
     const uint32_t n0 = hi1 ^ x1 ^ k0, n2 = hi0 ^ x3 ^ k1;
     x0 = n0;
     x1 = lo1;
@@ -187,36 +186,62 @@ __device__ __forceinline__ float pow2_int(int l) {
   return __uint_as_float(static_cast<uint32_t>(l + 127) << 23);
 }
 
-// |p_cam - x| in FP32, one rounding per operation.
-__device__ __forceinline__ float camera_distance(const KeyConst& kc, float x, float y, float z) {
+// |p_cam - x|^2 in FP32, one rounding per operation.
+__device__ __forceinline__ float camera_distance2(const KeyConst& kc, float x, float y, float z) {
   const float dx = __fsub_rn(kc.cam[0], x);
   const float dy = __fsub_rn(kc.cam[1], y);
   const float dz = __fsub_rn(kc.cam[2], z);
-  return __fsqrt_rn(__fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz)));
+  return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
 }
 
-// floor(log2(k * d)) from the exponent bits of the FP32 product.
-__device__ __forceinline__ int level_at(const KeyConst& kc, float d) {
-  const float F = __fmul_rn(kc.k, d);
+// |p_cam - x| in FP32, one rounding per operation.
+__device__ __forceinline__ float camera_distance(const KeyConst& kc, float x, float y, float z) {
+  return __fsqrt_rn(camera_distance2(kc, x, y, z));
+}
+
+// floor(log2 F) of an FP32 product F = k * d, from its exponent bits.
+__device__ __forceinline__ int level_of(const KeyConst& kc, float F) {
   const int e = static_cast<int>((__float_as_uint(F) >> 23) & 0xFFu) - 127;
   return min(max(e, kc.lod_min), kc.lod_max);
 }
 
+// floor(log2(k * d)) from the exponent bits of the FP32 product.
+__device__ __forceinline__ int level_at(const KeyConst& kc, float d) { return level_of(kc, __fmul_rn(kc.k, d)); }
+
 // Algorithm 1's level_of_detail(|p_cam - x|).
+//
+// Only the exponent of F = fl(k * fl(sqrt(d2))) counts.  sqrt.approx is within
+// 2^-23 of the square root relatively, and sqrt.rn and the products round by
+// 2^-24 each, so the product with the approximate root is within 4 units of
+// the last place of F, and both have the same exponent unless the approximate
+// one lies within 8 units of a power of two (0 and infinity among them; a
+// subnormal d2 reads as 0): there, about once in half a million vertices, the
+// correctly rounded root decides.  It costs some ten instructions and a branch
+// each of the two times a key needs a level (keys alone, 4.2 M vertices: 309
+// instructions a vertex and 51.6 us with it, 286 and 49.1 us without it and
+// with the fused forms below).
 __device__ __forceinline__ int level_of_detail(const KeyConst& kc, float x, float y, float z) {
-  return level_at(kc, camera_distance(kc, x, y, z));
+  const float d2 = camera_distance2(kc, x, y, z);
+  float d;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(d) : "f"(d2));
+  float F = __fmul_rn(kc.k, d);
+  if (((__float_as_uint(F) + 8u) & 0x7FFFFFu) < 16u) F = __fmul_rn(kc.k, __fsqrt_rn(d2));
+  return level_of(kc, F);
 }
 
+// floor(v), v's product with a power of two, as int32: clamped to
+// [-2^31, 2147483520] (the conversion rounds down).
 __device__ __forceinline__ int32_t quantize_coord(float v, float inv) {
-  float q = floorf(__fmul_rn(v, inv));
-  q = fminf(fmaxf(q, -2147483648.0f), 2147483520.0f);
-  return __float2int_rz(q);
+  const float q = __fmul_rn(v, inv);
+  return __float2int_rd(fminf(fmaxf(q, -2147483648.0f), 2147483520.0f));
 }
 
+// clamp(floor((c + 1) * 128), 0, 255).  Scaling by 128 is exact, so the fused
+// form rounds once, like c + 1; the conversion to 8 bits truncates and clamps.
 __device__ __forceinline__ uint32_t quantize_normal(float c) {
-  float q = floorf(__fmul_rn(__fadd_rn(c, 1.0f), 128.0f));
-  q = fminf(fmaxf(q, 0.0f), 255.0f);
-  return static_cast<uint32_t>(q);
+  uint32_t q;
+  asm("{\n .reg .u8 t;\n cvt.rzi.u8.f32 t, %1;\n cvt.u32.u8 %0, t;\n}" : "=r"(q) : "f"(__fmaf_rn(c, 128.0f, 128.0f)));
+  return q;
 }
 
 struct Key {
@@ -258,22 +283,24 @@ __device__ __forceinline__ KeyWords key_words(const KeyConst& kc, float px, floa
   if (kc.jitter) {
     // jitter(n): a point of the tangent plane, (u, w) uniform in [-0.5, 0.5)
     const uint2 rnd = philox_first2_rk(id, stream_id, kc);
-    const float u = __fsub_rn(__fmul_rn(__uint2float_rn(rnd.x >> 8), 0x1p-24f), 0.5f);
-    const float w = __fsub_rn(__fmul_rn(__uint2float_rn(rnd.y >> 8), 0x1p-24f), 0.5f);
+    // (products with powers of two, and with s = +-1, are exact: the fused
+    // forms below round once, like the separate operations)
+    const float u = __fmaf_rn(__uint2float_rn(rnd.x >> 8), 0x1p-24f, -0.5f);
+    const float w = __fmaf_rn(__uint2float_rn(rnd.y >> 8), 0x1p-24f, -0.5f);
     // tangent frame after Duff et al. (JCGT 2017)
     const float s = copysignf(1.0f, nz);
     const float a = -__frcp_rn(__fadd_rn(s, nz));  // = -1 / (s + nz), correctly rounded
     const float q = __fmul_rn(__fmul_rn(nx, ny), a);
-    const float tx = __fadd_rn(1.0f, __fmul_rn(s, __fmul_rn(__fmul_rn(nx, nx), a)));
+    const float tx = __fmaf_rn(s, __fmul_rn(__fmul_rn(nx, nx), a), 1.0f);
     const float ty = __fmul_rn(s, q);
     const float tz = -__fmul_rn(s, nx);
     const float bx = q;
     const float by = __fadd_rn(s, __fmul_rn(__fmul_rn(ny, ny), a));
     const float bz = -ny;
     const float E = pow2_int(l0);  // voxel edge at the pre-jitter level
-    xj = __fadd_rn(px, __fmul_rn(__fadd_rn(__fmul_rn(u, tx), __fmul_rn(w, bx)), E));
-    yj = __fadd_rn(py, __fmul_rn(__fadd_rn(__fmul_rn(u, ty), __fmul_rn(w, by)), E));
-    zj = __fadd_rn(pz, __fmul_rn(__fadd_rn(__fmul_rn(u, tz), __fmul_rn(w, bz)), E));
+    xj = __fmaf_rn(__fadd_rn(__fmul_rn(u, tx), __fmul_rn(w, bx)), E, px);
+    yj = __fmaf_rn(__fadd_rn(__fmul_rn(u, ty), __fmul_rn(w, by)), E, py);
+    zj = __fmaf_rn(__fadd_rn(__fmul_rn(u, tz), __fmul_rn(w, bz)), E, pz);
     l1 = ke.dist ? level_at(kc, __fadd_rn(__fsub_rn(__ldg(ke.dist + ke.j),
                                                     camera_distance(kc, px, py, pz)),
                                           camera_distance(kc, xj, yj, zj)))
@@ -386,6 +413,16 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64_keep(const unsigned
   unsigned long long v;
   asm volatile("ld.relaxed.gpu.global.L2::cache_hint.u64 %0, [%1], %2;"
                : "=l"(v)
+               : "l"(p), "l"(l2_evict_last())
+               : "memory");
+  return v;
+}
+
+// Two neighbouring slots (p 16-byte aligned), each a relaxed read of its own.
+__device__ __forceinline__ ulonglong2 ld_relaxed_u64x2_keep(const unsigned long long* p) {
+  ulonglong2 v;
+  asm volatile("ld.relaxed.gpu.global.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;"
+               : "=l"(v.x), "=l"(v.y)
                : "l"(p), "l"(l2_evict_last())
                : "memory");
   return v;
@@ -552,9 +589,10 @@ static __device__ __noinline__ uint32_t hist_claim_evict(const TableDev& t, uint
 }
 
 // Accumulate a group of `cnt` contributions (sums r, g, b) into cell `id`.
+template <bool FIXED>
 __device__ __forceinline__ void accumulate(const TableDev& t, uint32_t id, float r, float g, float b,
                                            long long fr, long long fg, long long fb, uint32_t cnt) {
-  if (!t.fixed) {
+  if (!FIXED) {
     red_add_v4_keep(t.acc + id, r, g, b, static_cast<float>(cnt));
     return;
   }
@@ -642,45 +680,88 @@ __device__ __forceinline__ HistRaw load_hist(const TableDev& t, uint32_t h) {
   return o;
 }
 
+// Write history entry h (fingerprint word fw): the whole 32-byte cell in FP32,
+// so that the sector needs no read-back when it leaves L2 (random 16-byte
+// stores run at 23 G/s on a table in DRAM, 32-byte ones at 42 G/s).
+__device__ __forceinline__ void store_hist(const TableDev& t, uint32_t h, uint32_t fw, float cr,
+                                           float cg, float cb, uint32_t N) {
+  unsigned char* c = t.hcells + static_cast<size_t>(h) * 32;
+  asm volatile("st.global.L2::cache_hint.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %6, %6}, %7;" ::"l"(c),
+               "r"(__float_as_uint(cr)), "r"(__float_as_uint(cg)), "r"(__float_as_uint(cb)), "r"(N),
+               "r"(fw), "r"(0u), "l"(l2_evict_first())
+               : "memory");
+}
+
 // Temporal filtering / integration of one cell (Sec. 3.4.1):
 // c = alpha c_old + (1 - alpha) c_new, alpha < 0 meaning alpha = N_old / (N_old +
-// N_new); no history -> c = c_new.  The history cell h is updated (h ==
-// kOverflowSlot: the history window was full; the cell keeps c_new and
-// N = N_new) and the result replaces the cell's accumulator for the lookups.
-__device__ __forceinline__ void blend_store(const TableDev& t, uint32_t id, uint32_t h,
-                                            const CellMean& m, const HistRaw& old, float alpha) {
-  float cr = m.r, cg = m.g, cb = m.b;
-  uint32_t N = m.n;
-  if (h != kOverflowSlot) {
-    if (old.n != 0u) {
-      const float a =
-          alpha >= 0.0f ? alpha
-                        : __fdiv_rn(__uint2float_rn(old.n),
-                                    __fadd_rn(__uint2float_rn(old.n), __uint2float_rn(m.n)));
-      const float a1 = __fsub_rn(1.0f, a);
-      cr = __fadd_rn(__fmul_rn(a, old.r), __fmul_rn(a1, cr));
-      cg = __fadd_rn(__fmul_rn(a, old.g), __fmul_rn(a1, cg));
-      cb = __fadd_rn(__fmul_rn(a, old.b), __fmul_rn(a1, cb));
-    }
-    unsigned char* c = t.hcells + static_cast<size_t>(h) * t.hstride;
-    if (t.hist_mode == 1) {
-      N = old.n + m.n;
-      st_once_u4(c, make_uint4(__float_as_uint(cr), __float_as_uint(cg), __float_as_uint(cb), N));
-    } else {
-      N = min(old.n + m.n, 65535u);
-      const __half2 rg = __floats2half2_rn(cr, cg);
-      const __half hb = __float2half_rn(cb);
-      const uint32_t lo = *reinterpret_cast<const uint32_t*>(&rg);
-      const uint32_t hi = static_cast<uint32_t>(__half_as_ushort(hb)) | (N << 16);
-      st_once_u2(c, make_uint2(lo, hi));
-      // lookups see what the history stores
-      const float2 back = __half22float2(rg);
-      cr = back.x;
-      cg = back.y;
-      cb = __half2float(hb);
-    }
+// N_new); no history -> c = c_new.  The history cell h (fingerprint word fw)
+// is updated (h == kOverflowSlot: the history window was full; the cell keeps
+// c_new and N = N_new) and the result replaces m.
+__device__ __forceinline__ void blend_value(const TableDev& t, uint32_t h, uint32_t fw, CellMean& m,
+                                            const HistRaw& old, float alpha) {
+  if (h == kOverflowSlot) return;
+  if (old.n != 0u) {
+    const float a =
+        alpha >= 0.0f ? alpha
+                      : __fdiv_rn(__uint2float_rn(old.n),
+                                  __fadd_rn(__uint2float_rn(old.n), __uint2float_rn(m.n)));
+    const float a1 = __fsub_rn(1.0f, a);
+    m.r = __fadd_rn(__fmul_rn(a, old.r), __fmul_rn(a1, m.r));
+    m.g = __fadd_rn(__fmul_rn(a, old.g), __fmul_rn(a1, m.g));
+    m.b = __fadd_rn(__fmul_rn(a, old.b), __fmul_rn(a1, m.b));
   }
-  __stcg(value_ptr(t, id), make_float4(cr, cg, cb, __uint_as_float(N)));
+  if (t.hist_mode == 1) {
+    m.n += old.n;
+    store_hist(t, h, fw, m.r, m.g, m.b, m.n);
+  } else {
+    m.n = min(old.n + m.n, 65535u);
+    const __half2 rg = __floats2half2_rn(m.r, m.g);
+    const __half hb = __float2half_rn(m.b);
+    const uint32_t lo = *reinterpret_cast<const uint32_t*>(&rg);
+    const uint32_t hi = static_cast<uint32_t>(__half_as_ushort(hb)) | (m.n << 16);
+    st_once_u2(t.hcells + static_cast<size_t>(h) * t.hstride, make_uint2(lo, hi));
+    // lookups see what the history stores
+    const float2 back = __half22float2(rg);
+    m.r = back.x;
+    m.g = back.y;
+    m.b = __half2float(hb);
+  }
+}
+
+// The same for a cell of the frame table: the result replaces the cell's
+// accumulator for the lookups.
+__device__ __forceinline__ void blend_store(const TableDev& t, uint32_t id, uint32_t h, uint32_t fw,
+                                            CellMean m, const HistRaw& old, float alpha) {
+  blend_value(t, h, fw, m, old, alpha);
+  __stcg(value_ptr(t, id), make_float4(m.r, m.g, m.b, __uint_as_float(m.n)));
+}
+
+// A history cell in one load: its value and its fingerprint word.
+__device__ __forceinline__ HistRaw load_hist_fp(const TableDev& t, uint32_t h, uint32_t* fw) {
+  HistRaw o;
+  const unsigned char* c = t.hcells + static_cast<size_t>(h) * t.hstride;
+  if (t.hist_mode == 1) {
+    uint32_t x, y, z, w, u0, u1, u2, u3;
+    asm volatile("ld.relaxed.gpu.global.L2::cache_hint.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
+                 : "=r"(x), "=r"(y), "=r"(z), "=r"(w), "=r"(u0), "=r"(u1), "=r"(u2), "=r"(u3)
+                 : "l"(c), "l"(l2_evict_first())
+                 : "memory");
+    (void)u1, (void)u2, (void)u3;  // padding
+    o.r = __uint_as_float(x);
+    o.g = __uint_as_float(y);
+    o.b = __uint_as_float(z);
+    o.n = w;
+    *fw = u0;
+  } else {
+    const uint4 v = ld_once_u4(c);
+    const float2 rg = __half22float2(*reinterpret_cast<const __half2*>(&v.x));
+    o.r = rg.x;
+    o.g = rg.y;
+    o.b = __half2float(__ushort_as_half(static_cast<unsigned short>(v.y & 0xFFFFu)));
+    o.n = v.y >> 16;
+    *fw = v.z;
+  }
+  return o;
 }
 
 // Value returned for cell `id`: the cell average, or the blended value.
@@ -702,13 +783,58 @@ __device__ __forceinline__ AccRaw load_value(const TableDev& t, uint32_t id, boo
   return a;
 }
 
-// Empty cell `id` (its accumulator and its slot) for the next frame.
-__device__ __forceinline__ void clear_cell(const TableDev& t, uint32_t id, uint32_t slot) {
-  float4* p = value_ptr(t, id);
-  st_zero16_keep(p);
-  if (t.fixed) st_zero16_keep(p + 1);
-  if (slot != kNoSlot) __stcg(t.slots + slot, 0ull);
+// ---------------------------------------------------------------- vertices in, results out
+struct Result {
+  float r, g, b;
+  uint32_t n;
+  uint8_t status;
+};
+
+template <int W>
+__device__ __forceinline__ void store_batch(const OutPtrs& o, size_t j, size_t end, bool vec,
+                                            const Result (&res)[W]) {
+  if (vec && j + W <= end) {
+    if constexpr (W == 4) {
+      __stcs(reinterpret_cast<float4*>(o.r + j), make_float4(res[0].r, res[1].r, res[2].r, res[3].r));
+      __stcs(reinterpret_cast<float4*>(o.g + j), make_float4(res[0].g, res[1].g, res[2].g, res[3].g));
+      __stcs(reinterpret_cast<float4*>(o.b + j), make_float4(res[0].b, res[1].b, res[2].b, res[3].b));
+      if (o.count)
+        __stcs(reinterpret_cast<uint4*>(o.count + j),
+               make_uint4(res[0].n, res[1].n, res[2].n, res[3].n));
+      if (o.status) {
+        const uint32_t w = res[0].status | (res[1].status << 8) | (res[2].status << 16) |
+                           (static_cast<uint32_t>(res[3].status) << 24);
+        __stcs(reinterpret_cast<unsigned int*>(o.status + j), w);
+      }
+    } else {
+      __stcs(reinterpret_cast<float2*>(o.r + j), make_float2(res[0].r, res[1].r));
+      __stcs(reinterpret_cast<float2*>(o.g + j), make_float2(res[0].g, res[1].g));
+      __stcs(reinterpret_cast<float2*>(o.b + j), make_float2(res[0].b, res[1].b));
+      if (o.count) __stcs(reinterpret_cast<uint2*>(o.count + j), make_uint2(res[0].n, res[1].n));
+      if (o.status) {
+        const unsigned short w = static_cast<unsigned short>(res[0].status | (res[1].status << 8));
+        __stcs(reinterpret_cast<unsigned short*>(o.status + j), w);
+      }
+    }
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < W; ++q) {
+    if (j + q < end) {
+      o.r[j + q] = res[q].r;
+      o.g[j + q] = res[q].g;
+      o.b[j + q] = res[q].b;
+      if (o.count) o.count[j + q] = res[q].n;
+      if (o.status) o.status[j + q] = res[q].status;
+    }
+  }
 }
+
+// This warp's place among the grid's warps.
+__device__ __forceinline__ uint32_t grid_warp() {
+  return blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+}
+__device__ __forceinline__ uint32_t grid_warps() { return gridDim.x * (blockDim.x >> 5); }
 
 // ---------------------------------------------------------------- grid barrier
 __device__ __forceinline__ unsigned long long globaltimer_ns() {

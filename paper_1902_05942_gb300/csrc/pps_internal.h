@@ -14,23 +14,16 @@ namespace pps {
 
 // Launch geometry of the persistent filter kernel for one call.
 struct FusedPlan {
-  int grid = 0;            // CTAs (a multiple of the SM count: SMs x CTAs per SM)
-  int block = 0;           // threads per CTA
-  int batch = 4;           // vertices per thread per insert step (2 or 4)
-  uint32_t cap_tiles = 0;  // tiles one CTA may take (stash capacity)
-  size_t smem = 0;         // dynamic shared memory per CTA (stash of cap_tiles tiles)
-  bool global_stash = false;
-  bool evict = false;      // the kernel variant for an evicting history
-  bool neigh = false;      // the kernel variant with the neighborhood search
-  int key_warps = 0;       // > 0: the pipelined insert (k_fused_ws) with this many key warps
-  int merge = 2;           // pipelined insert: warp aggregation of equal keys (pps_tuning.merge)
-};
-
-// How a table's persistent launch inserts (pps_tuning.insert / key_warps).
-struct InsertShape {
-  int pipelined = 1;  // 1: key warps and probe warps on alternate chunks; 0: per thread
-  int key_warps = 8;  // of the 16 warps of a CTA (4, 8 or 12)
-  int merge = 2;      // 1 none, 2 where neighbouring lanes repeat a key, 3 always
+  int grid = 0;       // CTAs
+  int block = 0;      // threads per CTA
+  int batch = 2;      // vertices per lane per insert step (2 or 4)
+  uint32_t tile = 0;  // vertices per warp tile
+  bool temporal = false;  // kernel variants: a table with a history
+  bool evict = false;     // ... an evicting one
+  bool neigh = false;     // ... the neighborhood search
+  bool kv = false;        // ... vertices with key variants
+  bool sweep = false;     // zero the whole slot table first, not the frame's slots at the end
+  int merge = 2;      // merging of equal keys within a warp (pps_tuning.merge)
 };
 
 // One view of a batched launch: its table, key constants, vertices and
@@ -43,32 +36,29 @@ struct ViewDesc {
   unsigned long long n;
   uint32_t tile_base;  // first tile of this view in the batch
   uint32_t ntiles;
-  int vec, ovec;
   int blended;  // blend this view's cells (temporal table and blending requested)
   int sweep;    // zero this view's slot table by a sweep at the end
 };
 
 struct MultiPlan {
   int grid = 0, block = 0, batch = 2;
-  uint32_t cap_tiles = 0;
-  size_t smem = 0;
-  bool global_stash = false;
+  uint32_t tile = 0;  // vertices per warp tile
 };
 
-// Plan / launch the batched persistent kernel over `total_tiles` tiles of the
-// views in device memory (`views`, nviews entries); `ctrl` carries the grid
-// barrier and the tile counter; `gstash` (total_tiles tiles) is used when the
-// stash does not fit on chip.
-cudaError_t plan_multi(size_t total_tiles, bool temporal, int batch, int block, MultiPlan* plan);
+// Plan / launch the batched persistent kernel over `total_tiles` warp tiles of
+// `tile` vertices of the views in device memory (`views`, nviews entries);
+// `ctrl` carries the grid barrier, `stash` (total_tiles
+// tiles) the vertices' cell ids.
+cudaError_t plan_multi(size_t total_tiles, uint32_t tile, bool temporal, int batch, int block,
+                       MultiPlan* plan);
 cudaError_t launch_multi(const ViewDesc* views, uint32_t nviews, uint32_t total_tiles, Ctrl* ctrl,
-                         bool temporal, float alpha, const MultiPlan& plan, uint32_t* gstash,
+                         bool temporal, float alpha, const MultiPlan& plan, uint32_t* stash,
                          cudaStream_t st);
-bool vec_inputs_host(const VertexPtrs& v);
-bool vec_outputs_host(const OutPtrs& o);
 bool sweep_pays_host(const TableDev& t, size_t vertices);
 
 cudaError_t launch_insert(const KeyConst& kc, const TableDev& t, const VertexPtrs& v, size_t n,
-                          uint32_t* id_out, uint32_t tile_base, int batch, cudaStream_t st);
+                          uint32_t* stash, uint32_t* id_out, uint32_t tile_base, int batch, int merge,
+                          cudaStream_t st);
 cudaError_t launch_query(const KeyConst& kc, const TableDev& t, const VertexPtrs& v, size_t n,
                          const uint32_t* id_in, const OutPtrs& o, bool blended, uint32_t id_limit,
                          cudaStream_t st);
@@ -86,14 +76,19 @@ cudaError_t launch_combine_coarse(size_t n, const uint8_t* fine_status, const Ou
                                   const OutPtrs& o, cudaStream_t st);
 cudaError_t launch_count_nonzero(const void* base, uint32_t stride, uint32_t off, uint32_t width,
                                  uint64_t n, unsigned long long* out, cudaStream_t st);
-cudaError_t plan_fused(size_t n, bool temporal, int batch, FusedPlan* plan, bool evict = false,
-                       bool neigh = false, InsertShape shape = InsertShape{}, bool fixed = false);
+// Fill in the geometry of a plan whose kernel variant and batch are set
+// (tiles whose id ranges span at most max_cells cells).
+cudaError_t plan_fused(size_t n, size_t max_cells, FusedPlan* plan);
 cudaError_t launch_fused(const KeyConst& kc, const TableDev& t, const VertexPtrs& v, size_t n,
-                         const OutPtrs& o, bool temporal, bool blend, float alpha,
-                         const FusedPlan& plan, uint32_t* gstash, uint32_t* nq, cudaStream_t st);
+                         const OutPtrs& o, bool blend, float alpha, const FusedPlan& plan, uint32_t* stash, uint32_t* nq, cudaStream_t st);
 
-int tile_size();        // vertices (and cell ids) per tile of the split path
-int fused_tile_size();  // vertices (and cell ids) per tile of the persistent kernel
+int sm_count();   // multiprocessors of the device
+int tile_size();  // vertices per warp tile of the split path
+int split_tile_ids();  // cell ids of such a tile's range
+// ... of the persistent kernels, for a launch over n vertices
+uint32_t fused_tile(size_t n, int batch);
+// Cells that the tiles' id ranges span (tiles of `tile` vertices).
+size_t fused_cells(size_t n, uint32_t tile, int batch);
 bool aligned16(const void* p);
 
 int record_error(int code, const char* msg);  // message for pps_last_error()

@@ -1,34 +1,27 @@
 // Kernels of the hashed path space filter (sm_103a) and their launchers.
 //
-//  k_insert        key construction (Alg. 1) + probing insert + atomic
-//                  accumulation (Sec. 3.2, 3.3.1) for one tile of vertices per
-//                  CTA iteration; a tile's new cells get ids from the tile's
-//                  own id range.
-//  k_blend_sweep   temporal blend of every cell claimed this frame (Sec. 3.4.1).
-//  k_query         one lookup per vertex: cell average or blended value.
-//  k_clear_sweep   empties the frame's cells for the next frame.
-//  k_fused         the whole frame in one persistent cooperative launch: the
-//                  four steps above separated by grid barriers; each vertex's
-//                  cell id stays in shared memory between the phases; the
-//                  blend's tiles come from a second counter, and each CTA
-//                  clears the cells its own tiles created.
-//  k_fused_ws      the same frame with a pipelined insert: key warps build
-//                  and merge keys into a shared-memory queue while probe warps
-//                  run the table operations of the previous chunk (the default
-//                  for frames without eviction or neighborhood search).
-//  k_fused<NEIGH>, k_neighbors, k_clear_fused
-//                  neighborhood-search frames: the persistent kernel queues
-//                  its low-count vertices after the lookups, a separate launch
-//                  searches them, a third empties the cells.
+//  k_fused         the whole frame in one persistent cooperative launch: sweep
+//                  of the slot table, key construction (Alg. 1) and probing
+//                  insert, accumulation (Sec. 3.2, 3.3.1), temporal blend
+//                  (Sec. 3.4.1), one lookup per vertex, separated by grid
+//                  barriers; within a phase every warp works alone.
+//  k_fused<NEIGH>, k_neighbors
+//                  neighborhood-search frames: the persistent kernel lists its
+//                  low-count vertices with the lookups, a separate launch
+//                  searches them.
+//  k_fused_multi   the same phases over the tiles of several views.
+//  k_insert, k_add, k_blend_sweep, k_query, k_clear_sweep
+//                  the same steps as launches of their own (the split path).
 //  k_blend_lookup, k_blend_apply
 //                  the blend of a history that follows changes of resolution.
 //
-// Vertex streams are read with streaming loads (ld.global.cs): in the split
-// kernels four consecutive vertices per thread (128-bit when the arrays are
-// 16-byte aligned), in the persistent kernels W consecutive vertices per
-// thread with each warp's sub-batch one contiguous run; table words are read
-// at L2 (ld.relaxed.gpu / ld.global.cg) because other CTAs write them.
+// Vertex streams are read with streaming loads (ld.global.cs), a warp's 32
+// lanes taking 32 consecutive vertices; table words are read at L2
+// (ld.relaxed.gpu / ld.global.cg) because other CTAs write them.
 #include <algorithm>
+#include <mutex>
+#include <utility>
+#include <vector>
 
 #include "pps_internal.h"
 
@@ -36,33 +29,11 @@ namespace pps {
 
 namespace {
 
-constexpr int kBlock = 256;            // split kernels
-constexpr int kTile = kBlock * 4;      // vertices (and cell ids) per split-path tile
-constexpr int kFusedBlock = 512;       // persistent kernel
-constexpr int kFusedTile = kFusedBlock * 4;  // vertices per persistent-kernel tile
-constexpr int kMaxTilesPerCta = 1024;  // tile list of one persistent CTA
-
-// W consecutive floats of one stream (one 8- or 16-byte load when aligned).
-template <int W>
-__device__ __forceinline__ void loadw(float (&x)[W], const float* p, size_t j, size_t end,
-                                      bool vec) {
-  if (vec && j + W <= end) {
-    if constexpr (W == 4) {
-      const float4 v = __ldcs(reinterpret_cast<const float4*>(p + j));
-      x[0] = v.x;
-      x[1] = v.y;
-      x[2] = v.z;
-      x[3] = v.w;
-    } else {
-      const float2 v = __ldcs(reinterpret_cast<const float2*>(p + j));
-      x[0] = v.x;
-      x[1] = v.y;
-    }
-    return;
-  }
-#pragma unroll
-  for (int q = 0; q < W; ++q) x[q] = j + q < end ? __ldcs(p + j + q) : 0.f;
-}
+constexpr int kBlock = 256;       // split kernels
+constexpr int kTile = 256;        // vertices per warp tile of the split path
+constexpr int kTileIds = kTile + 32 * 5;  // cell ids of its range (tile_ids, widest batch)
+constexpr int kFusedBlock = 512;  // persistent kernels
+constexpr int kFusedTile = 256;   // vertices per warp tile, large frames
 
 __device__ __forceinline__ float4 load4(const float* p, size_t j, size_t end, bool vec) {
   if (vec && j + 4 <= end) return __ldcs(reinterpret_cast<const float4*>(p + j));
@@ -100,213 +71,384 @@ struct Counters {
   uint32_t ovf = 0, cells = 0;  // per thread (summed to 64 bits per CTA)
 };
 
-// The rare continuation of a probe whose home slot held another key, kept out
-// of line so that the four-wide insert stays fully unrolled in registers.
-// `my` is the id reserved for this key (kOverflowSlot: none yet).
-struct MoreProbe {
-  uint32_t slot, id, my;
-  bool claimed;
+// ------------------------------------------------------------------ insert
+// The insert runs in two passes with a barrier between them.
+//
+// Pass one (insert_warp) finds or creates every vertex's cell and writes its id
+// to the stash.  The vertex that creates a cell owns it and STORES its own
+// contribution and a count of one as the cell's accumulator.  Pass two
+// (add_warp) adds the other vertices' contributions.  So an accumulator needs
+// no clearing, a new cell costs a coalesced store where an atomic on a cold
+// line would first fetch it from DRAM (random red.v4: 180 G/s on lines in L2,
+// 23 G/s otherwise), and only the vertices that met an existing cell (about
+// half) need an atomic, on lines written just before.  HD frame (5.06 M
+// vertices, 2^23 slots): insert and accumulation 191 us in one pass with an
+// atomic per vertex, 126 + 28 us in two; fixed point 293 us, 135 + 84 us.
+//
+// A warp inserts alone: no barrier and no shared counter between warps, so a
+// warp with long probe sequences holds up no other.  Every key's home slot
+// is tried with one compare-and-swap (no load before it: a load followed by a
+// compare-and-swap of the same line costs three times the compare-and-swap,
+// 42 against 121 G/s on a 64 MB table).  About one key in seven meets another
+// key there; finishing those on the spot would make the whole warp wait for
+// four or five more memory round trips of a few lanes.  They go into a queue of
+// the warp's own in shared memory instead, and whenever it holds enough of them
+// the warp advances 32 at once, each by one step of its probe sequence.
+//
+// What bounds pass one now is the keys: without any table access it takes
+// 84 us (about 330 instructions per vertex at 8 warps per scheduler, 64
+// registers), the compare-and-swaps add 20 us, the queue 20 us.
+constexpr int kQueue = 64;  // queue entries per warp
+
+// Shared memory of one warp: its queue of keys, and the contributions of a row
+// of 32 vertices while equal cells are merged.
+struct WarpShared {
+  union {
+    struct {
+      uint32_t h1[kQueue], f[kQueue], step[kQueue], members[kQueue], first[kQueue];
+    };
+    uint32_t list[kQueue * 5];  // the lookup's low-count vertices
+  };
+  float row[96];
 };
 
-__device__ __noinline__ MoreProbe probe_more(unsigned long long* slots, uint32_t mask,
-                                             uint32_t max_probes, uint32_t home, uint32_t f,
-                                             uint32_t my, uint32_t id_base, uint32_t* claims) {
-  MoreProbe r{kOverflowSlot, kOverflowSlot, my, false};
-  for (uint32_t p = 1; p < max_probes; ++p) {
-    const uint32_t s = (home + p) & mask;
-    unsigned long long w = ld_relaxed_u64(slots + s);
-    if (w == 0ull) {
-      if (r.my == kOverflowSlot) r.my = id_base + atomicAdd(claims, 1u);
-      w = atomicCAS(slots + s, 0ull, slot_word(f, r.my));
-      if (w == 0ull) {
-        r.slot = s;
-        r.id = r.my;
-        r.claimed = true;
-        return r;
-      }
-    }
-    if (slot_fp(w) == f) {
-      r.slot = s;
-      r.id = slot_id(w);
-      return r;
+constexpr uint32_t kDeferred = 0x7FFFFFFFu;  // cell id not known yet
+
+// The most cell ids that a warp draws from the range of one tile of `v`
+// vertices, W vertices per lane and step: one for each new cell made while it
+// works on the tile (its own vertices and up to 32 queued ones), and those its
+// lanes hold in reserve.
+__host__ __device__ constexpr uint32_t tile_ids(uint32_t v, int batch) { return v + 32u * (batch + 1); }
+
+// What a warp carries from one insert to the next.
+template <int W>
+struct WarpInsert {
+  uint32_t my[W];    // ids reserved for the lane's next new cells (kOverflowSlot: none)
+  uint32_t claims;   // ids handed out of the current tile's range (the same in every lane)
+  uint32_t id_base;  // that range's first id
+  uint32_t queued;   // entries in the queue (the same in every lane)
+  Counters cnt;
+  __device__ __forceinline__ WarpInsert() : claims(0u), id_base(0u), queued(0u) {
+#pragma unroll
+    for (int q = 0; q < W; ++q) my[q] = kOverflowSlot;
+  }
+  // Mark the reserved ids that ended up unused, for the passes over t.info.
+  __device__ __forceinline__ void retire(const TableDev& t, bool rec) {
+#pragma unroll
+    for (int q = 0; q < W; ++q) {
+      if (rec && my[q] != kOverflowSlot)
+        st_once_u4(t.info + my[q], make_uint4(kNoSlot, 0u, 0u, kOverflowSlot));
+      my[q] = kOverflowSlot;
     }
   }
-  return r;
-}
-
-template <int W>
-struct Batch {
-  uint32_t id[W];
+  // An id for every lane with `need` that has none in my[q].
+  __device__ __forceinline__ void reserve(int q, bool need) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, need && my[q] == kOverflowSlot);
+    if (m >> lane & 1u) my[q] = id_base + claims + __popc(m & ((1u << lane) - 1u));
+    claims += __popc(m);
+  }
 };
 
-// Insert the W vertices j..j+W-1 (those below `end`) and return their cell
-// ids (kOverflowSlot on probe overflow).  New cells take ids id_base + k, k
-// drawn from the tile's claim counter *claims (shared memory).
+// A new cell `id`: its creator's contribution is its first, and (`rec`) its
+// record {slot, home hash, fingerprint}.
+__device__ __forceinline__ void create_cell(const TableDev& t, uint32_t id, float r, float g, float b,
+                                            uint32_t slot, uint32_t h1, uint32_t f, bool rec) {
+  if (!t.fixed) {
+    __stcg(t.acc + id, make_float4(r, g, b, 1.0f));
+  } else {
+    ulonglong2* a = reinterpret_cast<ulonglong2*>(t.acc64 + 4 * static_cast<size_t>(id));
+    __stcg(a, make_ulonglong2(static_cast<unsigned long long>(to_fixed(r)),
+                              static_cast<unsigned long long>(to_fixed(g))));
+    __stcg(a + 1, make_ulonglong2(static_cast<unsigned long long>(to_fixed(b)), 1ull));
+  }
+  if (rec) st_once_u4(t.info + id, make_uint4(slot, h1, f, kOverflowSlot));
+}
+
+// Advance the last min(32, queued) queue entries by one step of their probe
+// sequences: read the next one or two slots (one 16-byte load when the slot is
+// even), take an empty one with a compare-and-swap; entries that met other
+// keys go back into the queue.  Slots are only ever filled within a frame, so
+// reading two at once is as good as one after the other: the first slot of
+// the sequence that holds the fingerprint or is empty decides, and an empty
+// one is taken only by its compare-and-swap.  All lanes.
+template <int W>
+__device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& v, WarpInsert<W>& s,
+                                           WarpShared& sh, bool rec, uint32_t* stash) {
+  const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
+  const uint32_t take = min(32u, s.queued), at = s.queued - take, e = at + lane;
+  const bool have = lane < take;
+  uint32_t h1 = 0u, f = 0u, step = 0u, members = 0u, first = 0u;
+  if (have) {
+    h1 = sh.h1[e];
+    f = sh.f[e];
+    step = sh.step[e];
+    members = sh.members[e];
+    first = sh.first[e];
+  }
+  s.reserve(0, have);
+  __syncwarp();
+  uint32_t id = kDeferred;
+  if (have) {
+    uint32_t slot = (h1 + step) & t.mask;
+    const ulonglong2 w = ld_relaxed_u64x2_keep(t.slots + (slot & ~1u));
+    unsigned long long a = slot & 1u ? w.y : w.x;
+    if (a != 0ull && slot_fp(a) != f && !(slot & 1u) && step + 1u < t.max_probes) {
+      a = w.y;
+      ++step;
+      ++slot;
+    }
+    uint32_t owner = 0u;
+    if (a == 0ull) {
+      a = atomicCAS(t.slots + slot, 0ull, slot_word(f, s.my[0]));
+      if (a == 0ull) owner = kOwnerBit;
+    }
+    const uint32_t lead = first + __ffs(members) - 1;
+    if (owner) {
+      id = s.my[0];
+      create_cell(t, id, __ldg(v.r + lead), __ldg(v.g + lead), __ldg(v.b + lead), slot, h1, f, rec);
+      ++s.cnt.cells;
+      s.my[0] = kOverflowSlot;
+    } else if (slot_fp(a) == f) {
+      id = slot_id(a);
+    } else if (++step >= t.max_probes) {
+      id = kOverflowSlot;
+      s.cnt.ovf += __popc(members);
+    }
+    if (id != kDeferred) {
+      st_once_u32(stash + lead, id | owner);
+      for (uint32_t m = members & (members - 1u); m; m &= m - 1u)
+        st_once_u32(stash + first + __ffs(m) - 1, id);
+    }
+  }
+  const unsigned again = __ballot_sync(0xFFFFFFFFu, id == kDeferred && have);
+  if (again >> lane & 1u) {
+    const uint32_t o = at + __popc(again & lt);
+    sh.h1[o] = h1;
+    sh.f[o] = f;
+    sh.step[o] = step;
+    sh.members[o] = members;
+    sh.first[o] = first;
+  }
+  s.queued = at + __popc(again);
+  __syncwarp();
+}
+
+// Pass one for the 32 W vertices from j0 on (those below `end`), one warp:
+// lane l takes vertices j0 + l, j0 + 32 + l, ...  Their cell ids go to
+// stash[vertex]: the id, with kOwnerBit for the cell's creator, or
+// kOverflowSlot on probe overflow; those of queued keys follow later.  New
+// cells take ids of the tile's own range; an id that a lane reserved and did
+// not need is used for its next new cell.
 //
-// The W vertices go through each step together so that their memory
-// operations overlap: keys; merging of equal keys among them (their
-// contributions are summed in registers and sent with one atomic); the first
-// probe of every distinct key (W loads in flight, then the compare-and-swaps
-// for empty slots); the rare longer probes; the accumulating reductions.
+// Equal keys within a row of 32 vertices go through the table once when
+// `merge` says so: 1 never; 2 when two neighbouring lanes hold equal keys,
+// which one shuffle and a vote find (coherent primary hits repeat keys across
+// neighbouring pixels, secondary bounces rarely repeat one within a warp, and
+// there the match costs more than the probes it saves); 3 always.
 //
 // `rec`: write each new cell's record (t.info) for the later blend and clear;
 // a frame that neither blends nor clears slot by slot never reads it.
-// KV: the vertices may carry the key variants (distance, extra word); the
-// persistent kernels are built without them.
-// KREC: also keep each new cell's quantized key in t.kw (for the history's
-// changes of resolution).
-template <int W, bool KV = false, bool KREC = false>
-__device__ __forceinline__ Batch<W> insert_batch(const KeyConst& kc, const TableDev& t,
-                                                 const VertexPtrs& v, size_t j, size_t end,
-                                                 bool vec, uint32_t id_base, uint32_t* claims,
-                                                 Counters& cnt_out, bool rec = true) {
-  float PX[W], PY[W], PZ[W], NX[W], NY[W], NZ[W];
-  loadw<W>(PX, v.px, j, end, vec);
-  loadw<W>(PY, v.py, j, end, vec);
-  loadw<W>(PZ, v.pz, j, end, vec);
-  loadw<W>(NX, v.nx, j, end, vec);
-  loadw<W>(NY, v.ny, j, end, vec);
-  loadw<W>(NZ, v.nz, j, end, vec);
+// KV: the vertices may carry the key variants (distance, extra word).
+// KREC: also keep each new cell's quantized key in t.kw (such tables finish
+// every key on the spot).
+template <int W, bool KV, bool KREC>
+__device__ __forceinline__ void insert_warp(const KeyConst& kc, const TableDev& t,
+                                            const VertexPtrs& v, size_t j0, size_t end,
+                                            WarpInsert<W>& s, WarpShared& sh, bool rec, int merge,
+                                            uint32_t* stash) {
+  const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
   uint32_t h1[W], f[W];
-  bool lead[W];
-  int of[W];
   uint4 kr[W];  // KREC: the quantized keys
+  {
+    float px[W], py[W], pz[W], nx[W], ny[W], nz[W];
 #pragma unroll
-  for (int q = 0; q < W; ++q) {
-    const bool valid = j + q < end;
-    Key k{0u, 0u};
-    kr[q] = make_uint4(0u, 0u, 0u, 0u);
-    if (valid) {
-      if constexpr (KREC) {
-        const KeyWords w = key_words(kc, PX[q], PY[q], PZ[q], NX[q], NY[q], NZ[q],
-                                     vertex_id(v, j + q), v.stream_id,
-                                     KV ? key_extra(v, j + q) : KeyExtra{});
-        k = key_hash(kc, w);
-        kr[q] = make_uint4(w.X, w.Y, w.Z, (w.L & 0xFFu) | (w.NQ << 8));
+    for (int q = 0; q < W; ++q) {
+      const size_t j = j0 + 32 * q + lane;
+      const bool ok = j < end;
+      px[q] = ok ? __ldcs(v.px + j) : 0.f;
+      py[q] = ok ? __ldcs(v.py + j) : 0.f;
+      pz[q] = ok ? __ldcs(v.pz + j) : 0.f;
+      nx[q] = ok ? __ldcs(v.nx + j) : 0.f;
+      ny[q] = ok ? __ldcs(v.ny + j) : 0.f;
+      nz[q] = ok ? __ldcs(v.nz + j) : 1.f;
+    }
+#pragma unroll
+    for (int q = 0; q < W; ++q) {
+      const size_t j = j0 + 32 * q + lane;
+      const bool ok = j < end;
+      const uint32_t vid = ok ? vertex_id(v, j) : 0u;
+      Key k;
+      if constexpr (KV || KREC) {
+        KeyExtra ke{};
+        if (KV && ok) ke = key_extra(v, j);
+        const KeyWords kw = key_words(kc, px[q], py[q], pz[q], nx[q], ny[q], nz[q], vid, v.stream_id, ke);
+        k = key_hash(kc, kw);
+        kr[q] = make_uint4(kw.X, kw.Y, kw.Z, (kw.L & 0xFFu) | (kw.NQ << 8));
       } else {
-        k = vertex_key(kc, PX[q], PY[q], PZ[q], NX[q], NY[q], NZ[q], vertex_id(v, j + q),
-                       v.stream_id, KV ? key_extra(v, j + q) : KeyExtra{});
+        k = vertex_key(kc, px[q], py[q], pz[q], nx[q], ny[q], nz[q], vid, v.stream_id);
       }
-    }
-    h1[q] = k.h1;
-    f[q] = k.fp;  // 0 marks an absent vertex (fingerprints are never 0)
-    lead[q] = valid;
-    of[q] = q;
-  }
-  // merge equal keys: a later vertex joins the first earlier one with its key
-#pragma unroll
-  for (int q = 1; q < W; ++q) {
-#pragma unroll
-    for (int p = 0; p < q; ++p) {
-      if (lead[q] && lead[p] && h1[p] == h1[q] && f[p] == f[q]) {
-        lead[q] = false;
-        of[q] = p;
-      }
+      h1[q] = k.h1;
+      f[q] = k.fp;
     }
   }
-  float rr[W], rg[W], rb[W];
-  loadw<W>(rr, v.r, j, end, vec);
-  loadw<W>(rg, v.g, j, end, vec);
-  loadw<W>(rb, v.b, j, end, vec);
-  long long xr[W], xg[W], xb[W];
+  unsigned grp[W];
+  uint32_t lead = 0u;  // bit q: this lane leads its group in row q
 #pragma unroll
   for (int q = 0; q < W; ++q) {
-    xr[q] = t.fixed ? to_fixed(rr[q]) : 0;
-    xg[q] = t.fixed ? to_fixed(rg[q]) : 0;
-    xb[q] = t.fixed ? to_fixed(rb[q]) : 0;
-  }
-  // group sums of each leader p over its members q >= p (static bounds, selects)
-  float sr[W], sg[W], sb[W];
-  long long fr[W], fg[W], fb[W];
-  uint32_t cnt[W];
-#pragma unroll
-  for (int p = 0; p < W; ++p) {
-    sr[p] = sg[p] = sb[p] = 0.f;
-    fr[p] = fg[p] = fb[p] = 0;
-    cnt[p] = 0u;
-#pragma unroll
-    for (int q = p; q < W; ++q) {
-      const bool m = f[q] != 0u && of[q] == p;
-      sr[p] = m ? __fadd_rn(sr[p], rr[q]) : sr[p];
-      sg[p] = m ? __fadd_rn(sg[p], rg[q]) : sg[p];
-      sb[p] = m ? __fadd_rn(sb[p], rb[q]) : sb[p];
-      fr[p] += m ? xr[q] : 0;
-      fg[p] += m ? xg[q] : 0;
-      fb[p] += m ? xb[q] : 0;
-      cnt[p] += m ? 1u : 0u;
+    const bool ok = j0 + 32 * q + lane < end;
+    const unsigned long long kk = (static_cast<unsigned long long>(h1[q]) << 32) | f[q];
+    bool match = merge == 3;
+    if (merge == 2) {
+      const unsigned long long up = __shfl_up_sync(0xFFFFFFFFu, kk, 1);
+      match = __ballot_sync(0xFFFFFFFFu, lane > 0 && ok && up == kk) != 0u;
     }
+    grp[q] = 1u << lane;
+    if (match) grp[q] = __match_any_sync(0xFFFFFFFFu, kk) & __ballot_sync(0xFFFFFFFFu, ok);
+    if (ok && (grp[q] & lt) == 0u) lead |= 1u << q;
+    s.reserve(q, lead >> q & 1u);
   }
-  // first probe step of every distinct key: loads in flight together
-  unsigned long long w[W];
-#pragma unroll
-  for (int q = 0; q < W; ++q)
-    w[q] = lead[q] ? ld_relaxed_u64_keep(t.slots + (h1[q] & t.mask)) : 1ull;
-  // an empty home needs a cell id to publish with the fingerprint
-  uint32_t my[W];
-#pragma unroll
-  for (int q = 0; q < W; ++q)
-    my[q] = lead[q] && w[q] == 0ull ? id_base + atomicAdd(claims, 1u) : kOverflowSlot;
   unsigned long long old[W];
 #pragma unroll
   for (int q = 0; q < W; ++q)
-    old[q] = my[q] != kOverflowSlot
-                 ? atomicCAS(t.slots + (h1[q] & t.mask), 0ull, slot_word(f[q], my[q]))
-                 : w[q];
-  uint32_t id[W], slot[W];
-  bool claimed[W];
-#pragma unroll
-  for (int q = 0; q < W; ++q) {
-    id[q] = kOverflowSlot;
-    slot[q] = kOverflowSlot;
-    claimed[q] = false;
-    if (!lead[q]) continue;
-    const uint32_t home = h1[q] & t.mask;
-    if (my[q] != kOverflowSlot && old[q] == 0ull) {
-      id[q] = my[q];
-      slot[q] = home;
-      claimed[q] = true;
-    } else if (slot_fp(old[q]) == f[q]) {
-      id[q] = slot_id(old[q]);
-      slot[q] = home;
-    } else {
-      // the home slot holds another key: keep probing (rare at low load)
-      const MoreProbe m = probe_more(t.slots, t.mask, t.max_probes, home, f[q], my[q], id_base,
-                                     claims);
-      slot[q] = m.slot;
-      id[q] = m.id;
-      my[q] = m.my;
-      claimed[q] = m.claimed;
-    }
-    // record the cell, or mark a reserved id that ended up unused
-    if (rec && my[q] != kOverflowSlot)
-      st_once_u4(t.info + my[q], claimed[q] ? make_uint4(slot[q], h1[q], f[q], kOverflowSlot)
-                                            : make_uint4(kNoSlot, 0u, 0u, kOverflowSlot));
-    if constexpr (KREC)
-      if (claimed[q]) __stcg(t.kw + my[q], kr[q]);
-  }
+    if (lead >> q & 1u)
+      old[q] = atomicCAS(t.slots + (h1[q] & t.mask), 0ull, slot_word(f[q], s.my[q]));
+  float r[W], g[W], b[W];
 #pragma unroll
   for (int q = 0; q < W; ++q)
-    if (lead[q] && id[q] != kOverflowSlot)
-      accumulate(t, id[q], sr[q], sg[q], sb[q], fr[q], fg[q], fb[q], cnt[q]);
-  Batch<W> out;
+    if (lead >> q & 1u) {
+      const size_t j = j0 + 32 * q + lane;
+      r[q] = __ldg(v.r + j);
+      g[q] = __ldg(v.g + j);
+      b[q] = __ldg(v.b + j);
+    }
 #pragma unroll
   for (int q = 0; q < W; ++q) {
-    uint32_t d = id[0];
-#pragma unroll
-    for (int p = 1; p <= q; ++p)
-      if (of[q] == p) d = id[p];
-    out.id[q] = f[q] == 0u ? kOverflowSlot : d;
-    if (f[q] != 0u && out.id[q] == kOverflowSlot) ++cnt_out.ovf;
-    cnt_out.cells += claimed[q] ? 1u : 0u;
+    const size_t j = j0 + 32 * q + lane;
+    uint32_t id = kDeferred, owner = 0u;
+    if (lead >> q & 1u) {
+      uint32_t slot = h1[q] & t.mask;
+      bool won = old[q] == 0ull;
+      if (won)
+        id = s.my[q];
+      else if (slot_fp(old[q]) == f[q])
+        id = slot_id(old[q]);
+      else if (t.max_probes == 1u)
+        id = kOverflowSlot;
+      if constexpr (KREC) {
+        if (id == kDeferred) {
+          id = kOverflowSlot;
+          slot = probe_rest(t, slot, f[q], 1u, s.my[q], id, won);
+        }
+        if (won) __stcg(t.kw + id, kr[q]);
+      }
+      if (won) {
+        create_cell(t, id, r[q], g[q], b[q], slot, h1[q], f[q], rec);
+        owner = kOwnerBit;
+        ++s.cnt.cells;
+        s.my[q] = kOverflowSlot;
+      }
+      if (id == kOverflowSlot) s.cnt.ovf += __popc(grp[q]);
+    }
+    const uint32_t mine = __shfl_sync(0xFFFFFFFFu, id, __ffs(grp[q]) - 1);
+    if (j < end && mine != kDeferred) st_once_u32(stash + j, mine | owner);
+    if constexpr (!KREC) {
+      const unsigned put = __ballot_sync(0xFFFFFFFFu, (lead >> q & 1u) && id == kDeferred);
+      if (put) {
+        if (put >> lane & 1u) {
+          const uint32_t o = s.queued + __popc(put & lt);
+          sh.h1[o] = h1[q];
+          sh.f[o] = f[q];
+          sh.step[o] = 1u;
+          sh.members[o] = grp[q];
+          sh.first[o] = static_cast<uint32_t>(j0 + 32 * q);
+        }
+        s.queued += __popc(put);
+        __syncwarp();
+        while (s.queued > kQueue - 32) queue_step<W>(t, v, s, sh, rec, stash);
+      }
+    }
   }
-  return out;
 }
 
-struct Result {
-  float r, g, b;
-  uint32_t n;
-  uint8_t status;
-};
+// Pass two for the 128 vertices from j0 on (those below `end`), one warp, four
+// rows of 32: the contributions of the vertices that do not own their cells.
+// Neighbouring vertices of the same cell are added up first, as in pass one.
+template <bool FIXED>
+__device__ __forceinline__ void add_warp_as(const TableDev& t, const VertexPtrs& v, size_t j0, size_t end,
+                                            const uint32_t* stash, int merge, WarpShared& sh) {
+  const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
+  constexpr int W = 4;
+  uint32_t id[W];
+  float r[W], g[W], b[W];
+#pragma unroll
+  for (int q = 0; q < W; ++q) {
+    const size_t j = j0 + 32 * q + lane;
+    id[q] = j < end ? __ldcg(stash + j) : kOverflowSlot;
+  }
+#pragma unroll
+  for (int q = 0; q < W; ++q) {
+    const size_t j = j0 + 32 * q + lane;
+    if (!(id[q] & kOwnerBit)) {  // neither an owner nor overflowed
+      r[q] = __ldcs(v.r + j);
+      g[q] = __ldcs(v.g + j);
+      b[q] = __ldcs(v.b + j);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < W; ++q) {
+    const bool ok = !(id[q] & kOwnerBit);
+    long long fr = 0, fg = 0, fb = 0;
+    if (FIXED && ok) {
+      fr = to_fixed(r[q]);
+      fg = to_fixed(g[q]);
+      fb = to_fixed(b[q]);
+    }
+    unsigned grp = 1u << lane;
+    if (merge != 1) {
+      const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, id[q], 1);
+      if (merge == 3 || __ballot_sync(0xFFFFFFFFu, lane > 0 && ok && up == id[q])) {
+        grp = __match_any_sync(0xFFFFFFFFu, id[q]);
+        if (ok) {
+          sh.row[lane] = r[q];
+          sh.row[32 + lane] = g[q];
+          sh.row[64 + lane] = b[q];
+        }
+        __syncwarp();
+        if (ok && (grp & lt) == 0u) {  // the group's lowest lane
+          for (unsigned m = grp & (grp - 1u); m; m &= m - 1u) {
+            const int l = __ffs(m) - 1;
+            const float mr = sh.row[l], mg = sh.row[32 + l], mb = sh.row[64 + l];
+            if (FIXED) {
+              fr += to_fixed(mr);
+              fg += to_fixed(mg);
+              fb += to_fixed(mb);
+            } else {
+              r[q] = __fadd_rn(r[q], mr);
+              g[q] = __fadd_rn(g[q], mg);
+              b[q] = __fadd_rn(b[q], mb);
+            }
+          }
+        }
+        __syncwarp();
+      }
+    }
+    if (ok && (grp & lt) == 0u) accumulate<FIXED>(t, id[q], r[q], g[q], b[q], fr, fg, fb, __popc(grp));
+  }
+}
+
+__device__ __forceinline__ void add_warp(const TableDev& t, const VertexPtrs& v, size_t j0, size_t end,
+                                         const uint32_t* stash, int merge, WarpShared& sh) {
+  if (t.fixed)
+    add_warp_as<true>(t, v, j0, end, stash, merge, sh);
+  else
+    add_warp_as<false>(t, v, j0, end, stash, merge, sh);
+}
+
+// The cell id of a stash word (kOverflowSlot: probe overflow).
+__device__ __forceinline__ uint32_t stash_id(uint32_t w) {
+  return w == kOverflowSlot ? w : w & ~kOwnerBit;
+}
 
 // Neighborhood search (Sec. 3.3.1) for vertex j, whose own cell holds fewer
 // than t.lowcount members: the pooled average of the 3 x 3 x 3 block of cells
@@ -535,129 +677,83 @@ __device__ __forceinline__ void resolve_batch(const TableDev& t, const VertexPtr
   }
 }
 
-template <int W>
-__device__ __forceinline__ void store_batch(const OutPtrs& o, size_t j, size_t end, bool vec,
-                                            const Result (&res)[W]) {
-  if (vec && j + W <= end) {
-    if constexpr (W == 4) {
-      __stcs(reinterpret_cast<float4*>(o.r + j), make_float4(res[0].r, res[1].r, res[2].r, res[3].r));
-      __stcs(reinterpret_cast<float4*>(o.g + j), make_float4(res[0].g, res[1].g, res[2].g, res[3].g));
-      __stcs(reinterpret_cast<float4*>(o.b + j), make_float4(res[0].b, res[1].b, res[2].b, res[3].b));
-      if (o.count)
-        __stcs(reinterpret_cast<uint4*>(o.count + j),
-               make_uint4(res[0].n, res[1].n, res[2].n, res[3].n));
-      if (o.status) {
-        const uint32_t w = res[0].status | (res[1].status << 8) | (res[2].status << 16) |
-                           (static_cast<uint32_t>(res[3].status) << 24);
-        __stcs(reinterpret_cast<unsigned int*>(o.status + j), w);
-      }
-    } else {
-      __stcs(reinterpret_cast<float2*>(o.r + j), make_float2(res[0].r, res[1].r));
-      __stcs(reinterpret_cast<float2*>(o.g + j), make_float2(res[0].g, res[1].g));
-      __stcs(reinterpret_cast<float2*>(o.b + j), make_float2(res[0].b, res[1].b));
-      if (o.count) __stcs(reinterpret_cast<uint2*>(o.count + j), make_uint2(res[0].n, res[1].n));
-      if (o.status) {
-        const unsigned short w = static_cast<unsigned short>(res[0].status | (res[1].status << 8));
-        __stcs(reinterpret_cast<unsigned short*>(o.status + j), w);
-      }
-    }
-    return;
-  }
-#pragma unroll
-  for (int q = 0; q < W; ++q) {
-    if (j + q < end) {
-      o.r[j + q] = res[q].r;
-      o.g[j + q] = res[q].g;
-      o.b[j + q] = res[q].b;
-      if (o.count) o.count[j + q] = res[q].n;
-      if (o.status) o.status[j + q] = res[q].status;
-    }
-  }
-}
-
-// Blend BW cells whose ids, history homes and fingerprints are known (`use`
-// false: no cell): history probes issued together, then the blends.
-template <int BW>
-__device__ __forceinline__ void blend_cells(const TableDev& t, const uint32_t (&d)[BW],
-                                            const uint32_t (&home)[BW], const uint32_t (&f)[BW],
-                                            const bool (&use)[BW], const AccRaw (&a)[BW],
-                                            float alpha, unsigned long long& n_hovf) {
-  uint32_t old[BW], h[BW];
-#pragma unroll
-  for (int q = 0; q < BW; ++q) old[q] = use[q] ? atomicCAS(hist_fp(t, home[q]), 0u, f[q]) : 0u;
-#pragma unroll
-  for (int q = 0; q < BW; ++q) {
-    h[q] = home[q];
-    if (use[q] && old[q] != 0u && old[q] != f[q]) h[q] = hist_probe_rest(t, home[q], f[q], 1u);
-    if (use[q] && h[q] == kOverflowSlot) ++n_hovf;
-  }
-  HistRaw hv[BW];
-#pragma unroll
-  for (int q = 0; q < BW; ++q) {
-    hv[q] = HistRaw{0.f, 0.f, 0.f, 0u};
-    if (use[q] && h[q] != kOverflowSlot) hv[q] = load_hist(t, h[q]);
-  }
-#pragma unroll
-  for (int q = 0; q < BW; ++q)
-    if (use[q]) blend_store(t, d[q], h[q], mean_of(t, a[q]), hv[q], alpha);
-}
-
-// The same for an evicting history (Sec. 3.4.3), one cell at a time, kept
-// out of line so that the common path above keeps its registers.
-__device__ __noinline__ unsigned long long blend_cell_evict(const TableDev& t, uint32_t d,
-                                                            uint32_t home, uint32_t f,
-                                                            float alpha) {
-  const AccRaw a = load_acc(t, d);
-  bool fresh = true;
-  const uint32_t h = hist_claim_evict(t, home, f, &fresh);
-  const HistRaw hv = h != kOverflowSlot && !fresh ? load_hist(t, h) : HistRaw{0.f, 0.f, 0.f, 0u};
-  blend_store(t, d, h, mean_of(t, a), hv, alpha);
-  return h == kOverflowSlot ? 1ull : 0ull;
-}
-
-// Blend the cells [base, base + count): each thread takes BW cells, one from
-// each of BW consecutive runs of `stride` ids (coalesced loads), and issues
-// their history probes together.  `first` is this thread's offset.
-template <int BW, bool EVICT>
-__device__ __forceinline__ void blend_range(const TableDev& t, uint32_t base, uint32_t count,
-                                            uint32_t first, uint32_t stride, float alpha,
+// Blend the cells of tiles first, first + stride, ... below ntiles (tile_i ids
+// each, bcount[tile] of them drawn), one warp.  Every lane carries one cell at a
+// time through its probe sequence and takes the next cell as soon as its own
+// is stored, so that a long probe holds up its lane only: a round reads one
+// history entry per lane, value and fingerprint in one load; an empty entry is
+// claimed with a compare-and-swap, an entry of another cell moves the lane's
+// probe on.
+template <bool EVICT>
+__device__ __forceinline__ void blend_tiles(const TableDev& t, uint32_t first, uint32_t stride,
+                                            uint32_t ntiles, uint32_t tile_i, float alpha,
                                             unsigned long long& n_hovf) {
-  for (uint32_t k0 = first; k0 < count; k0 += BW * stride) {
-    uint32_t d[BW], home[BW], f[BW];
-    bool use[BW];
-    AccRaw a[BW];
-#pragma unroll
-    for (int q = 0; q < BW; ++q) {
-      const uint32_t k = k0 + q * stride;
-      d[q] = base + k;
-      use[q] = false;
-      home[q] = 0u;
-      f[q] = 0u;
-      if (k < count) {
-        const uint4 in = ld_once_u4(t.info + d[q]);
-        use[q] = in.x != kNoSlot;
-        home[q] = in.y & t.hmask;
-        f[q] = in.z;
-        if (use[q] && !EVICT) a[q] = load_acc(t, d[q]);
+  const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
+  uint32_t tile = first, pos = 0u, count = tile < ntiles ? __ldcg(t.bcount + tile) : 0u;
+  bool busy = false;
+  uint32_t d = 0u, h = 0u, f = 0u, step = 0u;
+  AccRaw a;
+  for (;;) {
+    const unsigned idle = __ballot_sync(0xFFFFFFFFu, !busy);
+    if (idle && tile < ntiles) {
+      const uint32_t k = pos + __popc(idle & lt);
+      if (!busy && k < count) {
+        d = tile * tile_i + k;
+        const uint4 in = ld_once_u4(t.info + d);
+        a = load_acc(t, d);
+        if (in.x != kNoSlot) {
+          busy = true;
+          h = in.y & t.hmask;
+          f = in.z;
+          step = 0u;
+        }
       }
+      pos += __popc(idle);
+      if (pos >= count) {
+        tile += stride;
+        pos = 0u;
+        count = tile < ntiles ? __ldcg(t.bcount + tile) : 0u;
+      }
+    } else if (idle == 0xFFFFFFFFu) {
+      break;  // no tile left, no lane busy
     }
+    if (!busy) continue;
     if constexpr (EVICT) {
-#pragma unroll
-      for (int q = 0; q < BW; ++q)
-        if (use[q]) n_hovf += blend_cell_evict(t, d[q], home[q], f[q], alpha);
+      bool fresh = true;
+      const uint32_t e = hist_claim_evict(t, h, f, &fresh);
+      const HistRaw old = e != kOverflowSlot && !fresh ? load_hist(t, e) : HistRaw{0.f, 0.f, 0.f, 0u};
+      if (e == kOverflowSlot) ++n_hovf;
+      blend_store(t, d, e, (t.hist_rank << 24) | (f & 0xFFFFFFu), mean_of(t, a), old, alpha);
+      busy = false;
     } else {
-      blend_cells<BW>(t, d, home, f, use, a, alpha, n_hovf);
+      uint32_t fw;
+      HistRaw old = load_hist_fp(t, h, &fw);
+      if (fw == 0u) {
+        fw = atomicCAS(hist_fp(t, h), 0u, f);
+        // claimed, or taken meanwhile: by a cell whose value is this frame's
+        if (fw == 0u) fw = f;
+        old = HistRaw{0.f, 0.f, 0.f, 0u};
+      }
+      if (fw == f) {
+        blend_store(t, d, h, f, mean_of(t, a), old, alpha);
+        busy = false;
+      } else if (++step >= t.max_probes) {
+        ++n_hovf;
+        blend_store(t, d, kOverflowSlot, f, mean_of(t, a), old, alpha);
+        busy = false;
+      } else {
+        h = (h + 1u) & t.hmask;
+      }
     }
   }
 }
 
-// Empty the cells [base, base + count): their accumulators, and their slots
-// unless the whole slot table is swept separately (`slots_swept`).
+// Empty the slots of the cells [base, base + count).
 __device__ __forceinline__ void clear_range(const TableDev& t, uint32_t base, uint32_t count,
-                                            uint32_t first, uint32_t stride, bool slots_swept) {
+                                            uint32_t first, uint32_t stride) {
   for (uint32_t k = first; k < count; k += stride) {
-    const uint32_t slot = slots_swept ? kNoSlot : ld_once_u4(t.info + base + k).x;
-    clear_cell(t, base + k, slot);
+    const uint32_t slot = ld_once_u4(t.info + base + k).x;
+    if (slot != kNoSlot) __stcg(t.slots + slot, 0ull);
   }
 }
 
@@ -671,39 +767,47 @@ __device__ __forceinline__ void sweep_slots(const TableDev& t, size_t gid, size_
 }
 
 // ------------------------------------------------------------------ split path
+// Pass one of the insert, one warp per tile of kTile vertices; a tile's new
+// cells get ids from the tile's own range.
 template <int W, bool KREC>
 __global__ void __launch_bounds__(kBlock) k_insert(KeyConst kc, TableDev t, VertexPtrs v,
-                                                   size_t n, uint32_t* id_out, int vec,
-                                                   uint32_t tile_base) {
-  __shared__ uint32_t s_claims;
-  Counters c;
-  const size_t tiles = (n + kTile - 1) / kTile;
-  for (size_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-    if (threadIdx.x == 0) s_claims = 0;
-    __syncthreads();
-    const uint32_t tix = tile_base + static_cast<uint32_t>(tile);
+                                                   size_t n, uint32_t* stash, uint32_t tile_base,
+                                                   int merge) {
+  __shared__ WarpShared s_warp[kBlock / 32];
+  WarpShared& sh = s_warp[threadIdx.x >> 5];
+  WarpInsert<W> s;
+  const uint32_t tiles = static_cast<uint32_t>((n + kTile - 1) / kTile);
+  for (uint32_t tile = grid_warp(); tile < tiles; tile += grid_warps()) {
+    const uint32_t tix = tile_base + tile;
+    const size_t t0 = static_cast<size_t>(tile) * kTile, end = min(n, t0 + kTile);
+    s.claims = 0u;
+    s.id_base = tix * kTileIds;
 #pragma unroll 1
-    for (int sub = 0; sub < 4; sub += W) {
-      const size_t j = tile * kTile + threadIdx.x * 4 + sub;
-      if (j < n) {
-        const Batch<W> b =
-            insert_batch<W, true, KREC>(kc, t, v, j, n, vec != 0, tix * kTile, &s_claims, c);
-        if (id_out) {
-#pragma unroll
-          for (int q = 0; q < W; ++q)
-            if (j + q < n) id_out[j + q] = b.id[q];
-        }
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) t.bcount[tix] = s_claims;
+    for (size_t j0 = t0; j0 < end; j0 += 32 * W)
+      insert_warp<W, true, KREC>(kc, t, v, j0, end, s, sh, true, merge, stash);
+    if (tile + grid_warps() >= tiles)  // the warp's last
+      while (s.queued) queue_step<W>(t, v, s, sh, true, stash);
+    if ((threadIdx.x & 31u) == 0u) t.bcount[tix] = s.claims;
   }
-  const unsigned long long a = block_sum(static_cast<unsigned long long>(c.ovf));
-  const unsigned long long b = block_sum(static_cast<unsigned long long>(c.cells));
+  s.retire(t, true);
+  const unsigned long long a = block_sum(static_cast<unsigned long long>(s.cnt.ovf));
+  const unsigned long long b = block_sum(static_cast<unsigned long long>(s.cnt.cells));
   if (threadIdx.x == 0) {
     if (a) atomicAdd(&t.ctrl->overflow_vertices, a);
     if (b) atomicAdd(&t.ctrl->frame_cells, b);
     if (blockIdx.x == 0) atomicAdd(&t.ctrl->vertices, static_cast<unsigned long long>(n));
+  }
+}
+
+// Pass two; id_out (nullable): the vertices' cell ids for the caller.
+__global__ void __launch_bounds__(kBlock) k_add(TableDev t, VertexPtrs v, size_t n,
+                                                const uint32_t* stash, uint32_t* id_out, int merge) {
+  __shared__ WarpShared s_warp[kBlock / 32];
+  const uint32_t lane = threadIdx.x & 31u;
+  for (size_t j0 = grid_warp() * static_cast<size_t>(128); j0 < n; j0 += grid_warps() * static_cast<size_t>(128)) {
+    add_warp(t, v, j0, n, stash, merge, s_warp[threadIdx.x >> 5]);
+    if (id_out)
+      for (size_t j = j0 + lane; j < min(n, j0 + 128); j += 32) id_out[j] = stash_id(stash[j]);
   }
 }
 
@@ -759,11 +863,10 @@ __global__ void __launch_bounds__(kBlock) k_query(KeyConst kc, TableDev t, Verte
 
 __global__ void __launch_bounds__(kBlock) k_blend_sweep(TableDev t, uint32_t ntiles, float alpha) {
   unsigned long long n_hovf = 0;
-  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-    if (t.hist_evict)
-      blend_range<4, true>(t, tile * kTile, t.bcount[tile], threadIdx.x, blockDim.x, alpha, n_hovf);
-    else
-      blend_range<4, false>(t, tile * kTile, t.bcount[tile], threadIdx.x, blockDim.x, alpha, n_hovf);
+  if (t.hist_evict)
+    blend_tiles<true>(t, grid_warp(), grid_warps(), ntiles, kTileIds, alpha, n_hovf);
+  else
+    blend_tiles<false>(t, grid_warp(), grid_warps(), ntiles, kTileIds, alpha, n_hovf);
   const unsigned long long h = block_sum(n_hovf);
   if (threadIdx.x == 0 && h) atomicAdd(&t.ctrl->hist_overflow, h);
 }
@@ -844,9 +947,9 @@ __device__ __noinline__ HistRaw migrate_history(const KeyConst& kc, const TableD
 // entry in info.w; k_blend_apply blends and stores.
 __global__ void __launch_bounds__(kBlock) k_blend_lookup(KeyConst kc, TableDev t, uint32_t ntiles) {
   unsigned long long n_hovf = 0;
-  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const uint32_t base = tile * kTile, count = t.bcount[tile];
-    for (uint32_t k = threadIdx.x; k < count; k += blockDim.x) {
+  for (uint32_t tile = grid_warp(); tile < ntiles; tile += grid_warps()) {
+    const uint32_t base = tile * kTileIds, count = t.bcount[tile];
+    for (uint32_t k = threadIdx.x & 31u; k < count; k += 32) {
       const uint32_t d = base + k;
       const uint4 in = __ldcg(t.info + d);
       if (in.x == kNoSlot) continue;
@@ -869,15 +972,15 @@ __global__ void __launch_bounds__(kBlock) k_blend_lookup(KeyConst kc, TableDev t
 }
 
 __global__ void __launch_bounds__(kBlock) k_blend_apply(TableDev t, uint32_t ntiles, float alpha) {
-  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const uint32_t base = tile * kTile, count = t.bcount[tile];
-    for (uint32_t k = threadIdx.x; k < count; k += blockDim.x) {
+  for (uint32_t tile = grid_warp(); tile < ntiles; tile += grid_warps()) {
+    const uint32_t base = tile * kTileIds, count = t.bcount[tile];
+    for (uint32_t k = threadIdx.x & 31u; k < count; k += 32) {
       const uint32_t d = base + k;
       const uint4 in = __ldcg(t.info + d);
       if (in.x == kNoSlot) continue;
       const AccRaw a = load_acc(t, d);
       const float4 o = __ldcg(t.hold + d);
-      blend_store(t, d, in.w, mean_of(t, a), HistRaw{o.x, o.y, o.z, __float_as_uint(o.w)}, alpha);
+      blend_store(t, d, in.w, in.z, mean_of(t, a), HistRaw{o.x, o.y, o.z, __float_as_uint(o.w)}, alpha);
     }
   }
 }
@@ -892,12 +995,14 @@ __global__ void __launch_bounds__(kBlock) k_neighbors(KeyConst kc, TableDev t, V
     neighbors_of_queued(kc, t, v, o, __ldcs(nq + i), blended != 0);
 }
 
-__global__ void __launch_bounds__(kBlock) k_clear_sweep(TableDev t, uint32_t ntiles, int sweep) {
-  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-    clear_range(t, tile * kTile, t.bcount[tile], threadIdx.x, blockDim.x, sweep != 0);
+__global__ void __launch_bounds__(kBlock) k_clear_sweep(TableDev t, uint32_t ntiles, uint32_t tile_i,
+                                                        int sweep) {
   if (sweep)
     sweep_slots(t, blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x,
                 static_cast<size_t>(gridDim.x) * blockDim.x);
+  else
+    for (uint32_t tile = grid_warp(); tile < ntiles; tile += grid_warps())
+      clear_range(t, tile * tile_i, t.bcount[tile], threadIdx.x & 31u, 32);
 }
 
 __global__ void __launch_bounds__(kBlock) k_keys(KeyConst kc, VertexPtrs v, size_t n,
@@ -926,822 +1031,307 @@ __global__ void __launch_bounds__(kBlock) k_count_nonzero(const unsigned char* b
   if (threadIdx.x == 0 && s) atomicAdd(out, s);
 }
 
-// Empty the cells of the persistent kernel's tiles (kFusedTile ids each), for
-// the kernel variant that leaves them to a later launch.
-__global__ void __launch_bounds__(kBlock) k_clear_fused(TableDev t, uint32_t ntiles, int sweep) {
-  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-    clear_range(t, tile * static_cast<uint32_t>(kFusedTile), __ldcg(t.bcount + tile), threadIdx.x,
-                blockDim.x, sweep != 0);
-  if (sweep)
-    sweep_slots(t, blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x,
-                static_cast<size_t>(gridDim.x) * blockDim.x);
-}
-
 // ------------------------------------------------------------------ fused path
-// Offset in its tile of the first of the W vertices a thread takes in
-// sub-batch `sub` (0, W, ..): sub-batch k covers the k-th run of
-// kFusedBlock * W vertices, W consecutive ones per thread, so that each
-// warp's loads and stores of a stream are one contiguous run.
-template <int W, int BLOCK = kFusedBlock>
-__device__ __forceinline__ uint32_t fused_offset(int sub) {
-  return static_cast<uint32_t>(sub / W) * (BLOCK * W) + threadIdx.x * W;
-}
-
-// Next tile of the frame's tile counter (ntiles once all are taken), in
-// stream order or, with `backwards`, from the end of the vertex stream.  The
-// pipelined insert takes them backwards: streams are bounce-major, so the
-// secondary-bounce tiles, whose vertices nearly all create cells of their own
-// and cost the most, go first and the cheap primary-hit tiles balance the CTAs
-// at the end of the insert (HD plain frame 6 %, temporal 3 % shorter).  The
-// per-thread insert measured slower backwards (stress frame +3 %).
-__device__ __forceinline__ uint32_t claim_tile(Ctrl* ctrl, uint32_t ntiles, bool backwards = false) {
-  const unsigned long long k = atomicAdd(&ctrl->tile_next, 1ull);
-  if (k >= ntiles) return ntiles;
-  return backwards ? ntiles - 1u - static_cast<uint32_t>(k) : static_cast<uint32_t>(k);
-}
-
 struct FusedArgs {
   KeyConst kc;
   TableDev t;
   VertexPtrs v;
   OutPtrs o;
   size_t n;
-  uint32_t cap_tiles;  // tiles this CTA may take (its stash capacity)
-  uint32_t* gstash;    // global stash (indexed by vertex) when it does not fit on chip
+  uint32_t tile_v;   // vertices (and cell ids) per warp tile
+  uint32_t* stash;   // each vertex's cell id
   float alpha;
-  int vec, ovec, blend;
-  int sweep;     // zero the whole slot table at the end instead of slot by slot
-  uint32_t* nq;  // neighborhood search: the queue of low-count vertices
-  int merge;     // pipelined insert: 1 no warp aggregation, 2 gated, 3 always
+  int blend;
+  int sweep;         // zero the whole slot table first, instead of the frame's slots at the end
+  uint32_t* nq;      // neighborhood search: the queue of low-count vertices
+  int merge;         // merging of equal keys within a warp (insert_warp)
 };
 
-// The persistent kernel.  Phase A hands out tiles of kFusedTile consecutive
-// vertices from a per-frame counter, so CTAs that meet cheap (coherent)
-// vertices take more tiles; each CTA remembers its tiles, keeps every vertex's
-// cell id in its shared-memory stash, and later looks up and clears exactly
-// those tiles (the blend hands tiles out again from a second counter).  A
-// tile's new cells take ids from the tile's own range
-// [tile * kFusedTile, tile * kFusedTile + claims).
-template <bool TEMPORAL, int W, bool EVICT = false, bool NEIGH = false>
+// The warp's list of low-count vertices (in its shared memory, the key queue's
+// place) to the end of the frame's.
+constexpr uint32_t kLowList = kQueue * 5;
+__device__ __forceinline__ void flush_low(const TableDev& t, uint32_t* nq, WarpShared& sh, uint32_t& queued) {
+  const uint32_t lane = threadIdx.x & 31u;
+  __syncwarp();
+  unsigned long long b = 0ull;
+  if (lane == 0 && queued) b = atomicAdd(&t.ctrl->neigh_count, static_cast<unsigned long long>(queued));
+  b = __shfl_sync(0xFFFFFFFFu, b, 0);
+  for (uint32_t i = lane; i < queued; i += 32) nq[b + i] = sh.list[i];
+  __syncwarp();
+  queued = 0u;
+}
+
+// One lookup for each of the 128 vertices from j0 on (those below `end`), one
+// warp, four rows of 32: the vertices of a row mostly have cells of
+// neighbouring ids, so a row's loads fall on few lines.
+template <bool NEIGH>
+__device__ __forceinline__ void lookup_warp(const TableDev& t, const VertexPtrs& v, const OutPtrs& o,
+                                            size_t j0, size_t end, const uint32_t* stash,
+                                            bool blended, uint32_t* nq, WarpShared& sh, uint32_t& queued) {
+  const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
+  uint32_t id[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const size_t j = j0 + 32 * q + lane;
+    id[q] = j < end ? stash_id(__ldcs(stash + j)) : kOverflowSlot;
+  }
+  AccRaw a[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (id[q] != kOverflowSlot) a[q] = load_value(t, id[q], blended);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const size_t j = j0 + 32 * q + lane;
+    bool low = false;
+    if (j < end) {
+      CellMean m;
+      uint32_t status;
+      if (id[q] == kOverflowSlot) {
+        // probe limit exceeded: the unfiltered contribution of the vertex itself
+        m = CellMean{__ldcs(v.r + j), __ldcs(v.g + j), __ldcs(v.b + j), 0u};
+        status = 2u;
+      } else {
+        m = value_of(t, a[q], blended);
+        low = m.n < t.lowcount;
+        status = low ? 1u : 0u;
+      }
+      __stcs(o.r + j, m.r);
+      __stcs(o.g + j, m.g);
+      __stcs(o.b + j, m.b);
+      if (o.count) __stcs(o.count + j, m.n);
+      if (o.status) __stcs(o.status + j, static_cast<uint8_t>(status));
+    }
+    // neighborhood search: list the low-count vertices, for k_neighbors, which
+    // searches them at full occupancy (so the irregular searches neither
+    // unbalance this kernel's warps nor cost it registers).  They gather in
+    // shared memory first: one atomic on the list's counter per few hundred.
+    if constexpr (NEIGH) {
+      const unsigned m = __ballot_sync(0xFFFFFFFFu, low);
+      if (low) sh.list[queued + __popc(m & lt)] = static_cast<uint32_t>(j);
+      queued += __popc(m);
+    }
+  }
+  if constexpr (NEIGH)
+    if (queued > kLowList - 128u) flush_low(t, nq, sh, queued);
+}
+
+// The persistent kernel.  Every phase is a loop of independent warps:
+//   0   the slot table is emptied (sweep), just before it is filled, so that
+//       the compare-and-swaps meet it in L2;
+//   A1  keys, probing insert, in tiles of a.tile_v vertices, every nw-th tile
+//       to one warp (a counter that hands them out costs more than it
+//       balances: its atomics serialize on one address, HD 146 us against 126);
+//       a tile's new cells take ids from the tile's own range, and each
+//       vertex's cell id goes to the stash;
+//   A2  accumulation (128 vertices at a time);
+//   B   temporal blend of each tile's new cells;
+//   C   one lookup per vertex (128 at a time); a frame that did not sweep
+//       empties its slots,
+// with a grid barrier between them.
+template <bool TEMPORAL, int W, bool EVICT = false, bool NEIGH = false, bool KV = false>
 __global__ void __launch_bounds__(kFusedBlock, W == 4 ? 1 : 2) k_fused(FusedArgs a) {
-  extern __shared__ __align__(16) uint32_t s_stash[];
-  __shared__ uint32_t s_tile[kMaxTilesPerCta];
-  __shared__ uint32_t s_claims[kMaxTilesPerCta];
-  __shared__ uint32_t s_cur, s_taken;
-  __shared__ unsigned long long s_nv;  // vertices of this CTA's tiles
+  __shared__ WarpShared s_warp[kFusedBlock / 32];
+  WarpShared& sh = s_warp[threadIdx.x >> 5];
   const TableDev& t = a.t;
-  const uint32_t ntiles = static_cast<uint32_t>((a.n + kFusedTile - 1) / kFusedTile);
-  const bool vec = a.vec != 0;
-  if (threadIdx.x == 0) {
-    s_taken = 0;
-    s_nv = 0;
+  const uint32_t tile_v = a.tile_v, tile_i = tile_ids(tile_v, W), lane = threadIdx.x & 31u;
+  const uint32_t ntiles = static_cast<uint32_t>((a.n + tile_v - 1) / tile_v);
+  const uint32_t gw = grid_warp(), nw = grid_warps();
+  const bool blended = TEMPORAL && a.blend;
+  if (a.sweep) {
+    sweep_slots(t, blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x,
+                static_cast<size_t>(gridDim.x) * blockDim.x);
+    if (!grid_barrier(t.ctrl, gridDim.x)) return;
   }
 
-  // Phase A: keys, probing insert, accumulation, tile by tile.
-  Counters c;
-  for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t tile = ntiles;
-      if (s_taken < a.cap_tiles) tile = claim_tile(t.ctrl, ntiles);
-      s_cur = tile;
-      if (tile < ntiles) {
-        s_tile[s_taken] = tile;
-        s_claims[s_taken] = 0;
-        s_nv += min(a.n, static_cast<size_t>(tile) * kFusedTile + kFusedTile) -
-                static_cast<size_t>(tile) * kFusedTile;
-      }
-    }
-    __syncthreads();
-    const uint32_t tile = s_cur;
-    if (tile >= ntiles) break;
-    const uint32_t k = s_taken;
-    const size_t t0 = static_cast<size_t>(tile) * kFusedTile;
-    const size_t end = min(a.n, t0 + kFusedTile);
-    uint32_t* stash = a.gstash ? a.gstash + t0 : s_stash + static_cast<size_t>(k) * kFusedTile;
-#pragma unroll 1
-    for (int sub = 0; sub < 4; sub += W) {
-      const size_t j = t0 + fused_offset<W>(sub);
-      if (j < end) {
-        const Batch<W> b = insert_batch<W>(a.kc, t, a.v, j, end, vec, static_cast<uint32_t>(t0),
-                                           &s_claims[k], c,
-                                           (TEMPORAL && a.blend) || !a.sweep);
-#pragma unroll
-        for (int q = 0; q < W; ++q) stash[j - t0 + q] = b.id[q];
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      // for the blend, which any CTA may take, and for the separate clear
-      if ((TEMPORAL && a.blend) || NEIGH) __stcg(t.bcount + tile, s_claims[k]);
-      ++s_taken;
-    }
-  }
   {
-    const unsigned long long o = block_sum(static_cast<unsigned long long>(c.ovf));
-    const unsigned long long k = block_sum(static_cast<unsigned long long>(c.cells));
+    WarpInsert<W> s;
+    const bool rec = blended || !a.sweep;
+    for (uint32_t k = gw; k < ntiles; k += nw) {
+      // from the end of the vertex stream: streams are bounce-major, so the
+      // secondary-bounce tiles, whose vertices nearly all create cells of
+      // their own and cost the most, go first and the cheap primary-hit tiles
+      // balance the warps at the end
+      const uint32_t tile = ntiles - 1u - k;
+      const size_t t0 = static_cast<size_t>(tile) * tile_v;
+      const size_t end = min(a.n, t0 + tile_v);
+      s.claims = 0u;
+      s.id_base = tile * tile_i;
+#pragma unroll 1
+      for (size_t j0 = t0; j0 < end; j0 += 32 * W)
+        insert_warp<W, KV, false>(a.kc, t, a.v, j0, end, s, sh, rec, a.merge, a.stash);
+      if (k + nw >= ntiles)  // the warp's last tile
+        while (s.queued) queue_step<W>(t, a.v, s, sh, rec, a.stash);
+      if (lane == 0) __stcg(t.bcount + tile, s.claims);
+    }
+    s.retire(t, rec);
+    const unsigned long long o = block_sum(static_cast<unsigned long long>(s.cnt.ovf));
+    const unsigned long long c = block_sum(static_cast<unsigned long long>(s.cnt.cells));
     if (threadIdx.x == 0) {
       if (o) atomicAdd(&t.ctrl->overflow_vertices, o);
-      if (k) atomicAdd(&t.ctrl->frame_cells, k);
-      if (s_nv) atomicAdd(&t.ctrl->vertices, s_nv);
+      if (c) atomicAdd(&t.ctrl->frame_cells, c);
+      if (blockIdx.x == 0) atomicAdd(&t.ctrl->vertices, static_cast<unsigned long long>(a.n));
     }
   }
   if (!grid_barrier(t.ctrl, gridDim.x)) return;
-  const uint32_t taken = s_taken;
 
-  // Phase B: temporal blend of the frame's cells, tile by tile from a second
-  // counter, so that CTAs whose tiles created few cells take more.
-  const bool blended = TEMPORAL && a.blend;
+  for (size_t j = gw * static_cast<size_t>(128); j < a.n; j += nw * static_cast<size_t>(128))
+    add_warp(t, a.v, j, a.n, a.stash, a.merge, sh);
+  if (!grid_barrier(t.ctrl, gridDim.x)) return;
+
   if (blended) {
     unsigned long long n_hovf = 0;
-    for (;;) {
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        const unsigned long long b = atomicAdd(&t.ctrl->blend_next, 1ull);
-        s_cur = b < ntiles ? static_cast<uint32_t>(b) : ntiles;
-      }
-      __syncthreads();
-      const uint32_t tile = s_cur;
-      if (tile >= ntiles) break;
-      blend_range<W, EVICT>(t, tile * static_cast<uint32_t>(kFusedTile), __ldcg(t.bcount + tile),
-                            threadIdx.x, blockDim.x, a.alpha, n_hovf);
-    }
+    blend_tiles<EVICT>(t, gw, nw, ntiles, tile_i, a.alpha, n_hovf);
     const unsigned long long h = block_sum(n_hovf);
     if (threadIdx.x == 0 && h) atomicAdd(&t.ctrl->hist_overflow, h);
     if (!grid_barrier(t.ctrl, gridDim.x)) return;
   }
 
-  // Phase C: one lookup per vertex of this CTA's tiles.
-  const bool ovec = a.ovec != 0;
-  for (uint32_t k = 0; k < taken; ++k) {
-    const size_t t0 = static_cast<size_t>(s_tile[k]) * kFusedTile;
-    const size_t end = min(a.n, t0 + kFusedTile);
-    const uint32_t* stash = a.gstash ? a.gstash + t0 : s_stash + static_cast<size_t>(k) * kFusedTile;
-#pragma unroll 1
-    for (int sub = 0; sub < 4; sub += W) {
-      const size_t j = t0 + fused_offset<W>(sub);
-      if (j < end) {
-        uint32_t id[W];
-#pragma unroll
-        for (int q = 0; q < W; ++q) id[q] = stash[j - t0 + q];
-        Result res[W];
-        resolve_batch<W>(t, a.v, j, end, id, blended, res);
-        store_batch<W>(a.o, j, end, ovec, res);
-      }
-    }
-  }
-  // Neighborhood search: this kernel variant only queues its low-count
-  // vertices (one atomic per warp); k_neighbors then searches the whole queue
-  // at full occupancy and k_clear_fused empties the cells, so that the
-  // irregular searches neither unbalance the persistent CTAs nor cost the
-  // persistent kernel registers.
-  if constexpr (NEIGH) {
-    const int lane = threadIdx.x & 31;
-    for (uint32_t k = 0; k < taken; ++k) {
-      const size_t t0 = static_cast<size_t>(s_tile[k]) * kFusedTile;
-      const size_t end = min(a.n, t0 + kFusedTile);
-      const uint32_t* stash = a.gstash ? a.gstash + t0 : s_stash + static_cast<size_t>(k) * kFusedTile;
-      for (size_t base = t0 + (threadIdx.x & ~31u); base < end; base += blockDim.x) {
-        const size_t j = base + lane;
-        bool low = false;
-        if (j < end) {
-          const uint32_t id = stash[j - t0];
-          low = id != kOverflowSlot &&
-                value_of(t, load_value(t, id, blended), blended).n < t.lowcount;
-        }
-        const unsigned mask = __ballot_sync(0xFFFFFFFFu, low);
-        if (mask) {
-          unsigned long long b0 = 0ull;
-          if (lane == 0) b0 = atomicAdd(&t.ctrl->neigh_count, static_cast<unsigned long long>(__popc(mask)));
-          b0 = __shfl_sync(0xFFFFFFFFu, b0, 0);
-          if (low) a.nq[b0 + __popc(mask & ((1u << lane) - 1u))] = static_cast<uint32_t>(j);
-        }
-      }
-    }
-    return;
-  }
-  if (!grid_barrier(t.ctrl, gridDim.x)) return;
-
-  // Phase D: empty the cells this CTA's tiles created (and, when many slots
-  // are in use, sweep the slot table instead of clearing slot by slot).
-  for (uint32_t k = 0; k < taken; ++k)
-    clear_range(t, s_tile[k] * static_cast<uint32_t>(kFusedTile), s_claims[k], threadIdx.x,
-                blockDim.x, a.sweep != 0);
-  if (a.sweep)
-    sweep_slots(t, blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x,
-                static_cast<size_t>(gridDim.x) * blockDim.x);
+  uint32_t low = 0u;  // listed vertices not handed on yet
+  for (size_t j = gw * static_cast<size_t>(128); j < a.n; j += nw * static_cast<size_t>(128))
+    lookup_warp<NEIGH>(t, a.v, a.o, j, a.n, a.stash, blended, a.nq, sh, low);
+  if (NEIGH) flush_low(t, a.nq, sh, low);
+  if (!NEIGH && !a.sweep)  // (the neighborhood search still reads the slots)
+    for (uint32_t tile = gw; tile < ntiles; tile += nw)
+      clear_range(t, tile * tile_i, __ldcg(t.bcount + tile), lane, 32);
 }
 
-// ------------------------------------------------------------------ pipelined insert
-// k_fused_ws: the persistent kernel with its insert (phase A) split between
-// two groups of warps that work on different chunks of vertices at once.
-//
-//  key warps    read a chunk's vertex streams (coalesced; two vertices per
-//               thread at a time, whose keys are built together so that their
-//               chains of Philox rounds and hash steps overlap), build each
-//               vertex's key (Algorithm 1), merge equal keys within the
-//               warp (__match_any_sync: the lowest lane of each group of equal
-//               keys becomes its leader and the members add their
-//               contributions to the leader's entry with shared-memory
-//               atomics), and append one queue entry per distinct key:
-//               {home hash, fingerprint, member lanes, first vertex of the
-//               warp} and the group's sums and count.
-//  probe warps  take a full chunk's entries, four per thread at a time, and
-//               run the table operations of Sec. 3.2 for all four together
-//               (first probes, id claims, compare-and-swaps, the rare longer
-//               probes, then the accumulating reductions); each entry's cell id
-//               goes to the stash word of every member vertex.
-//
-// Two queue buffers alternate, so the key warps fill one chunk while the
-// probe warps drain the other.  The handover uses two mbarriers per buffer
-// (full: every key thread arrives after writing its entries; empty: every
-// probe thread arrives after reading them), waited with a bounded
-// try_wait loop (about two seconds of wall time, then kErrBarrierTimeout and
-// the launch ends like a timed-out grid barrier).  The key warps decide
-// together whether to go on (a named-barrier AND vote), so none of them is
-// left waiting at a barrier.  The stash is the global one (indexed by
-// vertex); phases B, C and D are those of k_fused.  Cell records, stash words
-// and history cells are written and read with an evict-first L2 policy, so
-// that the slot index and the accumulators stay in L2.
-constexpr int kWsChunk = 1024;  // vertices per queue chunk: half a tile
-constexpr int kWsChunksPerTile = kFusedTile / kWsChunk;
-constexpr uint32_t kWsEnd = 0xFFFFFFFFu;  // chunk header: no more tiles
-
-struct WsHeader {
-  uint32_t count;  // entries in the chunk
-  uint32_t k;      // the tile's place in this CTA's tile list
-  uint32_t tile;   // the tile, or kWsEnd
-};
-
-__device__ __forceinline__ void mbar_init(uint64_t* m, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(
-                   static_cast<uint32_t>(__cvta_generic_to_shared(m))),
-               "r"(count)
-               : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* m) {
-  unsigned long long state;
-  asm volatile("mbarrier.arrive.shared::cta.b64 %0, [%1];"
-               : "=l"(state)
-               : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(m)))
-               : "memory");
-  (void)state;
-}
-
-// Wait for the phase of parity `parity` of mbarrier m to complete, for about
-// `limit_ns` of wall time at most; false when the wait gave up.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* m, uint32_t parity,
-                                                  unsigned long long limit_ns = 2000000000ull) {
-  const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(m));
-  const unsigned long long t0 = globaltimer_ns();
-  for (;;) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (globaltimer_ns() - t0 > limit_ns) return false;
-  }
-}
-
-// AND of `pred` over the `nthreads` threads that use named barrier `id`.
-__device__ __forceinline__ bool bar_and(int id, int nthreads, bool pred) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n"
-      " bar.red.and.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}"
-      : "=r"(r)
-      : "r"(pred ? 1u : 0u), "r"(id), "r"(nthreads)
-      : "memory");
-  return r != 0;
-}
-
-// Shared-memory layout of k_fused_ws (dynamic part): 2 headers, 4 mbarriers
-// (full[2], empty[2]), two queue buffers of kWsChunk entries and their FP32
-// group sums {r, g, b, count} (fixed-point tables leave the sums to the probe
-// warps, which add the members' contributions exactly in int64).
-struct WsLayout {
-  static constexpr size_t kHeaders = 64;
-  __host__ __device__ static constexpr size_t keys_off() { return kHeaders; }
-  __host__ __device__ static constexpr size_t sums_off() {
-    return kHeaders + 2 * kWsChunk * sizeof(uint4);
-  }
-  __host__ __device__ static constexpr size_t sum_words(bool) { return 1; }
-  __host__ __device__ static constexpr size_t bytes(bool fixed) {
-    return sums_off() + 2 * kWsChunk * sum_words(fixed) * sizeof(float4);
-  }
-};
-
-// Append the queue entry of vertex j (valid) of this warp's lanes `vm` (the
-// valid lanes are consecutive vertices): merge equal keys among the warp's
-// lanes (the lowest lane of a group leads, the others add their contributions
-// to its entry), one entry per group.  `merge`: 1 no merging (every lane its
-// own group); 2 merge only when two neighbouring lanes hold equal keys, which
-// one shuffle and a vote find (coherent primary hits repeat keys across
-// neighbouring pixels, secondary bounces rarely repeat one within a warp, and
-// there the match costs more than the probes it saves); 3 always merge.
-__device__ __forceinline__ void ws_enqueue(const TableDev& t, uint4* keys, float4* sums, WsHeader* h,
-                                           unsigned vm, const Key& k, size_t j, float r, float g,
-                                           float b, int merge) {
-  const uint32_t lane = threadIdx.x & 31;
-  const unsigned long long kk = (static_cast<unsigned long long>(k.h1) << 32) | k.fp;
-  bool match = merge == 3;
-  if (merge == 2) {
-    const unsigned long long up = __shfl_up_sync(vm, kk, 1);
-    match = __ballot_sync(vm, lane > 0 && up == kk) != 0u;
-  }
-  const unsigned grp = match ? __match_any_sync(vm, kk) : 1u << lane;
-  const uint32_t leader = __ffs(grp) - 1;
-  const bool lead = leader == lane;
-  const unsigned lm = __ballot_sync(vm, lead);
-  const uint32_t first = __ffs(vm) - 1;
-  uint32_t e = 0;
-  if (lane == first) e = atomicAdd(&h->count, static_cast<uint32_t>(__popc(lm)));
-  e = __shfl_sync(vm, e, first) + __popc(lm & ((1u << lane) - 1u));
-  e = __shfl_sync(vm, e, leader);
-  if (lead) {
-    keys[e] = make_uint4(k.h1, k.fp, grp, static_cast<uint32_t>(j - lane));
-    if (!t.fixed)
-      sums[e] = make_float4(r, g, b, __uint_as_float(static_cast<uint32_t>(__popc(grp))));
-  }
-  // fixed point: the probe warps sum the members exactly; no match: every lane leads
-  if (t.fixed || !match) return;
-  __syncwarp(vm);
-  if (!lead) {
-    atomicAdd(&sums[e].x, r);
-    atomicAdd(&sums[e].y, g);
-    atomicAdd(&sums[e].z, b);
-  }
-}
-
-// The key warps' work on one chunk [c0, c0 + kWsChunk) of the vertices below
-// `end`: KV vertices per thread at a time (KT apart, so that each warp's loads
-// of a stream are one coalesced run), their keys built together so that the
-// independent chains of Philox rounds and hash steps overlap.
-template <int KEYW, int KV>
-__device__ __forceinline__ void ws_key_chunk(const FusedArgs& a, uint4* keys, float4* sums,
-                                             WsHeader* h, size_t c0, size_t end) {
-  const TableDev& t = a.t;
-  const VertexPtrs& v = a.v;
-  constexpr int KT = KEYW * 32;
-  const size_t cend = min(end, c0 + kWsChunk);
-#pragma unroll 1
-  for (size_t base = c0 + threadIdx.x; base < c0 + kWsChunk; base += KV * KT) {
-    float px[KV], py[KV], pz[KV], nx[KV], ny[KV], nz[KV], r[KV], g[KV], b[KV];
-#pragma unroll
-    for (int q = 0; q < KV; ++q) {
-      const size_t j = base + q * KT;
-      const bool ok = j < cend;
-      px[q] = ok ? __ldcs(v.px + j) : 0.f;
-      py[q] = ok ? __ldcs(v.py + j) : 0.f;
-      pz[q] = ok ? __ldcs(v.pz + j) : 0.f;
-      nx[q] = ok ? __ldcs(v.nx + j) : 0.f;
-      ny[q] = ok ? __ldcs(v.ny + j) : 0.f;
-      nz[q] = ok ? __ldcs(v.nz + j) : 1.f;
-      const bool rgb = ok && !t.fixed;  // fixed point: summed by the probe warps
-      r[q] = rgb ? __ldcs(v.r + j) : 0.f;
-      g[q] = rgb ? __ldcs(v.g + j) : 0.f;
-      b[q] = rgb ? __ldcs(v.b + j) : 0.f;
-    }
-    Key k[KV];
-#pragma unroll
-    for (int q = 0; q < KV; ++q) {
-      const size_t j = base + q * KT;
-      k[q] = vertex_key(a.kc, px[q], py[q], pz[q], nx[q], ny[q], nz[q],
-                        j < cend ? vertex_id(v, j) : 0u, v.stream_id);
-    }
-#pragma unroll
-    for (int q = 0; q < KV; ++q) {
-      const size_t j = base + q * KT;
-      const bool valid = j < cend;
-      const unsigned vm = __ballot_sync(0xFFFFFFFFu, valid);
-      if (valid) ws_enqueue(t, keys, sums, h, vm, k[q], j, r[q], g[q], b[q], a.merge);
-    }
-  }
-}
-
-// One probe thread's entries e0, e0 + stride, ... (at most 4) of a chunk:
-// the table operations of all of them together.
-template <int PB>
-__device__ __forceinline__ void ws_probe_group(const TableDev& t, const VertexPtrs& v,
-                                               const uint4* keys,
-                                               const float4* sums, uint32_t q, uint32_t e0,
-                                               uint32_t stride, uint32_t id_base,
-                                               uint32_t* claims, uint32_t* gstash, bool rec,
-                                               Counters& cnt) {
-  uint32_t h1[PB], f[PB], mask[PB], vb[PB];
-  bool use[PB];
-#pragma unroll
-  for (int i = 0; i < PB; ++i) {
-    const uint32_t e = e0 + i * stride;
-    use[i] = e < q;
-    const uint4 kq = use[i] ? keys[e] : make_uint4(0u, 0u, 0u, 0u);
-    h1[i] = kq.x;
-    f[i] = kq.y;
-    mask[i] = kq.z;
-    vb[i] = kq.w;
-  }
-  unsigned long long w[PB];
-#pragma unroll
-  for (int i = 0; i < PB; ++i) w[i] = use[i] ? ld_relaxed_u64_keep(t.slots + (h1[i] & t.mask)) : 1ull;
-  // ids for the entries whose first probe found an empty slot: one
-  // shared-memory atomic per warp, the lanes' ids in (entry, lane) order
-  uint32_t my[PB];
-  {
-    // the lanes of this warp in this call: those whose first entry is below q
-    const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
-    const uint32_t e_lane0 = e0 - lane;
-    const uint32_t nin = q > e_lane0 ? min(32u, q - e_lane0) : 0u;
-    const unsigned am = nin >= 32u ? 0xFFFFFFFFu : (1u << nin) - 1u;
-    unsigned bm[PB];
-    uint32_t tot = 0;
-#pragma unroll
-    for (int i = 0; i < PB; ++i) {
-      bm[i] = __ballot_sync(am, use[i] && w[i] == 0ull);
-      tot += __popc(bm[i]);
-    }
-    const uint32_t first = __ffs(am) - 1u;
-    uint32_t base = 0;
-    if (lane == first && tot) base = atomicAdd(claims, tot);
-    base = __shfl_sync(am, base, first);
-    uint32_t off = 0;
-#pragma unroll
-    for (int i = 0; i < PB; ++i) {
-      my[i] = (bm[i] >> lane) & 1u ? id_base + base + off + __popc(bm[i] & lt) : kOverflowSlot;
-      off += __popc(bm[i]);
-    }
-  }
-  unsigned long long old[PB];
-#pragma unroll
-  for (int i = 0; i < PB; ++i)
-    old[i] = my[i] != kOverflowSlot
-                 ? atomicCAS(t.slots + (h1[i] & t.mask), 0ull, slot_word(f[i], my[i]))
-                 : w[i];
-  uint32_t id[PB];
-#pragma unroll
-  for (int i = 0; i < PB; ++i) {
-    id[i] = kOverflowSlot;
-    if (!use[i]) continue;
-    const uint32_t home = h1[i] & t.mask;
-    uint32_t slot = home;
-    bool claimed = false;
-    if (my[i] != kOverflowSlot && old[i] == 0ull) {
-      id[i] = my[i];
-      claimed = true;
-    } else if (slot_fp(old[i]) == f[i]) {
-      id[i] = slot_id(old[i]);
-    } else {
-      const MoreProbe m = probe_more(t.slots, t.mask, t.max_probes, home, f[i], my[i], id_base,
-                                     claims);
-      slot = m.slot;
-      id[i] = m.id;
-      my[i] = m.my;
-      claimed = m.claimed;
-    }
-    if (rec && my[i] != kOverflowSlot)
-      st_once_u4(t.info + my[i], claimed ? make_uint4(slot, h1[i], f[i], kOverflowSlot)
-                                         : make_uint4(kNoSlot, 0u, 0u, kOverflowSlot));
-    cnt.cells += claimed ? 1u : 0u;
-  }
-#pragma unroll
-  for (int i = 0; i < PB; ++i) {
-    if (!use[i]) continue;
-    const uint32_t e = e0 + i * stride;
-    if (id[i] != kOverflowSlot) {
-      if (!t.fixed) {
-        const float4 s = sums[e];
-        red_add_v4_keep(t.acc + id[i], s.x, s.y, s.z, static_cast<float>(__float_as_uint(s.w)));
-      } else {
-        // exact int64 sums of the members' fixed-point contributions
-        long long fr = 0, fg = 0, fb = 0;
-        for (uint32_t m = mask[i]; m; m &= m - 1u) {
-          const uint32_t j = vb[i] + __ffs(m) - 1;
-          fr += to_fixed(__ldg(v.r + j));
-          fg += to_fixed(__ldg(v.g + j));
-          fb += to_fixed(__ldg(v.b + j));
-        }
-        accumulate(t, id[i], 0.f, 0.f, 0.f, fr, fg, fb, __popc(mask[i]));
-      }
-    } else {
-      cnt.ovf += __popc(mask[i]);
-    }
-    for (uint32_t m = mask[i]; m; m &= m - 1u) st_once_u32(gstash + vb[i] + __ffs(m) - 1, id[i]);
-  }
-}
-
-template <bool TEMPORAL, int KEYW, int PRW, int KV>
-__global__ void __launch_bounds__((KEYW + PRW) * 32, 2) k_fused_ws(FusedArgs a) {
-  extern __shared__ __align__(16) unsigned char s_dyn[];
-  __shared__ uint32_t s_tile[kMaxTilesPerCta];
-  __shared__ uint32_t s_claims[kMaxTilesPerCta];
-  __shared__ uint32_t s_cur, s_taken;
-  constexpr int KT = KEYW * 32, PT = PRW * 32;
-  const TableDev& t = a.t;
-  const uint32_t ntiles = static_cast<uint32_t>((a.n + kFusedTile - 1) / kFusedTile);
-  WsHeader* hdr = reinterpret_cast<WsHeader*>(s_dyn);
-  uint64_t* full = reinterpret_cast<uint64_t*>(s_dyn + 32);
-  uint64_t* empty = full + 2;
-  uint4* keys = reinterpret_cast<uint4*>(s_dyn + WsLayout::keys_off());
-  float4* sums = reinterpret_cast<float4*>(s_dyn + WsLayout::sums_off());
-  const size_t sw = WsLayout::sum_words(t.fixed != 0);
-  if (threadIdx.x == 0) {
-    s_taken = 0;
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(full + b, KT);
-      mbar_init(empty + b, PT);
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-
-  // Phase A: key warps and probe warps on alternate chunks.
-  Counters c;
-  unsigned long long nv = 0;  // vertices of this CTA's tiles (key thread 0)
-  bool ok = true;
-  if (threadIdx.x < KT) {
-    uint32_t tile = 0, k = 0;
-    for (uint32_t ch = 0;; ++ch) {
-      const uint32_t bsel = ch & 1u;
-      bool go = true;
-      if (ch >= 2) go = mbar_wait_bounded(empty + bsel, ((ch >> 1) + 1u) & 1u);
-      if (threadIdx.x == 0 && go) {
-        if (ch % kWsChunksPerTile == 0) {
-          tile = s_taken < a.cap_tiles ? claim_tile(t.ctrl, ntiles, true) : ntiles;
-          if (tile < ntiles) {
-            k = s_taken;
-            s_tile[k] = tile;
-            s_claims[k] = 0;
-            s_taken = k + 1;
-            nv += min(a.n, static_cast<size_t>(tile) * kFusedTile + kFusedTile) -
-                  static_cast<size_t>(tile) * kFusedTile;
-          }
-        }
-        hdr[bsel].count = 0;
-        hdr[bsel].k = k;
-        hdr[bsel].tile = tile < ntiles ? tile : kWsEnd;
-      }
-      go = bar_and(1, KT, go);  // also publishes the header to the key warps
-      if (!go) {
-        ok = false;
-        break;
-      }
-      // this buffer's header is rewritten only after the probe warps have
-      // released it, which needs every key thread's arrival for this chunk
-      const uint32_t cur = hdr[bsel].tile;
-      if (cur != kWsEnd) {
-        const size_t t0 = static_cast<size_t>(cur) * kFusedTile;
-        ws_key_chunk<KEYW, KV>(a, keys + bsel * kWsChunk, sums + bsel * kWsChunk * sw, hdr + bsel,
-                           t0 + (ch % kWsChunksPerTile) * kWsChunk, min(a.n, t0 + kFusedTile));
-      }
-      mbar_arrive(full + bsel);
-      if (cur == kWsEnd) break;
-    }
-  } else {
-    const uint32_t pt = threadIdx.x - KT;
-    const bool rec = (TEMPORAL && a.blend) || !a.sweep;
-    for (uint32_t ch = 0;; ++ch) {
-      const uint32_t bsel = ch & 1u;
-      if (!mbar_wait_bounded(full + bsel, (ch >> 1) & 1u)) {
-        ok = false;
-        break;
-      }
-      const WsHeader hh = hdr[bsel];
-      if (hh.tile == kWsEnd) break;
-      const uint32_t id_base = hh.tile * static_cast<uint32_t>(kFusedTile);
-      const uint4* kq = keys + bsel * kWsChunk;
-      const float4* sq = sums + bsel * kWsChunk * sw;
-#pragma unroll 1
-      for (uint32_t e0 = pt; e0 < hh.count; e0 += 4 * PT)
-        ws_probe_group<4>(t, a.v, kq, sq, hh.count, e0, PT, id_base, &s_claims[hh.k], a.gstash, rec,
-                          c);
-      mbar_arrive(empty + bsel);
-    }
-  }
-  if (!ok) atomicOr(&t.ctrl->error, kErrBarrierTimeout);
-  __syncthreads();
-  const uint32_t taken = s_taken;
-  {
-    const unsigned long long o = block_sum(static_cast<unsigned long long>(c.ovf));
-    const unsigned long long kk = block_sum(static_cast<unsigned long long>(c.cells));
-    if (threadIdx.x == 0) {
-      if (o) atomicAdd(&t.ctrl->overflow_vertices, o);
-      if (kk) atomicAdd(&t.ctrl->frame_cells, kk);
-      if (nv) atomicAdd(&t.ctrl->vertices, nv);
-      if (TEMPORAL && a.blend)
-        for (uint32_t i = 0; i < taken; ++i) __stcg(t.bcount + s_tile[i], s_claims[i]);
-    }
-  }
-  if (!grid_barrier(t.ctrl, gridDim.x)) return;
-
-  // Phase B: temporal blend, tiles from the second counter (as k_fused).
-  const bool blended = TEMPORAL && a.blend;
-  if (blended) {
-    unsigned long long n_hovf = 0;
-    for (;;) {
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        const unsigned long long bb = atomicAdd(&t.ctrl->blend_next, 1ull);
-        s_cur = bb < ntiles ? static_cast<uint32_t>(bb) : ntiles;
-      }
-      __syncthreads();
-      const uint32_t tile = s_cur;
-      if (tile >= ntiles) break;
-      blend_range<2, false>(t, tile * static_cast<uint32_t>(kFusedTile), __ldcg(t.bcount + tile),
-                            threadIdx.x, blockDim.x, a.alpha, n_hovf);
-    }
-    const unsigned long long hs = block_sum(n_hovf);
-    if (threadIdx.x == 0 && hs) atomicAdd(&t.ctrl->hist_overflow, hs);
-    if (!grid_barrier(t.ctrl, gridDim.x)) return;
-  }
-
-  // Phase C: one lookup per vertex of this CTA's tiles (cell ids from the stash).
-  const bool ovec = a.ovec != 0;
-  for (uint32_t k = 0; k < taken; ++k) {
-    const size_t t0 = static_cast<size_t>(s_tile[k]) * kFusedTile;
-    const size_t end = min(a.n, t0 + kFusedTile);
-#pragma unroll 1
-    for (int sub = 0; sub < 4; sub += 2) {
-      const size_t j = t0 + fused_offset<2>(sub);
-      if (j < end) {
-        uint32_t id[2];
-        if (j + 2 <= end) {  // j is even and the stash 8-byte aligned
-          const uint2 w2 = __ldcs(reinterpret_cast<const uint2*>(a.gstash + j));
-          id[0] = w2.x;
-          id[1] = w2.y;
-        } else {
-          id[0] = __ldcs(a.gstash + j);
-          id[1] = kOverflowSlot;
-        }
-        Result res[2];
-        resolve_batch<2>(t, a.v, j, end, id, blended, res);
-        store_batch<2>(a.o, j, end, ovec, res);
-      }
-    }
-  }
-  if (!grid_barrier(t.ctrl, gridDim.x)) return;
-
-  // Phase D: empty the cells this CTA's tiles created.
-  for (uint32_t k = 0; k < taken; ++k)
-    clear_range(t, s_tile[k] * static_cast<uint32_t>(kFusedTile), s_claims[k], threadIdx.x,
-                blockDim.x, a.sweep != 0);
-  if (a.sweep)
-    sweep_slots(t, blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x,
-                static_cast<size_t>(gridDim.x) * blockDim.x);
-}
-
-// The batched persistent kernel: the same phases as k_fused over the tiles of
-// several views, each with its own table.  Tiles are numbered across views
-// (view v owns tiles [tile_base, tile_base + ntiles)) and handed out from one
-// counter; a CTA copies the descriptor of the view of each tile it takes into
-// shared memory and remembers (view, tile) for the later phases.
+// The batched persistent kernel: the same phases over the tiles of several
+// views, each with its own table.  Tiles are numbered across views (view v
+// owns tiles [tile_base, tile_base + ntiles)); the insert and the blend give a
+// warp every nw-th tile, the other phases a contiguous run.  A warp keeps the
+// descriptor of the view it is working on in shared memory of its own.
 struct MultiArgs {
   const ViewDesc* views;
-  Ctrl* ctrl;  // grid barrier and tile counter of the batch
-  uint32_t* gstash;
-  uint32_t nviews, total_tiles, cap_tiles;
+  Ctrl* ctrl;  // grid barrier of the batch
+  uint32_t* stash;  // indexed by tile, tile_v words each
+  uint32_t nviews, total_tiles, tile_v;
   float alpha;
 };
 
-__device__ __forceinline__ void copy_view(ViewDesc* dst, const ViewDesc* src) {
+// The warp's copy of the descriptor of the view that tile gt belongs to;
+// `cur` is the view it holds.  All lanes.
+__device__ __forceinline__ void take_view(ViewDesc* mine, const MultiArgs& a, uint32_t gt,
+                                          uint32_t& cur) {
+  uint32_t v = cur == kOverflowSlot || gt < mine->tile_base ? 0u : cur;
+  while (v + 1 < a.nviews && __ldg(&a.views[v + 1].tile_base) <= gt) ++v;
+  if (v == cur) return;
+  __syncwarp();
   const int words = static_cast<int>(sizeof(ViewDesc) / sizeof(uint32_t));
-  for (int i = threadIdx.x; i < words; i += blockDim.x)
-    reinterpret_cast<uint32_t*>(dst)[i] = reinterpret_cast<const uint32_t*>(src)[i];
+  for (int i = threadIdx.x & 31; i < words; i += 32)
+    reinterpret_cast<uint32_t*>(mine)[i] = __ldg(reinterpret_cast<const uint32_t*>(a.views + v) + i);
+  cur = v;
+  __syncwarp();
 }
 
 template <bool TEMPORAL, int W, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, (W == 4 ? 1 : 2) * (kFusedBlock / BLOCK)) k_fused_multi(MultiArgs a) {
-  constexpr int kPer = kFusedTile / BLOCK;  // vertices per thread per tile
-  extern __shared__ __align__(16) uint32_t s_stash[];
-  __shared__ uint32_t s_tile[kMaxTilesPerCta];
-  __shared__ uint32_t s_claims[kMaxTilesPerCta];
-  __shared__ uint16_t s_view[kMaxTilesPerCta];
-  __shared__ __align__(16) ViewDesc s_vd;
-  __shared__ uint32_t s_next, s_taken;
-  __shared__ unsigned long long s_ovf, s_cells;
-  if (threadIdx.x == 0) s_taken = 0;
+  __shared__ __align__(16) ViewDesc s_vd[BLOCK / 32];
+  __shared__ WarpShared s_warp[BLOCK / 32];
+  WarpShared& sh = s_warp[threadIdx.x >> 5];
+  const uint32_t lane = threadIdx.x & 31u, tile_v = a.tile_v, tile_i = tile_ids(tile_v, W);
+  ViewDesc& vd = s_vd[threadIdx.x >> 5];
+  uint32_t cur = kOverflowSlot;  // the view in vd
+  // this warp's run of tiles in the later phases
+  const uint64_t gw = grid_warp(), nw = grid_warps();
+  const uint32_t run0 = static_cast<uint32_t>(gw * a.total_tiles / nw);
+  const uint32_t run1 = static_cast<uint32_t>((gw + 1) * a.total_tiles / nw);
 
-  // Phase A: keys, probing insert, accumulation, tile by tile across views.
-  for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t gt = a.total_tiles;
-      if (s_taken < a.cap_tiles) gt = static_cast<uint32_t>(atomicAdd(&a.ctrl->tile_next, 1ull));
-      s_next = gt;
-      if (gt < a.total_tiles) {
-        uint32_t v = 0;
-        while (v + 1 < a.nviews && a.views[v + 1].tile_base <= gt) ++v;
-        s_view[s_taken] = static_cast<uint16_t>(v);
-        s_tile[s_taken] = gt - a.views[v].tile_base;
-        s_claims[s_taken] = 0;
+  // empty the slot tables of the views that are swept
+  for (uint32_t v = 0; v < a.nviews; ++v) {
+    take_view(&vd, a, __ldg(&a.views[v].tile_base), cur);
+    if (cur == v && vd.sweep)
+      sweep_slots(vd.t, blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x,
+                  static_cast<size_t>(gridDim.x) * blockDim.x);
+  }
+  cur = kOverflowSlot;
+  if (!grid_barrier(a.ctrl, gridDim.x)) return;
+
+  {
+    WarpInsert<W> s;
+    uint32_t last = 0u;  // the last tile worked on
+    auto ids = [&]() { return a.stash + static_cast<size_t>(vd.tile_base) * tile_v; };
+    auto flush = [&]() {  // leave the view in vd
+      while (s.queued) queue_step<W>(vd.t, vd.v, s, sh, true, ids());
+      if (lane == 0) __stcg(vd.t.bcount + last, s.claims);
+      unsigned long long o = s.cnt.ovf, c = s.cnt.cells;
+      for (int off = 16; off > 0; off >>= 1) {
+        o += __shfl_xor_sync(0xFFFFFFFFu, o, off);
+        c += __shfl_xor_sync(0xFFFFFFFFu, c, off);
       }
-      s_ovf = 0;
-      s_cells = 0;
-    }
-    __syncthreads();
-    const uint32_t gt = s_next;
-    if (gt >= a.total_tiles) break;
-    const uint32_t k = s_taken;
-    copy_view(&s_vd, a.views + s_view[k]);
-    __syncthreads();
-    const size_t t0 = static_cast<size_t>(s_tile[k]) * kFusedTile;
-    const size_t end = min(static_cast<size_t>(s_vd.n), t0 + kFusedTile);
-    uint32_t* stash = a.gstash ? a.gstash + static_cast<size_t>(gt) * kFusedTile
-                               : s_stash + static_cast<size_t>(k) * kFusedTile;
-    Counters c;
+      if (lane == 0) {
+        if (o) atomicAdd(&vd.t.ctrl->overflow_vertices, o);
+        if (c) atomicAdd(&vd.t.ctrl->frame_cells, c);
+      }
+      s.cnt = Counters{};
+      s.retire(vd.t, true);  // reserved ids belong to the view
+    };
+    for (uint32_t gt = gw; gt < a.total_tiles; gt += nw) {
+      if (cur != kOverflowSlot && gt - vd.tile_base >= vd.ntiles) flush();
+      take_view(&vd, a, gt, cur);
+      last = gt - vd.tile_base;
+      const size_t t0 = static_cast<size_t>(last) * tile_v;
+      const size_t end = min(static_cast<size_t>(vd.n), t0 + tile_v);
+      s.claims = 0u;
+      s.id_base = last * tile_i;
 #pragma unroll 1
-    for (int sub = 0; sub < kPer; sub += W) {
-      const size_t j = t0 + fused_offset<W, BLOCK>(sub);
-      if (j < end) {
-        const Batch<W> b = insert_batch<W>(s_vd.kc, s_vd.t, s_vd.v, j, end, s_vd.vec != 0,
-                                           static_cast<uint32_t>(t0), &s_claims[k], c);
-#pragma unroll
-        for (int q = 0; q < W; ++q) stash[j - t0 + q] = b.id[q];
-      }
+      for (size_t j0 = t0; j0 < end; j0 += 32 * W)
+        insert_warp<W, false, false>(vd.kc, vd.t, vd.v, j0, end, s, sh, true, 2, ids());
+      if (lane == 0) __stcg(vd.t.bcount + last, s.claims);
     }
-    // per-view counters of this tile
-    unsigned long long o = c.ovf, cl = c.cells;
-    for (int off = 16; off > 0; off >>= 1) {
-      o += __shfl_xor_sync(0xFFFFFFFFu, o, off);
-      cl += __shfl_xor_sync(0xFFFFFFFFu, cl, off);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      if (o) atomicAdd(&s_ovf, o);
-      if (cl) atomicAdd(&s_cells, cl);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      if (s_ovf) atomicAdd(&s_vd.t.ctrl->overflow_vertices, s_ovf);
-      if (s_cells) atomicAdd(&s_vd.t.ctrl->frame_cells, s_cells);
-      atomicAdd(&s_vd.t.ctrl->vertices, static_cast<unsigned long long>(end - t0));
-      ++s_taken;
-    }
+    if (cur != kOverflowSlot) flush();
+    for (uint32_t v = blockIdx.x; v < a.nviews; v += gridDim.x)
+      if (threadIdx.x == 0)
+        atomicAdd(&a.views[v].t.ctrl->vertices, static_cast<unsigned long long>(a.views[v].n));
   }
   if (!grid_barrier(a.ctrl, gridDim.x)) return;
-  const uint32_t taken = s_taken;
 
-  // Phase B: temporal blend of the cells this CTA's tiles created.
+  for (uint32_t gt = run0; gt < run1; ++gt) {
+    take_view(&vd, a, gt, cur);
+    const size_t t0 = static_cast<size_t>(gt - vd.tile_base) * tile_v;
+    const size_t end = min(static_cast<size_t>(vd.n), t0 + tile_v);
+    for (size_t j = t0; j < end; j += 128)
+      add_warp(vd.t, vd.v, j, end, a.stash + static_cast<size_t>(vd.tile_base) * tile_v, 2, sh);
+  }
+  if (!grid_barrier(a.ctrl, gridDim.x)) return;
+
   if (TEMPORAL) {
-    for (uint32_t k = 0; k < taken; ++k) {
-      __syncthreads();
-      copy_view(&s_vd, a.views + s_view[k]);
-      __syncthreads();
-      if (!s_vd.blended) continue;
-      unsigned long long n_hovf = 0;
-      blend_range<W, false>(s_vd.t, s_tile[k] * static_cast<uint32_t>(kFusedTile), s_claims[k],
-                     threadIdx.x, blockDim.x, a.alpha, n_hovf);
-      if (n_hovf) atomicAdd(&s_vd.t.ctrl->hist_overflow, n_hovf);
+    // strided tiles: a view's costly (incoherent) tiles go to many warps
+    for (uint64_t gt = gw; gt < a.total_tiles;) {
+      take_view(&vd, a, static_cast<uint32_t>(gt), cur);
+      if (vd.blended) {
+        unsigned long long n_hovf = 0;
+        blend_tiles<false>(vd.t, static_cast<uint32_t>(gt - vd.tile_base), static_cast<uint32_t>(nw), vd.ntiles, tile_i,
+                           a.alpha, n_hovf);
+        if (n_hovf) atomicAdd(&vd.t.ctrl->hist_overflow, n_hovf);
+      }
+      gt += (vd.tile_base + static_cast<uint64_t>(vd.ntiles) - gt + nw - 1) / nw * nw;  // past this view
     }
     if (!grid_barrier(a.ctrl, gridDim.x)) return;
   }
 
-  // Phase C: one lookup per vertex of this CTA's tiles.
-  for (uint32_t k = 0; k < taken; ++k) {
-    __syncthreads();
-    copy_view(&s_vd, a.views + s_view[k]);
-    __syncthreads();
-    const size_t t0 = static_cast<size_t>(s_tile[k]) * kFusedTile;
-    const size_t end = min(static_cast<size_t>(s_vd.n), t0 + kFusedTile);
-    const size_t gt = static_cast<size_t>(s_vd.tile_base) + s_tile[k];
-    const uint32_t* stash = a.gstash ? a.gstash + gt * kFusedTile
-                                     : s_stash + static_cast<size_t>(k) * kFusedTile;
-    const bool blended = TEMPORAL && s_vd.blended;
-#pragma unroll 1
-    for (int sub = 0; sub < kPer; sub += W) {
-      const size_t j = t0 + fused_offset<W, BLOCK>(sub);
-      if (j < end) {
-        uint32_t id[W];
-#pragma unroll
-        for (int q = 0; q < W; ++q) id[q] = stash[j - t0 + q];
-        Result res[W];
-        resolve_batch<W>(s_vd.t, s_vd.v, j, end, id, blended, res);
-        store_batch<W>(s_vd.o, j, end, s_vd.ovec != 0, res);
-      }
-    }
+  for (uint32_t gt = run0; gt < run1; ++gt) {
+    take_view(&vd, a, gt, cur);
+    const size_t t0 = static_cast<size_t>(gt - vd.tile_base) * tile_v;
+    const size_t end = min(static_cast<size_t>(vd.n), t0 + tile_v);
+    uint32_t low = 0u;
+    for (size_t j = t0; j < end; j += 128)
+      lookup_warp<false>(vd.t, vd.v, vd.o, j, end, a.stash + static_cast<size_t>(vd.tile_base) * tile_v,
+                         TEMPORAL && vd.blended, nullptr, sh, low);
   }
-  if (!grid_barrier(a.ctrl, gridDim.x)) return;
-
-  // Phase D: empty the cells this CTA's tiles created; sweep the slot tables
-  // of the views that are swept.
-  for (uint32_t k = 0; k < taken; ++k) {
-    __syncthreads();
-    copy_view(&s_vd, a.views + s_view[k]);
-    __syncthreads();
-    clear_range(s_vd.t, s_tile[k] * static_cast<uint32_t>(kFusedTile), s_claims[k], threadIdx.x,
-                blockDim.x, s_vd.sweep != 0);
-  }
-  for (uint32_t v = 0; v < a.nviews; ++v) {
-    __syncthreads();
-    copy_view(&s_vd, a.views + v);
-    __syncthreads();
-    if (s_vd.sweep)
-      sweep_slots(s_vd.t, blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x,
-                  static_cast<size_t>(gridDim.x) * blockDim.x);
+  for (uint32_t gt = run0; gt < run1; ++gt) {
+    take_view(&vd, a, gt, cur);
+    const uint32_t tile = gt - vd.tile_base;
+    if (!vd.sweep) clear_range(vd.t, tile * tile_i, __ldcg(vd.t.bcount + tile), lane, 32);
   }
 }
+
+int split_grid(size_t work_items) {
+  const size_t want = (work_items + kBlock - 1) / kBlock;
+  const size_t cap = static_cast<size_t>(sm_count()) * 8;
+  return static_cast<int>(std::max<size_t>(1, std::min(want, cap)));
+}
+
+}  // namespace
 
 int sm_count() {
   static int cached = 0;
@@ -1754,16 +1344,20 @@ int sm_count() {
   return cached;
 }
 
-int split_grid(size_t work_items) {
-  const size_t want = (work_items + kBlock - 1) / kBlock;
-  const size_t cap = static_cast<size_t>(sm_count()) * 8;
-  return static_cast<int>(std::max<size_t>(1, std::min(want, cap)));
+int tile_size() { return kTile; }
+int split_tile_ids() { return kTileIds; }
+size_t fused_cells(size_t n, uint32_t tile, int batch) {
+  return (n + tile - 1) / tile * tile_ids(tile, batch);
 }
 
-}  // namespace
-
-int tile_size() { return kTile; }
-int fused_tile_size() { return kFusedTile; }
+// Vertices per warp tile of the persistent kernels: 256, or fewer so that a
+// small frame still gives every warp of the GPU work.
+uint32_t fused_tile(size_t n, int batch) {
+  const size_t warps = static_cast<size_t>(sm_count()) * 32;
+  uint32_t v = kFusedTile;
+  while (v > 32u * batch && n < 2 * warps * v) v /= 2;
+  return v;
+}
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -1779,20 +1373,21 @@ static bool vec_outputs(const OutPtrs& o) {
 }
 
 cudaError_t launch_insert(const KeyConst& kc, const TableDev& t, const VertexPtrs& v, size_t n,
-                          uint32_t* id_out, uint32_t tile_base, int batch, cudaStream_t st) {
+                          uint32_t* stash, uint32_t* id_out, uint32_t tile_base, int batch, int merge,
+                          cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  const int grid = split_grid((n + 3) / 4);
-  const int vec = vec_inputs(v) ? 1 : 0;
+  const int grid = split_grid((n + kTile - 1) / kTile * 32);
   if (t.hist_migrate || t.normal_search) {  // keep each new cell's quantized key
     if (batch == 2)
-      k_insert<2, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, id_out, vec, tile_base);
+      k_insert<2, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, merge);
     else
-      k_insert<4, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, id_out, vec, tile_base);
+      k_insert<4, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, merge);
   } else if (batch == 2) {
-    k_insert<2, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, id_out, vec, tile_base);
+    k_insert<2, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, merge);
   } else {
-    k_insert<4, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, id_out, vec, tile_base);
+    k_insert<4, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, merge);
   }
+  k_add<<<split_grid((n + 127) / 128 * 32), kBlock, 0, st>>>(t, v, n, stash, id_out, merge);
   return cudaGetLastError();
 }
 
@@ -1817,7 +1412,7 @@ cudaError_t launch_keys(const KeyConst& kc, const VertexPtrs& v, size_t n, uint3
 cudaError_t launch_blend(const KeyConst& kc, const TableDev& t, uint32_t ntiles, float alpha,
                          cudaStream_t st) {
   if (ntiles == 0) return cudaSuccess;
-  const uint32_t grid = std::min<uint32_t>(ntiles, static_cast<uint32_t>(sm_count()) * 8);
+  const int grid = split_grid(static_cast<size_t>(ntiles) * 32);
   if (t.hist_migrate) {
     k_blend_lookup<<<grid, kBlock, 0, st>>>(kc, t, ntiles);
     k_blend_apply<<<grid, kBlock, 0, st>>>(t, ntiles, alpha);
@@ -1835,9 +1430,8 @@ static bool sweep_pays(const TableDev& t, size_t vertices) {
 cudaError_t launch_clear(const TableDev& t, uint32_t ntiles, cudaStream_t st) {
   if (ntiles == 0) return cudaSuccess;
   const int sweep = sweep_pays(t, static_cast<size_t>(ntiles) * kTile) ? 1 : 0;
-  const uint32_t grid = std::min<uint32_t>(std::max<uint32_t>(ntiles, sweep ? 1u << 30 : 0u),
-                                           static_cast<uint32_t>(sm_count()) * 8);
-  k_clear_sweep<<<grid, kBlock, 0, st>>>(t, ntiles, sweep);
+  const int grid = split_grid(sweep ? ~size_t{0} / 2 : static_cast<size_t>(ntiles) * 32);
+  k_clear_sweep<<<grid, kBlock, 0, st>>>(t, ntiles, kTileIds, sweep);
   return cudaGetLastError();
 }
 
@@ -1890,179 +1484,94 @@ cudaError_t launch_count_nonzero(const void* base, uint32_t stride, uint32_t off
 }
 
 template <bool TEMPORAL, bool EVICT, bool NEIGH>
-static const void* fused_fn(int batch) {
+static const void* fused_fn(int batch, bool kv) {
+  if (kv)
+    return batch == 2 ? reinterpret_cast<const void*>(k_fused<TEMPORAL, 2, EVICT, NEIGH, true>)
+                      : reinterpret_cast<const void*>(k_fused<TEMPORAL, 4, EVICT, NEIGH, true>);
   return batch == 2 ? reinterpret_cast<const void*>(k_fused<TEMPORAL, 2, EVICT, NEIGH>)
                     : reinterpret_cast<const void*>(k_fused<TEMPORAL, 4, EVICT, NEIGH>);
 }
 
 // The kernel for a frame: with or without a history, an evicting one or not,
-// with or without the neighborhood search.
-static const void* fused_kernel(bool temporal, int batch, bool evict, bool neigh) {
-  if (temporal && evict)
-    return neigh ? fused_fn<true, true, true>(batch) : fused_fn<true, true, false>(batch);
-  if (temporal) return neigh ? fused_fn<true, false, true>(batch) : fused_fn<true, false, false>(batch);
-  return neigh ? fused_fn<false, false, true>(batch) : fused_fn<false, false, false>(batch);
+// with or without the neighborhood search, with or without key variants.
+static const void* fused_kernel(const FusedPlan& p) {
+  if (p.temporal && p.evict)
+    return p.neigh ? fused_fn<true, true, true>(p.batch, p.kv) : fused_fn<true, true, false>(p.batch, p.kv);
+  if (p.temporal)
+    return p.neigh ? fused_fn<true, false, true>(p.batch, p.kv) : fused_fn<true, false, false>(p.batch, p.kv);
+  return p.neigh ? fused_fn<false, false, true>(p.batch, p.kv) : fused_fn<false, false, false>(p.batch, p.kv);
 }
 
-// Largest dynamic shared memory a k_fused CTA may request: the opt-in limit
-// per block minus the kernel's static shared memory (set once per kernel).
-static cudaError_t fused_dyn_smem_limit(const void* fn, size_t* limit) {
-  static const void* done[32] = {nullptr};
-  static size_t lims[32] = {0};
-  for (int i = 0; i < 32; ++i)
-    if (done[i] == fn) {
-      *limit = lims[i];
+// CTAs of `fn` that are resident at once on one multiprocessor (asked once per
+// kernel).
+static cudaError_t resident_ctas(const void* fn, int block, int* out) {
+  static std::mutex mu;
+  static std::vector<std::pair<const void*, int>> known;
+  std::lock_guard<std::mutex> lock(mu);
+  for (const auto& k : known)
+    if (k.first == fn) {
+      *out = k.second;
       return cudaSuccess;
     }
-  int dev = 0, maxopt = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&maxopt, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  cudaFuncAttributes fa;
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
-  if (e != cudaSuccess) return e;
-  const size_t lim = static_cast<size_t>(maxopt) - fa.sharedSizeBytes;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(lim));
-  if (e != cudaSuccess) return e;
-  for (int i = 0; i < 32; ++i)
-    if (!done[i]) {
-      done[i] = fn;
-      lims[i] = lim;
-      break;
-    }
-  *limit = lim;
-  return cudaSuccess;
-}
-
-template <bool TEMPORAL>
-static const void* ws_fn(int key_warps) {
-  if (key_warps == 4) return reinterpret_cast<const void*>(k_fused_ws<TEMPORAL, 4, 12, 2>);
-  if (key_warps == 12) return reinterpret_cast<const void*>(k_fused_ws<TEMPORAL, 12, 4, 2>);
-  return reinterpret_cast<const void*>(k_fused_ws<TEMPORAL, 8, 8, 2>);
-}
-
-static const void* ws_kernel(bool temporal, int key_warps) {
-  return temporal ? ws_fn<true>(key_warps) : ws_fn<false>(key_warps);
-}
-
-// The pipelined insert: two CTAs of 512 threads per SM when their queues fit
-// (one otherwise); the stash is the global one.
-static cudaError_t plan_ws(size_t n, bool temporal, int key_warps, bool fixed, FusedPlan* plan) {
-  const void* fn = ws_kernel(temporal, key_warps);
-  size_t maxdyn = 0;
-  cudaError_t e = fused_dyn_smem_limit(fn, &maxdyn);
-  if (e != cudaSuccess) return e;
-  const size_t smem = WsLayout::bytes(fixed);
-  if (smem > maxdyn) return cudaErrorInvalidConfiguration;
   int nb = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kFusedBlock, smem);
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, block, 0);
   if (e != cudaSuccess) return e;
   if (nb < 1) return cudaErrorInvalidConfiguration;
-  plan->grid = sm_count() * std::min(nb, 2);
-  plan->block = kFusedBlock;
-  plan->batch = 2;
-  plan->cap_tiles = kMaxTilesPerCta;
-  plan->smem = smem;
-  plan->global_stash = true;
-  plan->evict = false;
-  plan->neigh = false;
-  plan->key_warps = key_warps;
-  const size_t ntiles = (n + kFusedTile - 1) / kFusedTile;
-  if (static_cast<size_t>(plan->grid) * kMaxTilesPerCta < ntiles) return cudaErrorInvalidValue;
+  known.emplace_back(fn, nb);
+  *out = nb;
   return cudaSuccess;
 }
 
-cudaError_t plan_fused(size_t n, bool temporal, int batch, FusedPlan* plan, bool evict,
-                       bool neigh, InsertShape shape, bool fixed) {
-  plan->key_warps = 0;
-  if (shape.pipelined && !evict && !neigh) {
-    const int kw = shape.key_warps == 4 || shape.key_warps == 12 ? shape.key_warps : 8;
-    plan->merge = shape.merge;
-    return plan_ws(n, temporal, kw, fixed, plan);
-  }
-  const void* fn = fused_kernel(temporal, batch, evict, neigh);
-  plan->evict = temporal && evict;
-  plan->neigh = neigh;
-  const int sms = sm_count();
-  size_t maxdyn = 0;
-  cudaError_t e = fused_dyn_smem_limit(fn, &maxdyn);
-  if (e != cudaSuccess) return e;
-  int b0 = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b0, fn, kFusedBlock, 0);
-  if (e != cudaSuccess) return e;
-  if (b0 < 1) return cudaErrorInvalidConfiguration;
-  int dev = 0, smem_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-  const size_t ntiles = (n + kFusedTile - 1) / kFusedTile;
-  const size_t tile_bytes = kFusedTile * sizeof(uint32_t);
+// CTAs of a persistent launch over `ntiles` warp tiles: all that are resident
+// at once, or one per four tiles for a small frame (a tile per scheduler), so
+// that its grid barriers wait for no idle CTAs.
+static int fused_grid(const void* fn, int block, size_t ntiles, cudaError_t* err) {
+  int nb = 0;
+  *err = resident_ctas(fn, block, &nb);
+  if (*err != cudaSuccess) return 0;
+  const size_t most = static_cast<size_t>(sm_count()) * std::min(nb, 1024 / block);
+  return static_cast<int>(std::max<size_t>(1, std::min(most, (ntiles + 3) / 4)));
+}
+
+cudaError_t plan_fused(size_t n, size_t max_cells, FusedPlan* plan) {
+  cudaError_t e = cudaSuccess;
+  plan->evict = plan->evict && plan->temporal;
   plan->block = kFusedBlock;
-  plan->batch = batch;
-  for (int b = b0; b >= 1; --b) {
-    // shared memory per CTA when b CTAs share an SM (static part and a reserve deducted)
-    const size_t per = std::min(maxdyn, static_cast<size_t>(smem_sm) / b - 12 * 1024);
-    size_t cap = std::min<size_t>(per / tile_bytes, kMaxTilesPerCta);
-    // the largest stash with which b CTAs still fit on an SM
-    int nb = 0;
-    for (; cap > 0; --cap) {
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kFusedBlock, cap * tile_bytes);
-      if (e != cudaSuccess) return e;
-      if (nb >= b) break;
-    }
-    if (cap == 0 || cap * static_cast<size_t>(sms) * b < ntiles) continue;
-    if (nb >= b) {
-      plan->grid = sms * b;
-      plan->cap_tiles = static_cast<uint32_t>(cap);
-      plan->smem = cap * tile_bytes;
-      plan->global_stash = false;
-      return cudaSuccess;
-    }
-  }
-  // The stash does not fit on chip: keep it in a global scratch buffer.
-  plan->grid = sms * b0;
-  plan->cap_tiles = kMaxTilesPerCta;
-  plan->smem = 0;
-  plan->global_stash = true;
-  if (static_cast<size_t>(plan->grid) * kMaxTilesPerCta < ntiles) return cudaErrorInvalidValue;
-  return cudaSuccess;
+  plan->tile = fused_tile(n, plan->batch);
+  while (plan->tile < kFusedTile && fused_cells(n, plan->tile, plan->batch) > max_cells) plan->tile *= 2;
+  const size_t ntiles = (n + plan->tile - 1) / plan->tile;
+  plan->grid = fused_grid(fused_kernel(*plan), kFusedBlock, ntiles, &e);
+  return e;
 }
 
 cudaError_t launch_fused(const KeyConst& kc, const TableDev& t, const VertexPtrs& v, size_t n,
-                         const OutPtrs& o, bool temporal, bool blend, float alpha,
-                         const FusedPlan& plan, uint32_t* gstash, uint32_t* nq, cudaStream_t st) {
+                         const OutPtrs& o, bool blend, float alpha, const FusedPlan& plan, uint32_t* stash, uint32_t* nq, cudaStream_t st) {
   FusedArgs a;
   a.kc = kc;
   a.t = t;
   a.v = v;
   a.o = o;
   a.n = n;
-  a.cap_tiles = plan.cap_tiles;
-  a.gstash = plan.global_stash ? gstash : nullptr;
+  a.tile_v = plan.tile;
+  a.stash = stash;
   a.alpha = alpha;
-  a.vec = vec_inputs(v) ? 1 : 0;
-  a.ovec = vec_outputs(o) ? 1 : 0;
   a.blend = blend ? 1 : 0;
-  a.sweep = sweep_pays(t, n) ? 1 : 0;
+  a.sweep = plan.sweep ? 1 : 0;
   a.nq = nq;
   a.merge = plan.merge;
   void* args[] = {&a};
-  if (plan.key_warps > 0)
-    return cudaLaunchCooperativeKernel(ws_kernel(temporal, plan.key_warps), dim3(plan.grid),
-                                       dim3(plan.block), args, plan.smem, st);
-  cudaError_t e = cudaLaunchCooperativeKernel(
-      fused_kernel(temporal, plan.batch, plan.evict, plan.neigh), dim3(plan.grid), dim3(plan.block),
-      args, plan.smem, st);
+  cudaError_t e = cudaLaunchCooperativeKernel(fused_kernel(plan), dim3(plan.grid), dim3(plan.block), args,
+                                              0, st);
   if (e != cudaSuccess || !plan.neigh) return e;
-  // the queued neighborhood searches, then the clear the persistent kernel left
-  const int sms = sm_count();
-  k_neighbors<<<sms * 8, kBlock, 0, st>>>(kc, t, v, o, nq, blend ? 1 : 0);
-  const uint32_t ntiles = static_cast<uint32_t>((n + kFusedTile - 1) / kFusedTile);
-  k_clear_fused<<<std::min<uint32_t>(ntiles, static_cast<uint32_t>(sms) * 8), kBlock, 0, st>>>(
-      t, ntiles, a.sweep);
+  k_neighbors<<<sm_count() * 8, kBlock, 0, st>>>(kc, t, v, o, nq, blend ? 1 : 0);
+  if (!plan.sweep) {
+    const uint32_t ntiles = static_cast<uint32_t>((n + plan.tile - 1) / plan.tile);
+    k_clear_sweep<<<split_grid(static_cast<size_t>(ntiles) * 32), kBlock, 0, st>>>(
+        t, ntiles, tile_ids(plan.tile, plan.batch), 0);
+  }
   return cudaGetLastError();
 }
 
-bool vec_inputs_host(const VertexPtrs& v) { return vec_inputs(v); }
-bool vec_outputs_host(const OutPtrs& o) { return vec_outputs(o); }
 bool sweep_pays_host(const TableDev& t, size_t vertices) { return sweep_pays(t, vertices); }
 
 template <bool TEMPORAL, int W>
@@ -2076,60 +1585,30 @@ static const void* multi_kernel(bool temporal, int batch, int block) {
   return batch == 2 ? multi_fn<false, 2>(block) : multi_fn<false, 4>(block);
 }
 
-cudaError_t plan_multi(size_t total_tiles, bool temporal, int batch, int block, MultiPlan* plan) {
-  block = block == 256 ? 256 : kFusedBlock;
-  const void* fn = multi_kernel(temporal, batch, block);
-  const int sms = sm_count();
-  size_t maxdyn = 0;
-  cudaError_t e = fused_dyn_smem_limit(fn, &maxdyn);
-  if (e != cudaSuccess) return e;
-  int b0 = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b0, fn, block, 0);
-  if (e != cudaSuccess) return e;
-  if (b0 < 1) return cudaErrorInvalidConfiguration;
-  int dev = 0, smem_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-  const size_t tile_bytes = kFusedTile * sizeof(uint32_t);
-  plan->block = block;
+cudaError_t plan_multi(size_t total_tiles, uint32_t tile, bool temporal, int batch, int block,
+                       MultiPlan* plan) {
+  cudaError_t e = cudaSuccess;
+  plan->block = block == 256 ? 256 : kFusedBlock;
   plan->batch = batch;
-  for (int b = b0; b >= 1; --b) {
-    const size_t per = std::min(maxdyn, static_cast<size_t>(smem_sm) / b - 12 * 1024);
-    const size_t cap = std::min<size_t>(per / tile_bytes, kMaxTilesPerCta);
-    if (cap == 0 || cap * static_cast<size_t>(sms) * b < total_tiles) continue;
-    int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, block, cap * tile_bytes);
-    if (e != cudaSuccess) return e;
-    if (nb >= b) {
-      plan->grid = sms * b;
-      plan->cap_tiles = static_cast<uint32_t>(cap);
-      plan->smem = cap * tile_bytes;
-      plan->global_stash = false;
-      return cudaSuccess;
-    }
-  }
-  plan->grid = sms * b0;
-  plan->cap_tiles = kMaxTilesPerCta;
-  plan->smem = 0;
-  plan->global_stash = true;
-  if (static_cast<size_t>(plan->grid) * kMaxTilesPerCta < total_tiles) return cudaErrorInvalidValue;
-  return cudaSuccess;
+  plan->tile = tile;
+  plan->grid = fused_grid(multi_kernel(temporal, batch, plan->block), plan->block, total_tiles, &e);
+  return e;
 }
 
 cudaError_t launch_multi(const ViewDesc* views, uint32_t nviews, uint32_t total_tiles, Ctrl* ctrl,
-                         bool temporal, float alpha, const MultiPlan& plan, uint32_t* gstash,
+                         bool temporal, float alpha, const MultiPlan& plan, uint32_t* stash,
                          cudaStream_t st) {
   MultiArgs a;
   a.views = views;
   a.ctrl = ctrl;
-  a.gstash = plan.global_stash ? gstash : nullptr;
+  a.stash = stash;
   a.nviews = nviews;
   a.total_tiles = total_tiles;
-  a.cap_tiles = plan.cap_tiles;
+  a.tile_v = plan.tile;
   a.alpha = alpha;
   void* args[] = {&a};
   return cudaLaunchCooperativeKernel(multi_kernel(temporal, plan.batch, plan.block), dim3(plan.grid),
-                                     dim3(plan.block), args, plan.smem, st);
+                                     dim3(plan.block), args, 0, st);
 }
 
 }  // namespace pps

@@ -44,15 +44,20 @@ constexpr uint32_t kNoAllocMaxLog2Slots = 20;                // up to 2^20 slots
 constexpr size_t kNoAllocMaxVertices = size_t{1} << 19;      // up to 524,288 vertices
 
 constexpr size_t kSlotBytes = (size_t{1} << kNoAllocMaxLog2Slots) * sizeof(unsigned long long);
-constexpr size_t kAccBytes = kNoAllocMaxVertices * sizeof(float4);
-constexpr size_t kInfoBytes = kNoAllocMaxVertices * sizeof(uint4);
+// Cells the id ranges of the warp tiles may span (pps::fused_cells): 64
+// vertices per tile up to 131,072 vertices, 128 up to 262,144, 256 beyond.
+constexpr size_t kNoAllocMaxCells = (size_t{1} << 19) / 256 * (256 + 96);
+constexpr size_t kAccBytes = kNoAllocMaxCells * sizeof(float4);
+constexpr size_t kInfoBytes = kNoAllocMaxCells * sizeof(uint4);
 constexpr size_t kStashBytes = kNoAllocMaxVertices * sizeof(uint32_t);
+constexpr size_t kCountBytes = kNoAllocMaxVertices / 64 * sizeof(uint32_t);  // cells per warp tile
 constexpr size_t kCtrlBytes = 256;
 constexpr size_t kOffAcc = kSlotBytes;
 constexpr size_t kOffInfo = kOffAcc + kAccBytes;
 constexpr size_t kOffStash = kOffInfo + kInfoBytes;
-constexpr size_t kOffCtrl = kOffStash + kStashBytes;
-constexpr size_t kScratchBytes = kOffCtrl + kCtrlBytes;  // 26 MB + 256 B
+constexpr size_t kOffCount = kOffStash + kStashBytes;
+constexpr size_t kOffCtrl = kOffCount + kCountBytes;
+constexpr size_t kScratchBytes = kOffCtrl + kCtrlBytes;  // about 33 MB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -159,13 +164,17 @@ extern "C" int pps_filter_noalloc(const pps_params* p, const pps_camera* cam, ui
   if (int rc = scratch_address("pps_filter_noalloc", &base)) return rc;
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   const uint32_t T = 1u << p->log2_slots;
-  const size_t tile = static_cast<size_t>(pps::fused_tile_size());
-  const size_t ids = (n + tile - 1) / tile * tile;
+  pps::FusedPlan plan;
+  plan.sweep = true;
+  cudaError_t e = pps::plan_fused(n, kNoAllocMaxCells, &plan);
+  if (e != cudaSuccess)
+    return noalloc_fail(PPS_ECUDA, std::string("pps_filter_noalloc: ") + cudaGetErrorString(e));
 
   pps::TableDev t{};
   t.slots = reinterpret_cast<unsigned long long*>(base);
   t.acc = reinterpret_cast<float4*>(base + kOffAcc);
   t.info = reinterpret_cast<uint4*>(base + kOffInfo);
+  t.bcount = reinterpret_cast<uint32_t*>(base + kOffCount);
   t.ctrl = reinterpret_cast<pps::Ctrl*>(base + kOffCtrl);
   t.mask = T - 1;
   t.hmask = 0;
@@ -191,10 +200,9 @@ extern "C" int pps_filter_noalloc(const pps_params* p, const pps_camera* cam, ui
   kc.jitter = p->jitter;
   kc.nih = p->normal_in_home_hash;
 
-  // The array keeps whatever the last call left: clear what must start empty.
-  cudaError_t e = cudaMemsetAsync(t.slots, 0, static_cast<size_t>(T) * sizeof(unsigned long long), st);
-  if (e == cudaSuccess && ids) e = cudaMemsetAsync(t.acc, 0, ids * sizeof(float4), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(t.ctrl, 0, kCtrlBytes, st);
+  // The array keeps whatever the last call left: the launch empties the slots
+  // itself, and the counters must start at zero.
+  e = cudaMemsetAsync(t.ctrl, 0, kCtrlBytes, st);
   if (e != cudaSuccess)
     return noalloc_fail(PPS_ECUDA, std::string("pps_filter_noalloc: ") + cudaGetErrorString(e));
   if (n == 0) return PPS_OK;
@@ -221,11 +229,8 @@ extern "C" int pps_filter_noalloc(const pps_params* p, const pps_camera* cam, ui
   dout.count = out->count;
   dout.status = out->status;
 
-  pps::FusedPlan plan;
-  e = pps::plan_fused(n, false, 2, &plan);
-  if (e == cudaSuccess)
-    e = pps::launch_fused(kc, t, dv, n, dout, false, false, 0.0f, plan,
-                          reinterpret_cast<uint32_t*>(base + kOffStash), nullptr, st);
+  e = pps::launch_fused(kc, t, dv, n, dout, false, 0.0f, plan,
+                      reinterpret_cast<uint32_t*>(base + kOffStash), nullptr, st);
   if (e != cudaSuccess)
     return noalloc_fail(PPS_ECUDA, std::string("pps_filter_noalloc: ") + cudaGetErrorString(e));
   return PPS_OK;
