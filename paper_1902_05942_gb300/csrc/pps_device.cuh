@@ -868,18 +868,20 @@ __device__ __forceinline__ bool grid_barrier(Ctrl* c, unsigned int nblocks,
       __threadfence();
       atomicAdd(&c->bar_gen, 1u);
     } else {
-      const unsigned long long t0 = globaltimer_ns();
-      while (ld_acquire_u32(&c->bar_gen) == gen) {
+      unsigned long long t0 = 0ull;
+      for (uint32_t i = 1; ld_acquire_u32(&c->bar_gen) == gen; ++i) {
+        if (i % 32u) continue;  // the error word and the clock now and then only
+        const unsigned long long now = globaltimer_ns();
+        if (t0 == 0ull) t0 = now;
         if (ld_acquire_u32(&c->error) & kErrBarrierTimeout) {
           ok = 0;
           break;
         }
-        if (globaltimer_ns() - t0 > limit_ns) {
+        if (now - t0 > limit_ns) {
           atomicOr(&c->error, kErrBarrierTimeout);
           ok = 0;
           break;
         }
-        __nanosleep(32);
       }
     }
     __threadfence();

@@ -8,7 +8,7 @@
 // accumulation, on the fifth-generation tensor cores: tcgen05.mma from
 // shared-memory tiles in the canonical no-swizzle layout into tensor memory,
 // tcgen05.ld back to registers for the bias / ReLU / rounding epilogues.
-// Inference: a CTA of 128 threads evaluates 128 vertices per tile.
+// Inference: each group of 128 threads evaluates tiles of 128 vertices.
 // Training: one cooperative launch per call takes all its Adam steps.  A CTA
 // of 384 threads takes 128 samples at a time through the forward pass, the
 // delta chain and the weight and bias gradients dZ^T X and dZ^T 1 (products
@@ -165,18 +165,31 @@ __global__ void __launch_bounds__(256) k_mlp_compact(size_t n, const uint8_t* st
     if (f[q]) list[pos++] = static_cast<int32_t>(j0 + q);
 }
 
-// One CTA of 128 threads takes tiles of 128 listed vertices (the MMA's M).
-// Each thread encodes its vertex into a shared-memory tile in the canonical
-// K-major layout without swizzle (core matrices of 8 rows x 16 bytes: byte of
-// (r, k) = (r / 8 * K / 8 + k / 8) * 128 + r % 8 * 16 + k % 8 * 2); one thread
-// issues tcgen05.mma for each layer (A = activations, B = W as [out][in], both
-// K-major, BF16; D = FP32 in tensor memory, 64 columns) and commits it to an
-// mbarrier; the four warps read their 32 rows back with tcgen05.ld, add the
-// bias, apply ReLU, round to BF16 and store the next layer's A tile.  The
+// A CTA is four groups of 128 threads, each with its own stream of tiles of 128
+// listed vertices (the MMA's M), activation tile, mbarrier and 64
+// tensor-memory columns; the groups share one copy of the weights.  Each thread
+// encodes its vertex into a shared-memory tile in the canonical K-major layout
+// without swizzle (core matrices of 8 rows x 16 bytes: byte of (r, k) =
+// (r / 8 * K / 8 + k / 8) * 128 + r % 8 * 16 + k % 8 * 2); one thread issues
+// tcgen05.mma for each layer (A = activations, B = W as [out][in], both
+// K-major, BF16; D = FP32 in tensor memory, 64 columns) and commits it to the
+// mbarrier; the group's four warps read their 32 rows back with tcgen05.ld, add
+// the bias, apply ReLU, round to BF16 and store the next layer's A tile.  The
 // output layer is N = 16 (rows 3..15 of W4 are zero).
+//
+// Bound by the latency of a tile's chain (encode, then four times MMA, wait and
+// epilogue): a tile took 6.3 us, of which its instructions were 2.2 us, with
+// four CTAs of one group per multiprocessor.  Sharing the weights makes room
+// for eight groups (32 warps at 64 registers, the epilogues in halves of 32
+// columns), and a layer has one barrier instead of two.HD frame,
+// 1.84 M listed vertices: 149 us with four single-group CTAs, 140 like this;
+// what bounds it now is shared memory (69 % of its cycles: the products'
+// operands 35 %, the activations' stores 21 %) and issue (53 %).
 namespace tc {
 constexpr int kRows = 128;
-constexpr uint32_t kTmemCols = 64;
+constexpr int kGroups = 4;
+constexpr int kThreads = 128 * kGroups;
+constexpr uint32_t kTmemCols = 64 * kGroups;
 
 __device__ __forceinline__ uint32_t cm(int r, int k, int K) {
   return static_cast<uint32_t>(((r >> 3) * (K >> 3) + (k >> 3)) * 128 + (r & 7) * 16 + (k & 7) * 2);
@@ -185,13 +198,13 @@ __device__ __forceinline__ uint32_t cm(int r, int k, int K) {
 // The activation tile holds the encoded input (K = 80) and, once layer 1's
 // product is complete, each hidden layer's output (K = 64) in turn.
 struct Smem {
-  alignas(128) unsigned char act[kRows * 80 * 2];
+  alignas(128) unsigned char act[kGroups][kRows * 80 * 2];
   alignas(128) unsigned char w1[64 * 80 * 2];
   alignas(128) unsigned char w2[64 * 64 * 2];
   alignas(128) unsigned char w3[64 * 64 * 2];
   alignas(128) unsigned char w4[16 * 64 * 2];
-  float bias[3 * 64 + 16];
-  alignas(8) unsigned long long mbar;
+  alignas(16) float bias[3 * 64 + 16];
+  alignas(8) unsigned long long mbar[kGroups];
   uint32_t tmem;
 };
 constexpr size_t kSmemBytes = sizeof(Smem) + 128;  // + alignment of the dynamic base
@@ -219,6 +232,17 @@ __device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uin
       : "memory");
 }
 
+// KS MMAs of K = 16, operand descriptors `a` and `b` for the first and `sa`,
+// `sb` (16-byte units) between them.  One thread issues them, and its
+// instruction stream sets their pace: 49 cycles each unrolled like this (N = 16
+// and 64; 65 for N = 128), 114 with the descriptors made in a loop.
+template <int KS>
+__device__ __forceinline__ void mma_steps(uint32_t d, uint64_t a, uint32_t sa, uint64_t b, uint32_t sb,
+                                          uint32_t id) {
+#pragma unroll
+  for (int k = 0; k < KS; ++k) mma_bf16(d, a + sa * k, b + sb * k, id, k > 0 ? 1u : 0u);
+}
+
 __device__ __forceinline__ void commit(uint32_t mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
                : "memory");
@@ -239,23 +263,30 @@ __device__ __forceinline__ void fence_smem_async() {
 // seconds unless given).
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity,
                                           unsigned long long limit_ns = 2000000000ull) {
-  const unsigned long long t0 = globaltimer_ns();
+  unsigned long long t0 = 0ull;
   for (;;) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(mbar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (globaltimer_ns() - t0 > limit_ns) return false;
+    // the clock is read only between groups of tries
+    for (int i = 0; i < 16; ++i) {
+      uint32_t done;
+      asm volatile(
+          "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+          " selp.u32 %0, 1, 0, p;\n}"
+          : "=r"(done)
+          : "r"(mbar), "r"(parity)
+          : "memory");
+      if (done) return true;
+    }
+    const unsigned long long t = globaltimer_ns();
+    if (t0 == 0ull)
+      t0 = t;
+    else if (t - t0 > limit_ns)
+      return false;
   }
 }
 
-__device__ __forceinline__ void tmem_ld_x64(uint32_t taddr, uint32_t (&v)[64]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31]), "=r"(v[32]), "=r"(v[33]), "=r"(v[34]), "=r"(v[35]), "=r"(v[36]), "=r"(v[37]), "=r"(v[38]), "=r"(v[39]), "=r"(v[40]), "=r"(v[41]), "=r"(v[42]), "=r"(v[43]), "=r"(v[44]), "=r"(v[45]), "=r"(v[46]), "=r"(v[47]), "=r"(v[48]), "=r"(v[49]), "=r"(v[50]), "=r"(v[51]), "=r"(v[52]), "=r"(v[53]), "=r"(v[54]), "=r"(v[55]), "=r"(v[56]), "=r"(v[57]), "=r"(v[58]), "=r"(v[59]), "=r"(v[60]), "=r"(v[61]), "=r"(v[62]), "=r"(v[63])
+__device__ __forceinline__ void tmem_ld_x32(uint32_t taddr, uint32_t (&v)[32]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
                : "r"(taddr));
 }
 
@@ -302,36 +333,54 @@ __device__ __forceinline__ void encode_row(unsigned char* x, int r, const Vertex
   encode_blocks<0, 9, true>(x, r, vi, valid);
 }
 
-// bias + ReLU + BF16 of 64 accumulator columns of row r, into the A tile h
-__device__ __forceinline__ void hidden_row(unsigned char* h, int r, const uint32_t (&acc)[64],
-                                           const float* bias) {
+// bias + ReLU + BF16 of 32 accumulator columns (c0 .. c0 + 31) of row r, into
+// the A tile h; `bias` points at column c0's bias
+__device__ __forceinline__ void hidden_half(unsigned char* h, int r, int c0, const uint32_t (&acc)[32],
+                                            const float* bias) {
 #pragma unroll
-  for (int kb = 0; kb < 8; ++kb) {
-    uint32_t w[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int c = 8 * kb + 2 * q;
-      w[q] = pack2_relu(__uint_as_float(acc[c]) + bias[c], __uint_as_float(acc[c + 1]) + bias[c + 1]);
-    }
-    st16(h, cm(r, 8 * kb, 64), make_uint4(w[0], w[1], w[2], w[3]));
+  for (int kb = 0; kb < 4; ++kb) {
+    const float4 b0 = *reinterpret_cast<const float4*>(bias + 8 * kb);
+    const float4 b1 = *reinterpret_cast<const float4*>(bias + 8 * kb + 4);
+    const uint32_t* a = acc + 8 * kb;
+    const uint32_t w0 = pack2_relu(__uint_as_float(a[0]) + b0.x, __uint_as_float(a[1]) + b0.y);
+    const uint32_t w1 = pack2_relu(__uint_as_float(a[2]) + b0.z, __uint_as_float(a[3]) + b0.w);
+    const uint32_t w2 = pack2_relu(__uint_as_float(a[4]) + b1.x, __uint_as_float(a[5]) + b1.y);
+    const uint32_t w3 = pack2_relu(__uint_as_float(a[6]) + b1.z, __uint_as_float(a[7]) + b1.w);
+    st16(h, cm(r, c0 + 8 * kb, 64), make_uint4(w0, w1, w2, w3));
   }
+}
+
+// Barrier of group g's 128 threads that also orders their shared-memory stores
+// and tensor-memory reads with the tensor cores; true when `pred` holds in all
+// of them.
+__device__ __forceinline__ bool group_sync(int g, bool pred) {
+  fence_smem_async();
+  fence_before();
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n"
+      " bar.red.and.pred q, %2, 128, p;\n selp.u32 %0, 1, 0, q;\n}"
+      : "=r"(r)
+      : "r"(pred ? 1u : 0u), "r"(g + 1)
+      : "memory");
+  fence_after();
+  return r != 0;
 }
 
 }  // namespace tc
 
-__global__ void __launch_bounds__(128) k_mlp_infer_tc(Dev d, VertexPtrs v, const int32_t* list,
+__global__ void __launch_bounds__(tc::kThreads, 2) k_mlp_infer_tc(Dev d, VertexPtrs v, const int32_t* list,
                                                       const uint32_t* counter, OutPtrs o, int all) {
   extern __shared__ unsigned char smem_raw[];
   tc::Smem& s = *reinterpret_cast<tc::Smem*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
   const int tid = threadIdx.x, warp = tid >> 5;
+  const int g = tid >> 7, row = tid & 127;  // the thread's group and row of its tile
   // weights in the canonical layout, 8 elements (one 16-byte chunk of a core
   // matrix row) per load, biases
   const uint4* wb4 = reinterpret_cast<const uint4*>(d.wb);
-#pragma unroll 5
   for (int c = tid; c < 64 * kIn / 8; c += blockDim.x)
     tc::st16(s.w1, tc::cm(c / 10, 8 * (c % 10), kIn), __ldg(wb4 + bW1 / 8 + c));
-#pragma unroll 4
   for (int c = tid; c < 64 * kHid / 8; c += blockDim.x) {
     tc::st16(s.w2, tc::cm(c / 8, 8 * (c % 8), kHid), __ldg(wb4 + bW2 / 8 + c));
     tc::st16(s.w3, tc::cm(c / 8, 8 * (c % 8), kHid), __ldg(wb4 + bW3 / 8 + c));
@@ -346,9 +395,10 @@ __global__ void __launch_bounds__(128) k_mlp_infer_tc(Dev d, VertexPtrs v, const
     else if (i < 192 + kOut) b = d.master[oB4 + i - 192];
     s.bias[i] = b;
   }
-  const uint32_t mbar = smem_u32(&s.mbar);
+  const uint32_t mbar = smem_u32(&s.mbar[g]);
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
+    for (int i = 0; i < tc::kGroups; ++i)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.mbar[i])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
@@ -364,57 +414,62 @@ __global__ void __launch_bounds__(128) k_mlp_infer_tc(Dev d, VertexPtrs v, const
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = s.tmem;
-  const uint32_t trow = tmem + (static_cast<uint32_t>(warp * 32) << 16);  // this warp's lanes
-  const uint32_t aa = smem_u32(s.act);
+  const uint32_t td = tmem + 64u * g;                                             // the group's columns
+  const uint32_t trow = td + (static_cast<uint32_t>((warp & 3) * 32) << 16);  // this warp's lanes
+  unsigned char* act = s.act[g];
+  const uint64_t a80 = tc::sdesc(smem_u32(act), 1280u), a64 = tc::sdesc(smem_u32(act), 1024u);
+  const uint64_t b1 = tc::sdesc(smem_u32(s.w1), 1280u), b2 = tc::sdesc(smem_u32(s.w2), 1024u),
+                 b3 = tc::sdesc(smem_u32(s.w3), 1024u), b4 = tc::sdesc(smem_u32(s.w4), 1024u);
   const uint32_t count = *counter;
   const uint32_t ntiles = (count + tc::kRows - 1) / tc::kRows;
+  const uint32_t stride = gridDim.x * tc::kGroups;
   uint32_t parity = 0;
   bool ok = true;
-  auto row_of = [&](uint32_t tile) -> int64_t {
-    const uint32_t i = tile * tc::kRows + tid;
+  auto row_of = [&](uint32_t tile) -> int32_t {
+    const uint32_t i = tile * tc::kRows + row;
     return tile < ntiles && i < count ? list[i] : -1;
   };
-  int64_t j = row_of(blockIdx.x);
+  uint32_t tile = blockIdx.x * tc::kGroups + g;
+  int32_t j = row_of(tile);
   VertexIn vi = load_vertex(d, v, j);
-  int64_t jn = row_of(blockIdx.x + gridDim.x);
-  for (uint32_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-    tc::encode_row(s.act, tid, vi, j >= 0);
+  int32_t jn = row_of(tile + stride);
+  for (; tile < ntiles && ok; tile += stride) {
+    tc::encode_row(act, row, vi, j >= 0);
     // while this tile goes through the layers: the next tile's vertex (its list
     // entry was read one tile ago, so the loads do not wait for it) and the
     // list entry of the tile after
-    const VertexIn vn = load_vertex(d, v, jn);
-    const int64_t jnn = row_of(tile + 2 * gridDim.x);
-    tc::fence_smem_async();
-    tc::fence_before();
-    __syncthreads();
-    tc::fence_after();
-    uint32_t acc[64];
+    vi = load_vertex(d, v, jn);
+    const int32_t jnn = row_of(tile + 2 * stride);
+    ok = tc::group_sync(g, ok);
+    if (!ok) break;
 #pragma unroll 1
     for (int layer = 0; layer < 4; ++layer) {
-      if (tid == 0) {
-        const uint32_t a = aa;
-        const uint32_t sboa = layer == 0 ? 1280u : 1024u;
-        const uint32_t b = smem_u32(layer == 0 ? s.w1 : layer == 1 ? s.w2 : layer == 2 ? s.w3 : s.w4);
-        const int ksteps = layer == 0 ? 5 : 4;
-        const uint32_t id = layer == 3 ? tc::idesc(128, 16) : tc::idesc(128, 64);
-        for (int k = 0; k < ksteps; ++k)
-          tc::mma_bf16(tmem, tc::sdesc(a + 256u * k, sboa), tc::sdesc(b + 256u * k, sboa), id,
-                       k > 0 ? 1u : 0u);
+      if (row == 32 * g) {  // a warp of another scheduler in each group
+        if (layer == 0)
+          tc::mma_steps<5>(td, a80, 16u, b1, 16u, tc::idesc(128, 64));
+        else if (layer < 3)
+          tc::mma_steps<4>(td, a64, 16u, layer == 1 ? b2 : b3, 16u, tc::idesc(128, 64));
+        else
+          tc::mma_steps<4>(td, a64, 16u, b4, 16u, tc::idesc(128, 16));
         tc::commit(mbar);
       }
-      ok = __syncthreads_and(tc::mbar_wait(mbar, parity)) != 0;  // the same outcome in every thread
+      __syncwarp();
+      ok = tc::mbar_wait(mbar, parity);
       parity ^= 1u;
-      if (!ok) break;
       tc::fence_after();
       if (layer < 3) {
-        tc::tmem_ld_x64(trow, acc);
-        tc::tmem_wait_ld();
-        tc::hidden_row(s.act, tid, acc, s.bias + 64 * layer);
-        tc::fence_smem_async();
-        tc::fence_before();
-        __syncthreads();
-        tc::fence_after();
+#pragma unroll 1
+        for (int c0 = 0; c0 < 64; c0 += 32) {
+          uint32_t acc[32];
+          tc::tmem_ld_x32(trow + c0, acc);
+          tc::tmem_wait_ld();
+          tc::hidden_half(act, row, c0, acc, s.bias + 64 * layer + c0);
+        }
+        ok = tc::group_sync(g, ok);  // the same outcome in every thread of the group
+        if (!ok) break;
       } else {
+        // (the next tile's product overwrites the accumulator after the group's
+        // barrier behind its encoding)
         uint32_t y[16];
         tc::tmem_ld_x16(trow, y);
         tc::tmem_wait_ld();
@@ -424,16 +479,12 @@ __global__ void __launch_bounds__(128) k_mlp_infer_tc(Dev d, VertexPtrs v, const
           o.b[j] = __uint_as_float(y[2]) + s.bias[194];
           if (!all) o.status[j] = PPS_STATUS_MLP;
         }
-        tc::fence_before();
-        __syncthreads();  // the next tile's MMA overwrites the accumulator
-        tc::fence_after();
       }
     }
     j = jn;
-    vi = vn;
     jn = jnn;
   }
-  if (!ok && tid == 0) atomicOr(d.err, 1u);
+  if (!ok && (tid & 31) == 0) atomicOr(d.err, 1u);
   tc::fence_before();
   __syncthreads();
   if (warp == 0)
@@ -529,7 +580,7 @@ struct Smem {
   alignas(128) unsigned char dz[128 * 64 * 2];  // dY (16 wide), then dZ_2, dZ_1, dZ_0 [sample][out]
   alignas(128) unsigned char pad[kPad];
   float4 tgt[2][128];  // the two work items' targets (w: the sample is valid)
-  float bias[3 * 64 + 16];
+  alignas(16) float bias[3 * 64 + 16];
   alignas(8) unsigned long long mbar;
   uint32_t tmem;
 };
@@ -558,13 +609,13 @@ __device__ __forceinline__ Operand mnmajor(const void* p, uint32_t C) {
   return Operand{smem_u32(p), C * 16u, 128u, C * 32u};
 }
 
-// Issue `ksteps` MMAs of K = 16 into tensor-memory column `dcol`.
+// Issue KS MMAs of K = 16 into tensor-memory column `dcol`.
+template <int KS>
 __device__ __forceinline__ void issue(uint32_t tmem, uint32_t dcol, Operand a, Operand b, uint32_t n,
-                                      int ksteps, bool a_mn, bool b_mn) {
+                                      bool a_mn, bool b_mn) {
   const uint32_t id = tc::idesc(128, n) | (a_mn ? 1u << 15 : 0u) | (b_mn ? 1u << 16 : 0u);
-  for (int k = 0; k < ksteps; ++k)
-    tc::mma_bf16(tmem + dcol, desc(a.addr + a.kstep * k, a.lbo, a.sbo),
-                 desc(b.addr + b.kstep * k, b.lbo, b.sbo), id, k > 0 ? 1u : 0u);
+  tc::mma_steps<KS>(tmem + dcol, desc(a.addr, a.lbo, a.sbo), a.kstep >> 4, desc(b.addr, b.lbo, b.sbo),
+                    b.kstep >> 4, id);
 }
 
 __device__ __forceinline__ void red_v4(float* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
@@ -648,28 +699,6 @@ __device__ __forceinline__ void adam_apply(const Dev& d, float* grad, int i, con
 }
 
 namespace tct {
-__device__ __forceinline__ void tmem_ld_x32(uint32_t taddr, uint32_t (&v)[32]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-               : "r"(taddr));
-}
-
-// bias + ReLU + BF16 of 32 accumulator columns (c0 .. c0 + 31) of row r, into
-// the A tile h; `bias` points at column c0's bias
-__device__ __forceinline__ void hidden_half(unsigned char* h, int r, int c0, const uint32_t (&acc)[32],
-                                            const float* bias) {
-#pragma unroll
-  for (int kb = 0; kb < 4; ++kb) {
-    uint32_t w[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int c = 8 * kb + 2 * q;
-      w[q] = pack2_relu(__uint_as_float(acc[c]) + bias[c], __uint_as_float(acc[c + 1]) + bias[c + 1]);
-    }
-    tc::st16(h, tc::cm(r, c0 + 8 * kb, 64), make_uint4(w[0], w[1], w[2], w[3]));
-  }
-}
-
 // The step's weights in shared memory: BF16 copies in the canonical layout
 // and the biases (FP32 masters).  Read through L2: the previous step's Adam
 // wrote them during this launch.  The BF16 copies are one contiguous run of
@@ -739,9 +768,12 @@ __device__ __forceinline__ bool grid_sync(Ctrl* c, unsigned int target) {
     int ok = 1;
     __threadfence();
     atomicAdd(&c->bar_count, 1u);
-    const unsigned long long t0 = globaltimer_ns();
-    while (static_cast<int>(ld_acquire_u32(&c->bar_count) - target) < 0) {
-      if ((ld_acquire_u32(&c->error) & kErrBarrierTimeout) || globaltimer_ns() - t0 > 2000000000ull) {
+    unsigned long long t0 = 0ull;
+    for (uint32_t i = 1; static_cast<int>(ld_acquire_u32(&c->bar_count) - target) < 0; ++i) {
+      if (i % 32u) continue;
+      const unsigned long long t = globaltimer_ns();
+      if (t0 == 0ull) t0 = t;
+      if ((ld_acquire_u32(&c->error) & kErrBarrierTimeout) || t - t0 > 2000000000ull) {
         atomicOr(&c->error, kErrBarrierTimeout);
         ok = 0;
         break;
@@ -826,9 +858,20 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_mlp_train_tc(TrainArgs a) 
       };
       // gradient of layer l: gW_l = dZ_l^T X_l and gb_l = dZ_l^T 1 from the delta in s.dz
       auto grad_issue = [&](int l) {
-        const uint32_t co = l == 3 ? 16u : 64u, ci = l == 0 ? kIn : kHid;
-        tct::issue(tmem, tct::gcol(l), tct::mnmajor(s.dz, co), tct::mnmajor(X(l), ci), ci, 8, true, true);
-        tct::issue(tmem, tct::bcol(l), tct::mnmajor(s.dz, co), tct::mnmajor(s.ones, 16), 16, 8, true, true);
+        // (the tile widths as constants, so that the descriptors' steps are)
+        const tct::Operand one = tct::mnmajor(s.ones, 16);
+        if (l == 3) {
+          const tct::Operand dy = tct::mnmajor(s.dz, 16);
+          tct::issue<8>(tmem, tct::gcol(3), dy, tct::mnmajor(s.h[2], kHid), kHid, true, true);
+          tct::issue<8>(tmem, tct::bcol(3), dy, one, 16, true, true);
+        } else {
+          const tct::Operand dz = tct::mnmajor(s.dz, 64);
+          if (l == 0)
+            tct::issue<8>(tmem, tct::gcol(0), dz, tct::mnmajor(x0, kIn), kIn, true, true);
+          else
+            tct::issue<8>(tmem, tct::gcol(l), dz, tct::mnmajor(s.h[l - 1], kHid), kHid, true, true);
+          tct::issue<8>(tmem, tct::bcol(l), dz, one, 16, true, true);
+        }
       };
       // this warp's half of row `row` of gW_l, and (lower) gb_l[row] or (upper,
       // layer 0) the row's inputs 64..79, into the global gradient
@@ -838,7 +881,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_mlp_train_tc(TrainArgs a) 
         const int off = l == 0 ? oW1 : l == 1 ? oW2 : l == 2 ? oW3 : oW4;
         const int boff = l == 0 ? oB1 : l == 1 ? oB2 : l == 2 ? oB3 : oB4;
         uint32_t g[32], e[16];
-        tct::tmem_ld_x32(tq + tct::gcol(l) + hc, g);
+        tc::tmem_ld_x32(tq + tct::gcol(l) + hc, g);
         if (lower) tc::tmem_ld_x16(tq + tct::bcol(l), e);
         else if (l == 0) tc::tmem_ld_x16(tq + tct::gcol(0) + 64, e);
         tc::tmem_wait_ld();
@@ -859,21 +902,23 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_mlp_train_tc(TrainArgs a) 
       uint32_t acc[32];
       // ---- forward: X_{l+1} = ReLU(X_l W_l^T + b_l), l = 0..2
       for (int l = 0; l < 3 && ok; ++l) {
-        const uint32_t C = l == 0 ? kIn : kHid;
         if (tid == 0) {
-          tct::issue(tmem, 0, tct::kmajor(X(l), C), tct::kmajor(W(l), C), 64, C / 16, false, false);
+          if (l == 0)
+            tct::issue<5>(tmem, 0, tct::kmajor(x0, kIn), tct::kmajor(s.w1, kIn), 64, false, false);
+          else
+            tct::issue<4>(tmem, 0, tct::kmajor(s.h[l - 1], kHid), tct::kmajor(W(l), kHid), 64, false, false);
           tc::commit(mbar);
         }
         wait();
         if (!ok) break;
-        tct::tmem_ld_x32(tq + hc, acc);
+        tc::tmem_ld_x32(tq + hc, acc);
         tc::tmem_wait_ld();
-        tct::hidden_half(s.h[l], row, static_cast<int>(hc), acc, s.bias + 64 * l + hc);
+        tc::hidden_half(s.h[l], row, static_cast<int>(hc), acc, s.bias + 64 * l + hc);
         chain_sync_tc();
       }
       if (ok) {
         if (tid == 0) {
-          tct::issue(tmem, 0, tct::kmajor(s.h[2], kHid), tct::kmajor(s.w4, kHid), 16, 4, false, false);
+          tct::issue<4>(tmem, 0, tct::kmajor(s.h[2], kHid), tct::kmajor(s.w4, kHid), 16, false, false);
           tc::commit(mbar);
         }
         wait();
@@ -904,14 +949,16 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_mlp_train_tc(TrainArgs a) 
       // by X_l > 0 and rounded replaces it
       for (int l = 3; l >= 1 && ok; --l) {
         if (tid == 0) {
-          const uint32_t co = l == 3 ? 16u : 64u;
-          tct::issue(tmem, 0, tct::kmajor(s.dz, co), tct::mnmajor(W(l), kHid), 64, co / 16, false, true);
+          if (l == 3)
+            tct::issue<1>(tmem, 0, tct::kmajor(s.dz, 16), tct::mnmajor(s.w4, kHid), 64, false, true);
+          else
+            tct::issue<4>(tmem, 0, tct::kmajor(s.dz, 64), tct::mnmajor(W(l), kHid), 64, false, true);
           grad_issue(l);
           tc::commit(mbar);
         }
         wait();
         if (!ok) break;
-        tct::tmem_ld_x32(tq + hc, acc);
+        tc::tmem_ld_x32(tq + hc, acc);
         const unsigned char* xl = X(l);
         uint4 hq[4];
 #pragma unroll
@@ -1303,8 +1350,9 @@ static int launch_infer(pps_mlp* m, const pps_vertices* v, size_t n, const pps::
   pps::mlp::k_mlp_compact<<<cgrid, 256, 0, st>>>(n, o.status, o.count, m->p.infer_max_count, all,
                                                  vec, m->list, m->counter);
   MLP_CUDA(cudaGetLastError());
-  const int grid = static_cast<int>(std::min<size_t>(static_cast<size_t>(sms) * 4, (n + 127) / 128));
-  pps::mlp::k_mlp_infer_tc<<<grid, 128, pps::mlp::tc::kSmemBytes, st>>>(m->dev, vptrs(v), m->list,
+  const int grid = static_cast<int>(std::min<size_t>(static_cast<size_t>(sms) * 2,
+                                                     (n + pps::mlp::tc::kThreads - 1) / pps::mlp::tc::kThreads));
+  pps::mlp::k_mlp_infer_tc<<<grid, pps::mlp::tc::kThreads, pps::mlp::tc::kSmemBytes, st>>>(m->dev, vptrs(v), m->list,
                                                                         m->counter, o, all);
   MLP_CUDA(cudaGetLastError());
   return PPS_OK;
