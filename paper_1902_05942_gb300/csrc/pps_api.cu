@@ -207,9 +207,9 @@ int empty_slots(pps_table* t, cudaStream_t st) {
   return PPS_OK;
 }
 
-// Begin a frame: reset its counters and, unless its launch empties the whole
-// slot table itself (`swept`), the slots.
-int reset_frame(pps_table* t, bool swept, cudaStream_t st) {
+// Begin a frame: unless its launch empties the whole slot table itself
+// (`swept`), empty the slots.
+int reset_slots(pps_table* t, bool swept, cudaStream_t st) {
   if (!swept) {
     if (int rc = empty_slots(t, st)) return rc;
   } else if (t->state != kClean) {
@@ -217,6 +217,11 @@ int reset_frame(pps_table* t, bool swept, cudaStream_t st) {
   }
   t->frame_tiles = 0;
   t->state = kClean;
+  return PPS_OK;
+}
+
+// The frame's counters to zero (a persistent launch does it itself).
+int reset_counters(pps_table* t, cudaStream_t st) {
   PPS_CUDA(cudaMemsetAsync(t->dev.ctrl, 0, pps::kCtrlFrameBytes, st));
   return PPS_OK;
 }
@@ -459,7 +464,8 @@ int pps_build(pps_table* t, const pps_camera* cam, uint32_t frame, void* stream)
   if (int rc = check_table(t)) return rc;
   if (!cam) return fail(PPS_EINVAL, "camera is NULL");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (int rc = reset_frame(t, false, st)) return rc;
+  if (int rc = reset_slots(t, false, st)) return rc;
+  if (int rc = reset_counters(t, st)) return rc;
   set_camera(t, cam, frame);
   t->state = kOpen;
   if (t->coarse) return pps_build(t->coarse, cam, frame, stream);
@@ -540,23 +546,28 @@ int filter_one(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_ve
   plan.neigh = t->dev.neighbors != 0;
   plan.kv = v->dist || v->extra;
   plan.sweep = n && pps::sweep_pays_host(t->dev, n);
-  if (int rc = reset_frame(t, plan.sweep, st)) return rc;
+  if (int rc = reset_slots(t, plan.sweep, st)) return rc;
   set_camera(t, cam, frame);
-  if (n == 0) return PPS_OK;
-  PPS_CUDA(pps::plan_fused(n, ~size_t{0}, &plan));
-  if (int rc = ensure_dense(t, pps::fused_cells(n, plan.tile, plan.batch), 0, st)) return rc;
-  if (t->dev.neighbors && t->neigh_q_cap < n) {
-    cudaFree(t->neigh_q);
-    t->neigh_q = nullptr;
-    t->neigh_q_cap = 0;
-    if (cudaMalloc(reinterpret_cast<void**>(&t->neigh_q), n * sizeof(uint32_t)) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(PPS_ENOMEM, "pps_filter: neighborhood queue allocation failed");
+  if (n == 0) return reset_counters(t, st);
+  auto ready = [&]() -> int {
+    PPS_CUDA(pps::plan_fused(n, ~size_t{0}, &plan));
+    if (int rc = ensure_dense(t, pps::fused_cells(n, plan.tile, plan.batch), 0, st)) return rc;
+    if (t->dev.neighbors && t->neigh_q_cap < n) {
+      cudaFree(t->neigh_q);
+      t->neigh_q = nullptr;
+      t->neigh_q_cap = 0;
+      if (cudaMalloc(reinterpret_cast<void**>(&t->neigh_q), n * sizeof(uint32_t)) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(PPS_ENOMEM, "pps_filter: neighborhood queue allocation failed");
+      }
+      t->neigh_q_cap = n;
     }
-    t->neigh_q_cap = n;
+    return blend ? next_epoch(t, st) : PPS_OK;
+  };
+  if (int rc = ready()) {  // no launch to reset the counters
+    cudaMemsetAsync(t->dev.ctrl, 0, pps::kCtrlFrameBytes, st);
+    return rc;
   }
-  if (blend)
-    if (int rc = next_epoch(t, st)) return rc;
   PPS_CUDA(pps::launch_fused(t->kc, t->dev, to_dev(v), n, out, blend != 0, alpha, plan, t->stash,
                              t->neigh_q, st));
   t->stale = plan.sweep;
@@ -849,7 +860,7 @@ int pps_stats(pps_table* t, pps_stats_t* out, void* stream) {
   out->frame = t->kc.frame;
   if (c.error) {
     // clear the error word and the barrier state so the table stays usable
-    PPS_CUDA(cudaMemsetAsync(&t->dev.ctrl->error, 0, 3 * sizeof(unsigned int), st));  // + barrier
+    PPS_CUDA(cudaMemsetAsync(&t->dev.ctrl->error, 0, pps::kCtrlErrorBytes, st));  // + barrier
     PPS_CUDA(cudaStreamSynchronize(st));
     return fail(PPS_EDEVICE, pps::device_error_text(c.error));
   }

@@ -115,16 +115,13 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
   if (e == cudaSuccess && b->total_tiles)
     e = cudaMalloc(&b->gstash, static_cast<size_t>(b->total_tiles) * tile * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
-  // capture: descriptor upload, counter resets, the persistent kernel
+  // capture: descriptor upload, the persistent kernel
   cudaStream_t cs = nullptr;
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
   for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
     cudaGraph_t g = nullptr;
     e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->dviews[k], b->hviews[k], bytes, cudaMemcpyHostToDevice, cs);
-    for (size_t i = 0; i < b->base.size() && e == cudaSuccess; ++i)
-      e = cudaMemsetAsync(b->base[i].t.ctrl, 0, pps::kCtrlFrameBytes, cs);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->ctrl, 0, pps::kCtrlFrameBytes, cs);
     if (e == cudaSuccess)
       e = pps::launch_multi(b->dviews[k], nviews, b->total_tiles, b->ctrl, b->temporal, alpha,
                             b->plan, b->gstash, cs);

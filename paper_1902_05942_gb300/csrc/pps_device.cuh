@@ -59,10 +59,10 @@ struct Ctrl {
   unsigned long long neigh_count;  // persistent kernel: low-count vertices queued for the search
   unsigned int error;
   unsigned int bar_count;
-  unsigned int bar_gen;
-  unsigned int pad[1];
+  unsigned int pad[2];
 };
 constexpr size_t kCtrlFrameBytes = 5 * sizeof(unsigned long long);  // reset per frame
+constexpr size_t kCtrlErrorBytes = 2 * sizeof(unsigned int);        // error word and barrier, from `error` on
 
 enum : unsigned int {
   kErrBarrierTimeout = 1u,
@@ -849,42 +849,58 @@ __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
   return v;
 }
 
-// Barrier over all CTAs of a cooperative launch.  Thread 0 of each CTA
-// arrives on a counter; the last arrival resets it and bumps the generation;
-// the others wait for the generation to change.  The wait is bounded (about
-// two seconds of wall time): on timeout the CTA raises kErrBarrierTimeout in
-// the device error word and every CTA returns false, so the launch ends.
+// The frame's counters to zero, by one thread; a grid barrier has to come
+// before the first one that adds to them.
+__device__ __forceinline__ void reset_counters(Ctrl* c) {
+  c->frame_cells = 0ull;
+  c->overflow_vertices = 0ull;
+  c->vertices = 0ull;
+  c->hist_overflow = 0ull;
+  c->neigh_count = 0ull;
+}
+
+// Barrier over all CTAs of a cooperative launch, sense-reversing (Mellor-Crummey
+// and Scott, 1991) on one word: the arrivals of one barrier add up to 2^31 (CTA 0
+// adds 2^31 less one per other CTA), so the word's top bit is the sense, flips
+// with the last arrival, and the low bits are back where they were: nobody
+// resets anything.  Thread 0 of each CTA reads the sense, arrives with one
+// reduction (it returns nothing, so nobody waits for it) and polls the same
+// word.  The reduction releases and the poll acquires what the CTA's threads
+// wrote.  An arrival counter whose last arrival resets it and then moves a
+// generation on is three dependent round trips.  Frames of 7,680 and 65,536
+// vertices (three barriers): 27.3 -> 24.4 us and 28.8 -> 24.5 us, about half of it
+// this, half the counters' reset moving into the launch.
+//
+// The wait is bounded (about two seconds of wall time): on timeout the CTA
+// raises kErrBarrierTimeout in the device error word and every CTA returns
+// false, so the launch ends.
 __device__ __forceinline__ bool grid_barrier(Ctrl* c, unsigned int nblocks,
                                              unsigned long long limit_ns = 2000000000ull) {
+  constexpr unsigned int kSense = 0x80000000u;
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
-    const unsigned int gen = ld_acquire_u32(&c->bar_gen);
-    __threadfence();
-    const unsigned int arrived = atomicAdd(&c->bar_count, 1u);
-    if (arrived == nblocks - 1u) {
-      atomicExch(&c->bar_count, 0u);
-      __threadfence();
-      atomicAdd(&c->bar_gen, 1u);
-    } else {
-      unsigned long long t0 = 0ull;
-      for (uint32_t i = 1; ld_acquire_u32(&c->bar_gen) == gen; ++i) {
-        if (i % 32u) continue;  // the error word and the clock now and then only
-        const unsigned long long now = globaltimer_ns();
-        if (t0 == 0ull) t0 = now;
-        if (ld_acquire_u32(&c->error) & kErrBarrierTimeout) {
-          ok = 0;
-          break;
-        }
-        if (now - t0 > limit_ns) {
-          atomicOr(&c->error, kErrBarrierTimeout);
-          ok = 0;
-          break;
-        }
+    unsigned int before;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(before) : "l"(&c->bar_count) : "memory");
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&c->bar_count),
+                 "r"(blockIdx.x == 0 ? kSense - (nblocks - 1u) : 1u)
+                 : "memory");
+    unsigned long long t0 = 0ull;
+    for (uint32_t i = 1; !((ld_acquire_u32(&c->bar_count) ^ before) & kSense); ++i) {
+      if (i % 32u) continue;  // the error word and the clock now and then only
+      const unsigned long long now = globaltimer_ns();
+      if (t0 == 0ull) t0 = now;
+      if (ld_acquire_u32(&c->error) & kErrBarrierTimeout) {
+        ok = 0;
+        break;
+      }
+      if (now - t0 > limit_ns) {
+        atomicOr(&c->error, kErrBarrierTimeout);
+        ok = 0;
+        break;
       }
     }
-    __threadfence();
     s_ok = ok;
   }
   __syncthreads();

@@ -1137,12 +1137,14 @@ __global__ void __launch_bounds__(kFusedBlock, W == 4 ? 1 : 2) k_fused(FusedArgs
   const uint32_t ntiles = static_cast<uint32_t>((a.n + tile_v - 1) / tile_v);
   const uint32_t gw = grid_warp(), nw = grid_warps();
   const bool blended = TEMPORAL && a.blend;
+  if (blockIdx.x == 0 && threadIdx.x == 0) reset_counters(t.ctrl);
   if (a.sweep) {
     sweep_slots(t, blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x,
                 static_cast<size_t>(gridDim.x) * blockDim.x);
     if (!grid_barrier(t.ctrl, gridDim.x)) return;
   }
 
+  unsigned long long n_ovf, n_cells;
   {
     WarpInsert<W> s;
     const bool rec = blended || !a.sweep;
@@ -1164,15 +1166,15 @@ __global__ void __launch_bounds__(kFusedBlock, W == 4 ? 1 : 2) k_fused(FusedArgs
       if (lane == 0) __stcg(t.bcount + tile, s.claims);
     }
     s.retire(t, rec);
-    const unsigned long long o = block_sum(static_cast<unsigned long long>(s.cnt.ovf));
-    const unsigned long long c = block_sum(static_cast<unsigned long long>(s.cnt.cells));
-    if (threadIdx.x == 0) {
-      if (o) atomicAdd(&t.ctrl->overflow_vertices, o);
-      if (c) atomicAdd(&t.ctrl->frame_cells, c);
-      if (blockIdx.x == 0) atomicAdd(&t.ctrl->vertices, static_cast<unsigned long long>(a.n));
-    }
+    n_ovf = block_sum(static_cast<unsigned long long>(s.cnt.ovf));
+    n_cells = block_sum(static_cast<unsigned long long>(s.cnt.cells));
   }
   if (!grid_barrier(t.ctrl, gridDim.x)) return;
+  if (threadIdx.x == 0) {
+    if (n_ovf) atomicAdd(&t.ctrl->overflow_vertices, n_ovf);
+    if (n_cells) atomicAdd(&t.ctrl->frame_cells, n_cells);
+    if (blockIdx.x == 0) atomicAdd(&t.ctrl->vertices, static_cast<unsigned long long>(a.n));
+  }
 
   for (size_t j = gw * static_cast<size_t>(128); j < a.n; j += nw * static_cast<size_t>(128))
     add_warp(t, a.v, j, a.n, a.stash, a.merge, sh);
@@ -1236,6 +1238,8 @@ __global__ void __launch_bounds__(BLOCK, (W == 4 ? 1 : 2) * (kFusedBlock / BLOCK
   const uint32_t run0 = static_cast<uint32_t>(gw * a.total_tiles / nw);
   const uint32_t run1 = static_cast<uint32_t>((gw + 1) * a.total_tiles / nw);
 
+  if (threadIdx.x == 0)
+    for (uint32_t v = blockIdx.x; v < a.nviews; v += gridDim.x) reset_counters(a.views[v].t.ctrl);
   // empty the slot tables of the views that are swept
   for (uint32_t v = 0; v < a.nviews; ++v) {
     take_view(&vd, a, __ldg(&a.views[v].tile_base), cur);

@@ -181,10 +181,11 @@ __global__ void __launch_bounds__(256) k_mlp_compact(size_t n, const uint8_t* st
 // epilogue): a tile took 6.3 us, of which its instructions were 2.2 us, with
 // four CTAs of one group per multiprocessor.  Sharing the weights makes room
 // for eight groups (32 warps at 64 registers, the epilogues in halves of 32
-// columns), and a layer has one barrier instead of two.HD frame,
-// 1.84 M listed vertices: 149 us with four single-group CTAs, 140 like this;
-// what bounds it now is shared memory (69 % of its cycles: the products'
-// operands 35 %, the activations' stores 21 %) and issue (53 %).
+// columns), and a layer has one barrier instead of two.  HD
+// frame, 1.84 M listed vertices: 149 us with four single-group CTAs, 140 like
+// this; what bounds it now is the shared-memory pipe (69 % of its cycles: 44 % of
+// that the biases, read by every row, 31 % the activations' stores) and issue
+// (53 %).
 namespace tc {
 constexpr int kRows = 128;
 constexpr int kGroups = 4;

@@ -253,8 +253,7 @@ extern "C" int pps_noalloc_stats(pps_stats_t* out, void* stream) {
   out->device_error = c.error;
   if (c.error) {
     // clear the error word and the grid-barrier state for the next call
-    e = cudaMemsetAsync(base + kOffCtrl + offsetof(pps::Ctrl, error), 0, 3 * sizeof(unsigned int),
-                        st);
+    e = cudaMemsetAsync(base + kOffCtrl + offsetof(pps::Ctrl, error), 0, pps::kCtrlErrorBytes, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess)
       return noalloc_fail(PPS_ECUDA, std::string("pps_noalloc_stats: ") + cudaGetErrorString(e));
