@@ -418,14 +418,12 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64_keep(const unsigned
   return v;
 }
 
-// Two neighbouring slots (p 16-byte aligned), each a relaxed read of its own.
-__device__ __forceinline__ ulonglong2 ld_relaxed_u64x2_keep(const unsigned long long* p) {
-  ulonglong2 v;
-  asm volatile("ld.relaxed.gpu.global.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;"
-               : "=l"(v.x), "=l"(v.y)
+// The four slots of a sector (p 32-byte aligned), each a relaxed read of its own.
+__device__ __forceinline__ void ld_relaxed_u64x4_keep(const unsigned long long* p, unsigned long long (&w)[4]) {
+  asm volatile("ld.relaxed.gpu.global.L2::cache_hint.v4.u64 {%0, %1, %2, %3}, [%4], %5;"
+               : "=l"(w[0]), "=l"(w[1]), "=l"(w[2]), "=l"(w[3])
                : "l"(p), "l"(l2_evict_last())
                : "memory");
-  return v;
 }
 
 __device__ __forceinline__ void red_add_v4_keep(float4* p, float a, float b, float c, float d) {
@@ -867,9 +865,8 @@ __device__ __forceinline__ void reset_counters(Ctrl* c) {
 // reduction (it returns nothing, so nobody waits for it) and polls the same
 // word.  The reduction releases and the poll acquires what the CTA's threads
 // wrote.  An arrival counter whose last arrival resets it and then moves a
-// generation on is three dependent round trips.  Frames of 7,680 and 65,536
-// vertices (three barriers): 27.3 -> 24.4 us and 28.8 -> 24.5 us, about half of it
-// this, half the counters' reset moving into the launch.
+// generation on is three dependent round trips.
+// @@BARRIER@@
 //
 // The wait is bounded (about two seconds of wall time): on timeout the CTA
 // raises kErrBarrierTimeout in the device error word and every CTA returns
