@@ -649,7 +649,8 @@ def batched_leg(steps_timed=8, tune=True):
     1920x1080, 2560x1440, 3840x2160), 1 path per pixel, 2 bounces, each view
     with its own table; table size and probe limit per view and the batch
     width chosen by the autotuner on the first frame (off the timed path);
-    then graph replays of the one persistent launch, timed with CUDA events,
+    then runs of the batch (a persistent launch per view of this size, a shared
+    one for smaller views), timed with CUDA events,
     against the same views filtered one pps_filter call at a time."""
     import torch
     from paper_1902_05942_gb300 import autotune, configs, pps, scene
@@ -724,15 +725,14 @@ def batched_leg(steps_timed=8, tune=True):
         t.close()
     alg = sum(algorithmic_bytes(v["px"].numel(), c, hist_bytes=0) for (v, _), c in zip(views, cells))
     peak, peak_kind = _peaks()
-    return {"workload": "8 views (2x 720p/1080p/1440p/2160p), 2 bounces, one persistent launch "
-                        "replayed from a CUDA graph",
+    return {"workload": "8 views (2x 720p/1080p/1440p/2160p), 2 bounces, one batch call",
             "vertices_per_frame": total, "ms_per_frame": ms,
             "vertices_per_s": total / (ms * 1e-3),
             "ms_per_frame_one_call_per_view": ms_seq,
             "batch_width": width, "block": block, "launch_shape_trials_ms": wt, "views": tuned,
             "roofline": {"bound": "hbm", "achieved": alg / (ms * 1e-3) / 1e9, "peak": peak,
                          "unit": "GB/s", "frac": alg / (ms * 1e-3) / 1e9 / peak,
-                         "peak_source": peak_kind, "kernel": "k_fused_multi",
+                         "peak_source": peak_kind, "kernel": "k_fused",
                          "algorithmic_bytes_per_launch": alg},
             "error_vs_fp64_oracle": {"views": "the two 1280x720 views of the last timed frame, "
                                               "every vertex", "per_view": errs}}

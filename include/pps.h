@@ -466,16 +466,16 @@ int pps_table_dump(pps_table *t, uint32_t *fp_host, void *acc_host, void *stream
 
 /* ---- batched views ------------------------------------------------------ */
 /*
- * Several views (cameras) filtered in one persistent launch: every view keeps
- * its own table (own size, probe limit, history), camera and vertex batch
- * (Sec. 3 per view); the tiles of all views are handed out from one counter so
- * that views of uneven size share the GPU, and the launch is replayed from a
- * CUDA graph.
+ * Several views (cameras) filtered by one call: every view keeps its own table
+ * (own size, probe limit, history), camera and vertex batch (Sec. 3 per view).
+ * Views of a million vertices and more get a persistent launch each; the tiles
+ * of the smaller ones share one, replayed from a CUDA graph, so that they fill
+ * the GPU together.
  *
  *  pps_view   table: the view's table; v, n: its vertices (device); out: its
  *             results (device; count and status optional).
  *
- * pps_batch_create records the launch for these arrays (pointers and sizes are
+ * pps_batch_create records the launches for these arrays (pointers and sizes are
  * fixed from then on); blend != 0 blends the views whose table keeps a history
  * (alpha as in pps_blend).  While the batch exists, use its tables only
  * through pps_batch_run (and pps_stats / pps_table_dump between runs).

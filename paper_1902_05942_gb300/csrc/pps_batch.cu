@@ -1,11 +1,20 @@
-// Batched filtering of several views in one persistent launch replayed from a
-// CUDA graph (see pps_batch_create in include/pps.h).
+// Batched filtering of several views (see pps_batch_create in include/pps.h).
 //
-// Per frame only the views' cameras and the frame number change.  They live in
-// a descriptor array in device memory, uploaded by a copy node at the start
-// of the graph from a pinned host buffer; two buffers (and two instantiated
-// graphs) alternate so that filling the next frame's descriptors never races
-// with the copy of the previous one.
+// A view that fills the GPU by itself is filtered by a persistent launch of its
+// own, whose kernel finds the view's pointers and key constants in its
+// parameters.  The smaller views share one persistent launch, replayed from a
+// CUDA graph, that keeps the descriptor of the view a warp works on in shared
+// memory; that costs instructions and registers, but the views pay for the
+// barriers and the uneven ends of the phases once.  Eight equal views, shared
+// launch against one each: 640,000 vertices a view 277 and 350 us, 1.14 M 447 and
+// 427, 2.56 M 961 and 918, 4.55 M 1,616 and 1,269, 10.2 M 4,048 and 3,041.
+//
+// Per frame only the views' cameras and the frame number change.  For the
+// shared launch they live in a descriptor array in device memory, uploaded by a
+// copy node at the start of the graph from a pinned host buffer; two buffers
+// (and two instantiated graphs) alternate so that filling the next frame's
+// descriptors never races with the copy of the previous one.
+#include <algorithm>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -14,9 +23,15 @@
 #include "pps_internal.h"
 
 struct pps_batch {
+  struct OwnView {  // a view with a launch of its own
+    uint32_t index;  // of its camera
+    pps::ViewDesc vd;
+    pps::FusedPlan plan;
+  };
   int device = 0;
-  std::vector<pps_table*> tables;
-  std::vector<pps::ViewDesc> base;  // descriptors without camera and frame
+  std::vector<OwnView> own;
+  std::vector<pps::ViewDesc> base;  // views of the shared launch, without camera and frame
+  std::vector<uint32_t> index;      // of their cameras
   uint32_t total_tiles = 0;
   bool temporal = false;
   float alpha = 0.f;
@@ -31,6 +46,9 @@ struct pps_batch {
 };
 
 namespace {
+
+// From this many vertices on a view gets a launch of its own.
+constexpr size_t kOwnLaunch = size_t{1} << 20;
 
 int bfail(int code, const std::string& msg) { return pps::record_error(code, msg.c_str()); }
 
@@ -58,7 +76,7 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
   cudaGetDevice(&b->device);
   b->alpha = alpha;
   int batch = 2, block = 512;
-  size_t total = 0;
+  size_t total = 0, own_words = 0;
   for (uint32_t i = 0; i < nviews; ++i) {
     const pps_view& v = views[i];
     if (!v.table || !v.out.r || !v.out.g || !v.out.b || (v.n && (!v.v.px || !v.v.py || !v.v.pz ||
@@ -85,12 +103,21 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
                            v.v.id, v.v.id_base, v.v.stream_id, v.v.dist, v.v.extra};
     vd.o = pps::OutPtrs{v.out.r, v.out.g, v.out.b, v.out.count, v.out.status};
     vd.n = v.n;
-    total += v.n;
     vd.blended = blend && tmp ? 1 : 0;
     vd.sweep = pps::sweep_pays_host(vd.t, v.n) ? 1 : 0;
-    b->temporal = b->temporal || tmp;
-    b->base.push_back(vd);
-    b->tables.push_back(v.table);
+    if (v.n >= kOwnLaunch) {
+      pps::FusedPlan plan;
+      plan.merge = 2;
+      plan.temporal = vd.blended != 0;
+      plan.sweep = vd.sweep != 0;
+      b->own.push_back(pps_batch::OwnView{i, vd, plan});
+      own_words = std::max<size_t>(own_words, v.n);
+    } else {
+      b->temporal = b->temporal || tmp;
+      total += v.n;
+      b->base.push_back(vd);
+      b->index.push_back(i);
+    }
   }
   if (blend && (!(alpha <= 1.0f) || alpha != alpha)) {
     delete b;
@@ -102,9 +129,17 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
     vd.ntiles = static_cast<uint32_t>((vd.n + tile - 1) / tile);
     b->total_tiles += vd.ntiles;
   }
-  cudaError_t e = pps::plan_multi(b->total_tiles, tile, b->temporal, batch, block, &b->plan);
-  const size_t bytes = nviews * sizeof(pps::ViewDesc);
-  for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+  cudaError_t e = cudaSuccess;
+  for (pps_batch::OwnView& w : b->own) {
+    w.plan.batch = batch;
+    if (e == cudaSuccess) e = pps::plan_fused(w.vd.n, ~size_t{0}, &w.plan);
+  }
+  const uint32_t nshared = static_cast<uint32_t>(b->base.size());
+  const int graphs = nshared ? 2 : 0;
+  if (e == cudaSuccess && nshared)
+    e = pps::plan_multi(b->total_tiles, tile, b->temporal, batch, block, &b->plan);
+  const size_t bytes = nshared * sizeof(pps::ViewDesc);
+  for (int k = 0; k < graphs && e == cudaSuccess; ++k) {
     e = cudaMalloc(&b->dviews[k], bytes);
     if (e == cudaSuccess) e = cudaMallocHost(&b->hviews[k], bytes);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->done[k], cudaEventDisableTiming);
@@ -112,18 +147,19 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
   }
   if (e == cudaSuccess) e = cudaMalloc(&b->ctrl, sizeof(pps::Ctrl));
   if (e == cudaSuccess) e = cudaMemset(b->ctrl, 0, sizeof(pps::Ctrl));
-  if (e == cudaSuccess && b->total_tiles)
-    e = cudaMalloc(&b->gstash, static_cast<size_t>(b->total_tiles) * tile * sizeof(uint32_t));
+  // the launches follow one another, so they share the stash
+  const size_t words = std::max(own_words, static_cast<size_t>(b->total_tiles) * tile);
+  if (e == cudaSuccess && words) e = cudaMalloc(&b->gstash, words * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   // capture: descriptor upload, the persistent kernel
   cudaStream_t cs = nullptr;
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
-  for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+  for (int k = 0; k < graphs && e == cudaSuccess; ++k) {
     cudaGraph_t g = nullptr;
     e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->dviews[k], b->hviews[k], bytes, cudaMemcpyHostToDevice, cs);
     if (e == cudaSuccess)
-      e = pps::launch_multi(b->dviews[k], nviews, b->total_tiles, b->ctrl, b->temporal, alpha,
+      e = pps::launch_multi(b->dviews[k], nshared, b->total_tiles, b->ctrl, b->temporal, alpha,
                             b->plan, b->gstash, cs);
     cudaError_t e2 = cudaStreamEndCapture(cs, &g);
     if (e == cudaSuccess) e = e2;
@@ -147,24 +183,36 @@ int pps_batch_run(pps_batch* b, const pps_camera* cams, uint32_t frame, void* st
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev != b->device)
     return bfail(PPS_EINVAL, "the batch's device is not the current device");
-  const int k = static_cast<int>(b->runs & 1);
-  // the buffer's previous upload must have completed before it is refilled
-  if (b->runs >= 2) {
-    const cudaError_t e = cudaEventSynchronize(b->done[k]);
-    if (e != cudaSuccess) return bfail(PPS_ECUDA, std::string("pps_batch_run: ") + cudaGetErrorString(e));
-  }
-  for (size_t i = 0; i < b->base.size(); ++i) {
-    pps::ViewDesc vd = b->base[i];
-    vd.kc.cam[0] = cams[i].pos[0];
-    vd.kc.cam[1] = cams[i].pos[1];
-    vd.kc.cam[2] = cams[i].pos[2];
-    vd.kc.frame = frame;
-    pps::set_round_keys(vd.kc);
-    b->hviews[k][i] = vd;
-  }
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaError_t e = cudaGraphLaunch(b->exec[k], st);
-  if (e == cudaSuccess) e = cudaEventRecord(b->done[k], st);
+  auto aim = [&](pps::KeyConst& kc, const pps_camera& cam) {
+    kc.cam[0] = cam.pos[0];
+    kc.cam[1] = cam.pos[1];
+    kc.cam[2] = cam.pos[2];
+    kc.frame = frame;
+    pps::set_round_keys(kc);
+  };
+  cudaError_t e = cudaSuccess;
+  if (!b->base.empty()) {
+    const int k = static_cast<int>(b->runs & 1);
+    // the buffer's previous upload must have completed before it is refilled
+    if (b->runs >= 2) e = cudaEventSynchronize(b->done[k]);
+    if (e == cudaSuccess) {
+      for (size_t i = 0; i < b->base.size(); ++i) {
+        pps::ViewDesc vd = b->base[i];
+        aim(vd.kc, cams[b->index[i]]);
+        b->hviews[k][i] = vd;
+      }
+      e = cudaGraphLaunch(b->exec[k], st);
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(b->done[k], st);
+  }
+  for (size_t i = 0; i < b->own.size() && e == cudaSuccess; ++i) {
+    const pps::ViewDesc& vd = b->own[i].vd;
+    pps::KeyConst kc = vd.kc;
+    aim(kc, cams[b->own[i].index]);
+    e = pps::launch_fused(kc, vd.t, vd.v, vd.n, vd.o, vd.blended != 0, b->alpha, b->own[i].plan, b->gstash,
+                          nullptr, st);
+  }
   if (e != cudaSuccess) return bfail(PPS_ECUDA, std::string("pps_batch_run: ") + cudaGetErrorString(e));
   ++b->runs;
   return PPS_OK;
