@@ -112,6 +112,8 @@ __global__ void __launch_bounds__(256) k_mlp_compact(size_t n, const uint8_t* st
                                                      const uint32_t* count, uint32_t max_count,
                                                      int all, int vec, int32_t* list,
                                                      uint32_t* counter) {
+  // the evaluation's CTAs may start setting up (they wait for this grid's end)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __shared__ uint32_t s_warp[8];
   __shared__ uint32_t s_base;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -422,7 +424,11 @@ __global__ void __launch_bounds__(tc::kThreads, 2) k_mlp_infer_tc(Dev d, VertexP
   const uint64_t a80 = tc::sdesc(smem_u32(act), 1280u), a64 = tc::sdesc(smem_u32(act), 1024u);
   const uint64_t b1 = tc::sdesc(smem_u32(s.w1), 1280u), b2 = tc::sdesc(smem_u32(s.w2), 1024u),
                  b3 = tc::sdesc(smem_u32(s.w3), 1024u), b4 = tc::sdesc(smem_u32(s.w4), 1024u);
-  const uint32_t count = *counter;
+  // The list and its length are the listing kernel's: up to here the launch ran
+  // beside its end (the weights were there before it).  HD frame 151.7 us with
+  // one launch after the other, 147.5 us like this.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const uint32_t count = __ldcg(counter);
   const uint32_t ntiles = (count + tc::kRows - 1) / tc::kRows;
   const uint32_t stride = gridDim.x * tc::kGroups;
   uint32_t parity = 0;
@@ -1364,9 +1370,19 @@ static int launch_infer(pps_mlp* m, const pps_vertices* v, size_t n, const pps::
   MLP_CUDA(cudaGetLastError());
   const int grid = static_cast<int>(std::min<size_t>(static_cast<size_t>(sms) * 2,
                                                      (n + pps::mlp::tc::kThreads - 1) / pps::mlp::tc::kThreads));
-  pps::mlp::k_mlp_infer_tc<<<grid, pps::mlp::tc::kThreads, pps::mlp::tc::kSmemBytes, st>>>(m->dev, vptrs(v), m->list,
-                                                                        m->counter, o, all);
-  MLP_CUDA(cudaGetLastError());
+  cudaLaunchAttribute early{};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(pps::mlp::tc::kThreads);
+  cfg.dynamicSmemBytes = pps::mlp::tc::kSmemBytes;
+  cfg.stream = st;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  MLP_CUDA(cudaLaunchKernelEx(&cfg, pps::mlp::k_mlp_infer_tc, m->dev, vptrs(v),
+                              static_cast<const int32_t*>(m->list),
+                              static_cast<const uint32_t*>(m->counter), o, all));
   return PPS_OK;
 }
 

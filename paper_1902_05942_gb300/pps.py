@@ -361,7 +361,8 @@ def pps_bench_rate(kind: str, region: torch.Tensor, ops: int, stream=None) -> fl
 
 # ---------------------------------------------------------------- batched views
 class Batch:
-    """Several views in one persistent launch replayed from a CUDA graph.
+    """Several views filtered by one call (large ones by a launch each, the
+    others by a shared launch replayed from a CUDA graph).
 
     views: list of (Table, vertex dict, output dict).  The arrays must stay
     alive (and in place) for the batch's lifetime."""
