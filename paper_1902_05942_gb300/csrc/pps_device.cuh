@@ -411,15 +411,6 @@ __device__ __forceinline__ void st_once_u32(void* p, uint32_t v) {
                : "memory");
 }
 
-__device__ __forceinline__ unsigned long long ld_relaxed_u64_keep(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.L2::cache_hint.u64 %0, [%1], %2;"
-               : "=l"(v)
-               : "l"(p), "l"(l2_evict_last())
-               : "memory");
-  return v;
-}
-
 // The four slots of a sector (p 32-byte aligned), each a relaxed read of its own.
 __device__ __forceinline__ void ld_relaxed_u64x4_keep(const unsigned long long* p, unsigned long long (&w)[4]) {
   asm volatile("ld.relaxed.gpu.global.L2::cache_hint.v4.u64 {%0, %1, %2, %3}, [%4], %5;"
@@ -458,52 +449,6 @@ __device__ __forceinline__ uint32_t slot_fp(unsigned long long w) {
 }
 __device__ __forceinline__ uint32_t slot_id(unsigned long long w) {
   return static_cast<uint32_t>(w >> 32) - 1u;
-}
-
-// One probe step in the hashed table (Sec. 3.2, linear probing on the
-// fingerprint): `w` is the word read at the slot.  A slot holding f is a hit; an
-// empty slot is claimed with one 64-bit compare-and-swap that publishes the
-// fingerprint and the cell id together (so a reader never sees a fingerprint
-// without its cell); a slot holding another key moves the probe on.  Words are
-// only ever published, never changed, within a frame, so a key present in the
-// window is met before any empty slot.
-enum ProbeOutcome { kHit, kClaimed, kNext };
-
-__device__ __forceinline__ ProbeOutcome probe_step(unsigned long long* slot, unsigned long long w,
-                                                   uint32_t f, uint32_t my_id, uint32_t& id) {
-  if (w != 0ull) {
-    if (slot_fp(w) == f) {
-      id = slot_id(w);
-      return kHit;
-    }
-    return kNext;
-  }
-  const unsigned long long old = atomicCAS(slot, 0ull, slot_word(f, my_id));
-  if (old == 0ull) {
-    id = my_id;
-    return kClaimed;
-  }
-  if (slot_fp(old) == f) {
-    id = slot_id(old);
-    return kHit;
-  }
-  return kNext;
-}
-
-// The rest of a probe sequence, one step at a time, from step p0.  Returns the
-// slot (kOverflowSlot after P steps) and the cell id through `id`.
-__device__ __forceinline__ uint32_t probe_rest(const TableDev& t, uint32_t home, uint32_t f,
-                                               uint32_t p0, uint32_t my_id, uint32_t& id,
-                                               bool& claimed) {
-  claimed = false;
-  for (uint32_t p = p0; p < t.max_probes; ++p) {
-    const uint32_t s = (home + p) & t.mask;
-    const ProbeOutcome o = probe_step(t.slots + s, ld_relaxed_u64(t.slots + s), f, my_id, id);
-    if (o == kNext) continue;
-    claimed = o == kClaimed;
-    return s;
-  }
-  return kOverflowSlot;
 }
 
 // Read-only lookup of a key's cell id (query without a stored id), from

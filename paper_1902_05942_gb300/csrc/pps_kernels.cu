@@ -83,7 +83,7 @@ struct Counters {
 // 23 G/s otherwise), and only the vertices that met an existing cell (about
 // half) need an atomic, on lines written just before.  HD frame (5.06 M
 // vertices, 2^23 slots): insert and accumulation 191 us in one pass with an
-// atomic per vertex, 126 + 28 us in two; fixed point 293 us, 135 + 84 us.
+// atomic per vertex, 120 + 28 us in two; fixed point 293 us, 130 + 71 us.
 //
 // A warp inserts alone: no barrier and no shared counter between warps, so a
 // warp with long probe sequences holds up no other.  Every key's home slot
@@ -177,13 +177,16 @@ __device__ __forceinline__ void create_cell(const TableDev& t, uint32_t id, floa
 // and the colours read after the compare-and-swap took 8,140 us on the 61 M
 // vertex frame (load 0.7), this takes 7,855; 117.9 and 114.4 us on a 720p frame.
 // All lanes.
-template <int W>
+template <int W, bool KREC = false>
 __device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& v, WarpInsert<W>& s,
-                                           WarpShared& sh, bool rec, uint32_t* stash) {
+                                           WarpShared& sh, bool rec, uint32_t* stash,
+                                           uint4* qkw = nullptr) {
   const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
   const uint32_t take = min(32u, s.queued), at = s.queued - take, e = at + lane;
   const bool have = lane < take;
   uint32_t h1 = 0u, f = 0u, step = 0u, members = 0u, first = 0u;
+  uint4 kr{};
+  if (KREC && have) kr = qkw[e];
   if (have) {
     h1 = sh.h1[e];
     f = sh.f[e];
@@ -220,6 +223,7 @@ __device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& 
     if (owner) {
       id = s.my[0];
       create_cell(t, id, r, g, b, slot, h1, f, rec);
+      if (KREC) __stcg(t.kw + id, kr);
       ++s.cnt.cells;
       s.my[0] = kOverflowSlot;
     } else if (hit < 4u && slot_fp(a) == f) {
@@ -245,6 +249,7 @@ __device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& 
     sh.step[o] = step;
     sh.members[o] = members;
     sh.first[o] = first;
+    if (KREC) qkw[o] = kr;
   }
   s.queued = at + __popc(again);
   __syncwarp();
@@ -266,13 +271,14 @@ __device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& 
 // `rec`: write each new cell's record (t.info) for the later blend and clear;
 // a frame that neither blends nor clears slot by slot never reads it.
 // KV: the vertices may carry the key variants (distance, extra word).
-// KREC: also keep each new cell's quantized key in t.kw (such tables finish
-// every key on the spot).
+// KREC: also keep each new cell's quantized key in t.kw; `qkw` holds those of the
+// queued keys (finishing every key on the spot instead, a 1.6 M vertex frame with
+// migrating history took 229.7 us, with the queue 215.2).
 template <int W, bool KV, bool KREC>
 __device__ __forceinline__ void insert_warp(const KeyConst& kc, const TableDev& t,
                                             const VertexPtrs& v, size_t j0, size_t end,
                                             WarpInsert<W>& s, WarpShared& sh, bool rec, int merge,
-                                            uint32_t* stash) {
+                                            uint32_t* stash, uint4* qkw = nullptr) {
   const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
   uint32_t h1[W], f[W];
   uint4 kr[W];  // KREC: the quantized keys
@@ -343,22 +349,16 @@ __device__ __forceinline__ void insert_warp(const KeyConst& kc, const TableDev& 
     const size_t j = j0 + 32 * q + lane;
     uint32_t id = kDeferred, owner = 0u;
     if (lead >> q & 1u) {
-      uint32_t slot = h1[q] & t.mask;
-      bool won = old[q] == 0ull;
+      const uint32_t slot = h1[q] & t.mask;
+      const bool won = old[q] == 0ull;
       if (won)
         id = s.my[q];
       else if (slot_fp(old[q]) == f[q])
         id = slot_id(old[q]);
       else if (t.max_probes == 1u)
         id = kOverflowSlot;
-      if constexpr (KREC) {
-        if (id == kDeferred) {
-          id = kOverflowSlot;
-          slot = probe_rest(t, slot, f[q], 1u, s.my[q], id, won);
-        }
-        if (won) __stcg(t.kw + id, kr[q]);
-      }
       if (won) {
+        if (KREC) __stcg(t.kw + id, kr[q]);
         create_cell(t, id, r[q], g[q], b[q], slot, h1[q], f[q], rec);
         owner = kOwnerBit;
         ++s.cnt.cells;
@@ -368,21 +368,20 @@ __device__ __forceinline__ void insert_warp(const KeyConst& kc, const TableDev& 
     }
     const uint32_t mine = __shfl_sync(0xFFFFFFFFu, id, __ffs(grp[q]) - 1);
     if (j < end && mine != kDeferred) st_once_u32(stash + j, mine | owner);
-    if constexpr (!KREC) {
-      const unsigned put = __ballot_sync(0xFFFFFFFFu, (lead >> q & 1u) && id == kDeferred);
-      if (put) {
-        if (put >> lane & 1u) {
-          const uint32_t o = s.queued + __popc(put & lt);
-          sh.h1[o] = h1[q];
-          sh.f[o] = f[q];
-          sh.step[o] = 1u;
-          sh.members[o] = grp[q];
-          sh.first[o] = static_cast<uint32_t>(j0 + 32 * q);
-        }
-        s.queued += __popc(put);
-        __syncwarp();
-        while (s.queued > kQueue - 32) queue_step<W>(t, v, s, sh, rec, stash);
+    const unsigned put = __ballot_sync(0xFFFFFFFFu, (lead >> q & 1u) && id == kDeferred);
+    if (put) {
+      if (put >> lane & 1u) {
+        const uint32_t o = s.queued + __popc(put & lt);
+        sh.h1[o] = h1[q];
+        sh.f[o] = f[q];
+        sh.step[o] = 1u;
+        sh.members[o] = grp[q];
+        sh.first[o] = static_cast<uint32_t>(j0 + 32 * q);
+        if (KREC) qkw[o] = kr[q];
       }
+      s.queued += __popc(put);
+      __syncwarp();
+      while (s.queued > kQueue - 32) queue_step<W, KREC>(t, v, s, sh, rec, stash, qkw);
     }
   }
 }
@@ -790,7 +789,9 @@ __global__ void __launch_bounds__(kBlock) k_insert(KeyConst kc, TableDev t, Vert
                                                    size_t n, uint32_t* stash, uint32_t tile_base,
                                                    int merge) {
   __shared__ WarpShared s_warp[kBlock / 32];
+  __shared__ uint4 s_kw[KREC ? kBlock / 32 : 1][kQueue];
   WarpShared& sh = s_warp[threadIdx.x >> 5];
+  uint4* qkw = s_kw[KREC ? threadIdx.x >> 5 : 0];
   WarpInsert<W> s;
   const uint32_t tiles = static_cast<uint32_t>((n + kTile - 1) / kTile);
   for (uint32_t tile = grid_warp(); tile < tiles; tile += grid_warps()) {
@@ -800,9 +801,9 @@ __global__ void __launch_bounds__(kBlock) k_insert(KeyConst kc, TableDev t, Vert
     s.id_base = tix * kTileIds;
 #pragma unroll 1
     for (size_t j0 = t0; j0 < end; j0 += 32 * W)
-      insert_warp<W, true, KREC>(kc, t, v, j0, end, s, sh, true, merge, stash);
+      insert_warp<W, true, KREC>(kc, t, v, j0, end, s, sh, true, merge, stash, qkw);
     if (tile + grid_warps() >= tiles)  // the warp's last
-      while (s.queued) queue_step<W>(t, v, s, sh, true, stash);
+      while (s.queued) queue_step<W, KREC>(t, v, s, sh, true, stash, qkw);
     if ((threadIdx.x & 31u) == 0u) t.bcount[tix] = s.claims;
   }
   s.retire(t, true);
