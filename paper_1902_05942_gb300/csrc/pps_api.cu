@@ -196,6 +196,10 @@ int batch_of(const pps_table* t) { return t->tune.batch == 4 ? 4 : 2; }
 
 int merge_of(const pps_table* t) { return t->tune.merge ? static_cast<int>(t->tune.merge) : 2; }
 
+// Plain and temporal frames on tables up to this size have always been inserted
+// from the end of the stream, the others from its start (add_ordered).
+constexpr uint32_t kBackwards = 1u << 23;
+
 // Empty the slot table: of the split path's frame, or of what a persistent
 // launch left.
 int empty_slots(pps_table* t, cudaStream_t st) {
@@ -545,6 +549,7 @@ int filter_one(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_ve
   plan.evict = t->dev.hist_evict != 0;
   plan.neigh = t->dev.neighbors != 0;
   plan.kv = v->dist || v->extra;
+  if (blend) plan.order = pps::add_order(t->dev, t->T <= kBackwards && !plan.evict && !plan.neigh && !plan.kv);
   plan.sweep = n && pps::sweep_pays_host(t->dev, n);
   if (int rc = reset_slots(t, plan.sweep, st)) return rc;
   set_camera(t, cam, frame);

@@ -34,6 +34,7 @@ struct pps_batch {
   std::vector<uint32_t> index;      // of their cameras
   uint32_t total_tiles = 0;
   bool temporal = false;
+  bool ordered = false;  // a view of the shared launch adds its contributions up in order
   float alpha = 0.f;
   pps::MultiPlan plan;
   pps::ViewDesc* dviews[2] = {nullptr, nullptr};
@@ -105,15 +106,18 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
     vd.n = v.n;
     vd.blended = blend && tmp ? 1 : 0;
     vd.sweep = pps::sweep_pays_host(vd.t, v.n) ? 1 : 0;
+    vd.ordered = vd.blended && pps::add_order(vd.t, false) != pps::kAnyOrder ? 1 : 0;
     if (v.n >= kOwnLaunch) {
       pps::FusedPlan plan;
       plan.merge = 2;
       plan.temporal = vd.blended != 0;
       plan.sweep = vd.sweep != 0;
+      if (vd.ordered) plan.order = pps::kPairsForwards;
       b->own.push_back(pps_batch::OwnView{i, vd, plan});
       own_words = std::max<size_t>(own_words, v.n);
     } else {
       b->temporal = b->temporal || tmp;
+      b->ordered = b->ordered || vd.ordered;
       total += v.n;
       b->base.push_back(vd);
       b->index.push_back(i);
@@ -159,7 +163,7 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
     e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->dviews[k], b->hviews[k], bytes, cudaMemcpyHostToDevice, cs);
     if (e == cudaSuccess)
-      e = pps::launch_multi(b->dviews[k], nshared, b->total_tiles, b->ctrl, b->temporal, alpha,
+      e = pps::launch_multi(b->dviews[k], nshared, b->total_tiles, b->ctrl, b->temporal, b->ordered, alpha,
                             b->plan, b->gstash, cs);
     cudaError_t e2 = cudaStreamEndCapture(cs, &g);
     if (e == cudaSuccess) e = e2;

@@ -59,11 +59,12 @@ struct Ctrl {
   unsigned long long vertices;
   unsigned long long hist_overflow;
   unsigned long long neigh_count;  // persistent kernel: low-count vertices queued for the search
+  unsigned long long tile_next;    // ordered additions: next tile to hand out
   unsigned int error;
   unsigned int bar_count;
   unsigned int pad[2];
 };
-constexpr size_t kCtrlFrameBytes = 5 * sizeof(unsigned long long);  // reset per frame
+constexpr size_t kCtrlFrameBytes = 6 * sizeof(unsigned long long);  // reset per frame
 constexpr size_t kCtrlErrorBytes = 2 * sizeof(unsigned int);        // error word and barrier, from `error` on
 
 enum : unsigned int {
@@ -802,6 +803,7 @@ __device__ __forceinline__ void reset_counters(Ctrl* c) {
   c->vertices = 0ull;
   c->hist_overflow = 0ull;
   c->neigh_count = 0ull;
+  c->tile_next = 0ull;
 }
 
 // Barrier over all CTAs of a cooperative launch, sense-reversing (Mellor-Crummey

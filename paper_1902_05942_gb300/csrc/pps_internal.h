@@ -12,6 +12,14 @@ struct pps_params;
 
 namespace pps {
 
+// The order in which pass two of the insert adds contributions up (add_ordered
+// in pps_kernels.cu says why).
+enum AddOrder : int {
+  kAnyOrder = 0,       // no order: the sums' FP32 rounding may take any of its values
+  kRowsBackwards = 1,  // rows of 32 vertices, from the end of the stream
+  kPairsForwards = 2,  // pairs of neighbouring vertices, from its start
+};
+
 // Launch geometry of the persistent filter kernel for one call.
 struct FusedPlan {
   int grid = 0;       // CTAs
@@ -24,6 +32,7 @@ struct FusedPlan {
   bool kv = false;        // ... vertices with key variants
   bool sweep = false;     // zero the whole slot table first, not the frame's slots at the end
   int merge = 2;      // merging of equal keys within a warp (pps_tuning.merge)
+  AddOrder order = kAnyOrder;
 };
 
 // One view of a batched launch: its table, key constants, vertices and
@@ -38,6 +47,7 @@ struct ViewDesc {
   uint32_t ntiles;
   int blended;  // blend this view's cells (temporal table and blending requested)
   int sweep;    // zero this view's slot table by a sweep at the end
+  int ordered;  // add contributions up in the order of kPairsForwards
 };
 
 struct MultiPlan {
@@ -52,8 +62,11 @@ struct MultiPlan {
 cudaError_t plan_multi(size_t total_tiles, uint32_t tile, bool temporal, int batch, int block,
                        MultiPlan* plan);
 cudaError_t launch_multi(const ViewDesc* views, uint32_t nviews, uint32_t total_tiles, Ctrl* ctrl,
-                         bool temporal, float alpha, const MultiPlan& plan, uint32_t* stash,
-                         cudaStream_t st);
+                         bool temporal, bool ordered, float alpha, const MultiPlan& plan,
+                         uint32_t* stash, cudaStream_t st);
+// The additions' order on frames of table t that are blended (`backwards`: ones
+// whose contributions have always been added up from the end of the stream).
+AddOrder add_order(const TableDev& t, bool backwards);
 bool sweep_pays_host(const TableDev& t, size_t vertices);
 
 cudaError_t launch_insert(const KeyConst& kc, const TableDev& t, const VertexPtrs& v, size_t n,

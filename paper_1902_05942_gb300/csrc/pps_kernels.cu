@@ -157,11 +157,16 @@ struct WarpInsert {
   }
 };
 
-// A new cell `id`: its creator's contribution is its first, and (`rec`) its
-// record {slot, home hash, fingerprint}.
+// A new cell `id`: its creator's contribution is its first (own = 0: none is,
+// pass two adds them all), and (`rec`) its record {slot, home hash,
+// fingerprint}.
 __device__ __forceinline__ void create_cell(const TableDev& t, uint32_t id, float r, float g, float b,
-                                            uint32_t slot, uint32_t h1, uint32_t f, bool rec) {
-  if (!t.fixed) {
+                                            uint32_t slot, uint32_t h1, uint32_t f, bool rec,
+                                            uint32_t own) {
+  if (!own) {
+    __stcg(value_ptr(t, id), make_float4(0.f, 0.f, 0.f, 0.f));
+    if (t.fixed) __stcg(value_ptr(t, id) + 1, make_float4(0.f, 0.f, 0.f, 0.f));
+  } else if (!t.fixed) {
     __stcg(t.acc + id, make_float4(r, g, b, 1.0f));
   } else {
     ulonglong2* a = reinterpret_cast<ulonglong2*>(t.acc64 + 4 * static_cast<size_t>(id));
@@ -186,7 +191,7 @@ __device__ __forceinline__ void create_cell(const TableDev& t, uint32_t id, floa
 // All lanes.
 template <int W, bool KREC = false>
 __device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& v, WarpInsert<W>& s,
-                                           WarpShared& sh, bool rec, uint32_t* stash,
+                                           WarpShared& sh, bool rec, uint32_t own, uint32_t* stash,
                                            uint4* qkw = nullptr) {
   const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
   const uint32_t take = min(32u, s.queued), at = s.queued - take, e = at + lane;
@@ -218,18 +223,18 @@ __device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& 
     step += hit - o;
     const uint32_t slot = slot0 - o + hit;
     const uint32_t lead = first + __ffs(members) - 1;
-    uint32_t owner = 0u;
+    bool made = false;
     float r = 0.f, g = 0.f, b = 0.f;
     if (a == 0ull) {
       a = atomicCAS(t.slots + slot, 0ull, slot_word(f, s.my[0]));
-      if (a == 0ull) owner = kOwnerBit;
+      made = a == 0ull;
       r = __ldg(v.r + lead);
       g = __ldg(v.g + lead);
       b = __ldg(v.b + lead);
     }
-    if (owner) {
+    if (made) {
       id = s.my[0];
-      create_cell(t, id, r, g, b, slot, h1, f, rec);
+      create_cell(t, id, r, g, b, slot, h1, f, rec, own);
       if (KREC) __stcg(t.kw + id, kr);
       ++s.cnt.cells;
       s.my[0] = kOverflowSlot;
@@ -243,7 +248,7 @@ __device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& 
       }
     }
     if (id != kDeferred) {
-      st_once_u32(stash + lead, id | owner);
+      st_once_u32(stash + lead, made ? id | own : id);
       for (uint32_t m = members & (members - 1u); m; m &= m - 1u)
         st_once_u32(stash + first + __ffs(m) - 1, id);
     }
@@ -277,6 +282,7 @@ __device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& 
 //
 // `rec`: write each new cell's record (t.info) for the later blend and clear;
 // a frame that neither blends nor clears slot by slot never reads it.
+// `own`: kOwnerBit, or 0 on frames whose contributions all wait for pass two.
 // KV: the vertices may carry the key variants (distance, extra word).
 // KREC: also keep each new cell's quantized key in t.kw; `qkw` holds those of the
 // queued keys (finishing every key on the spot instead, a 1.6 M vertex frame with
@@ -284,8 +290,8 @@ __device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& 
 template <int W, bool KV, bool KREC>
 __device__ __forceinline__ void insert_warp(const KeyConst& kc, const TableDev& t,
                                             const VertexPtrs& v, size_t j0, size_t end,
-                                            WarpInsert<W>& s, WarpShared& sh, bool rec, int merge,
-                                            uint32_t* stash, uint4* qkw = nullptr) {
+                                            WarpInsert<W>& s, WarpShared& sh, bool rec, uint32_t own,
+                                            int merge, uint32_t* stash, uint4* qkw = nullptr) {
   const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
   uint32_t h1[W], f[W];
   uint4 kr[W];  // KREC: the quantized keys
@@ -372,8 +378,8 @@ __device__ __forceinline__ void insert_warp(const KeyConst& kc, const TableDev& 
         id = kOverflowSlot;
       if (won) {
         if (KREC) __stcg(t.kw + id, kr[q]);
-        create_cell(t, id, r[q], g[q], b[q], slot, h1[q], f[q], rec);
-        owner = kOwnerBit;
+        create_cell(t, id, r[q], g[q], b[q], slot, h1[q], f[q], rec, own);
+        owner = own;
         ++s.cnt.cells;
         s.my[q] = kOverflowSlot;
       }
@@ -394,29 +400,29 @@ __device__ __forceinline__ void insert_warp(const KeyConst& kc, const TableDev& 
       }
       s.queued += __popc(put);
       __syncwarp();
-      while (s.queued > kQueue - 32) queue_step<W, KREC>(t, v, s, sh, rec, stash, qkw);
+      while (s.queued > kQueue - 32) queue_step<W, KREC>(t, v, s, sh, rec, own, stash, qkw);
     }
   }
 }
 
-// Pass two for the 128 vertices from j0 on (those below `end`), one warp, four
-// rows of 32: the contributions of the vertices that do not own their cells.
-// Neighbouring vertices of the same cell are added up first, as in pass one.
-template <bool FIXED>
+// Pass two for W rows of 32 vertices from j0 on, STEP apart (those below
+// `end`), one warp: the contributions of the vertices that do not own their
+// cells.  Neighbouring vertices of the same cell are added up first, as in pass
+// one.
+template <bool FIXED, int W = 4, int STEP = 32>
 __device__ __forceinline__ void add_warp_as(const TableDev& t, const VertexPtrs& v, size_t j0, size_t end,
                                             const uint32_t* stash, int merge, WarpShared& sh) {
   const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
-  constexpr int W = 4;
   uint32_t id[W];
   float r[W], g[W], b[W];
 #pragma unroll
   for (int q = 0; q < W; ++q) {
-    const size_t j = j0 + 32 * q + lane;
+    const size_t j = j0 + STEP * q + lane;
     id[q] = j < end ? __ldcg(stash + j) : kOverflowSlot;
   }
 #pragma unroll
   for (int q = 0; q < W; ++q) {
-    const size_t j = j0 + 32 * q + lane;
+    const size_t j = j0 + STEP * q + lane;
     if (!(id[q] & kOwnerBit)) {  // neither an owner nor overflowed
       r[q] = __ldcs(v.r + j);
       g[q] = __ldcs(v.g + j);
@@ -471,6 +477,31 @@ __device__ __forceinline__ void add_warp(const TableDev& t, const VertexPtrs& v,
     add_warp_as<true>(t, v, j0, end, stash, merge, sh);
   else
     add_warp_as<false>(t, v, j0, end, stash, merge, sh);
+}
+
+// Pass two for two neighbouring vertices per lane, j and j + 1 (those below
+// `end`), FP32: equal cells' contributions are added up first.
+__device__ __forceinline__ void add_pairs(const TableDev& t, const VertexPtrs& v, size_t j, size_t end,
+                                          const uint32_t* stash) {
+  uint32_t id[2];
+  float r[2], g[2], b[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) id[q] = j + q < end ? __ldcg(stash + j + q) : kOverflowSlot;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    if (id[q] & kOwnerBit) continue;  // overflowed
+    r[q] = __ldcs(v.r + j + q);
+    g[q] = __ldcs(v.g + j + q);
+    b[q] = __ldcs(v.b + j + q);
+  }
+  const bool both = !(id[0] & kOwnerBit) && id[0] == id[1];
+  if (both) {
+    r[0] = __fadd_rn(r[0], r[1]);
+    g[0] = __fadd_rn(g[0], g[1]);
+    b[0] = __fadd_rn(b[0], b[1]);
+  }
+  if (!(id[0] & kOwnerBit)) accumulate<false>(t, id[0], r[0], g[0], b[0], 0, 0, 0, both ? 2u : 1u);
+  if (!(id[1] & kOwnerBit) && !both) accumulate<false>(t, id[1], r[1], g[1], b[1], 0, 0, 0, 1u);
 }
 
 // The cell id of a stash word (kOverflowSlot: probe overflow).
@@ -800,7 +831,7 @@ __device__ __forceinline__ void sweep_slots(const TableDev& t, size_t gid, size_
 template <int W, bool KREC>
 __global__ void __launch_bounds__(kBlock) k_insert(KeyConst kc, TableDev t, VertexPtrs v,
                                                    size_t n, uint32_t* stash, uint32_t tile_base,
-                                                   int merge) {
+                                                   uint32_t own, int merge) {
   __shared__ WarpShared s_warp[kBlock / 32];
   __shared__ uint4 s_kw[KREC ? kBlock / 32 : 1][kQueue];
   WarpShared& sh = s_warp[threadIdx.x >> 5];
@@ -814,9 +845,9 @@ __global__ void __launch_bounds__(kBlock) k_insert(KeyConst kc, TableDev t, Vert
     s.id_base = tix * kTileIds;
 #pragma unroll 1
     for (size_t j0 = t0; j0 < end; j0 += 32 * W)
-      insert_warp<W, true, KREC>(kc, t, v, j0, end, s, sh, true, merge, stash, qkw);
+      insert_warp<W, true, KREC>(kc, t, v, j0, end, s, sh, true, own, merge, stash, qkw);
     if (tile + grid_warps() >= tiles)  // the warp's last
-      while (s.queued) queue_step<W, KREC>(t, v, s, sh, true, stash, qkw);
+      while (s.queued) queue_step<W, KREC>(t, v, s, sh, true, own, stash, qkw);
     if ((threadIdx.x & 31u) == 0u) t.bcount[tix] = s.claims;
   }
   s.retire(t, true);
@@ -830,10 +861,22 @@ __global__ void __launch_bounds__(kBlock) k_insert(KeyConst kc, TableDev t, Vert
 }
 
 // Pass two; id_out (nullable): the vertices' cell ids for the caller.
-__global__ void __launch_bounds__(kBlock) k_add(TableDev t, VertexPtrs v, size_t n,
-                                                const uint32_t* stash, uint32_t* id_out, int merge) {
+// `ordered`: all contributions in the order of kPairsForwards, in tiles of 1,024
+// vertices, four to a thread.
+__global__ void __launch_bounds__(kBlock) k_add(TableDev t, VertexPtrs v, size_t n, const uint32_t* stash,
+                                                uint32_t* id_out, int ordered, int merge) {
   __shared__ WarpShared s_warp[kBlock / 32];
   const uint32_t lane = threadIdx.x & 31u;
+  if (ordered) {
+    for (size_t t0 = blockIdx.x * static_cast<size_t>(4 * kBlock); t0 < n; t0 += gridDim.x * static_cast<size_t>(4 * kBlock)) {
+      const size_t j0 = t0 + 4 * threadIdx.x;
+      add_pairs(t, v, j0, n, stash);
+      add_pairs(t, v, j0 + 2, n, stash);
+      if (id_out)
+        for (size_t j = j0; j < min(n, j0 + 4); ++j) id_out[j] = stash_id(stash[j]);
+    }
+    return;
+  }
   for (size_t j0 = grid_warp() * static_cast<size_t>(128); j0 < n; j0 += grid_warps() * static_cast<size_t>(128)) {
     add_warp(t, v, j0, n, stash, merge, s_warp[threadIdx.x >> 5]);
     if (id_out)
@@ -1075,6 +1118,7 @@ struct FusedArgs {
   int sweep;         // zero the whole slot table first, instead of the frame's slots at the end
   uint32_t* nq;      // neighborhood search: the queue of low-count vertices
   int merge;         // merging of equal keys within a warp (insert_warp)
+  int order;         // AddOrder of pass two
 };
 
 // The warp's list of low-count vertices (in its shared memory, the key queue's
@@ -1145,6 +1189,46 @@ __device__ __forceinline__ void lookup_warp(const TableDev& t, const VertexPtrs&
     if (queued > kLowList - 128u) flush_low(t, nq, sh, queued);
 }
 
+// Pass two of a frame whose half-precision history is blended (all threads):
+// nobody owns a cell, and tiles of 2,048 vertices are handed out from a counter,
+// in the order of FusedArgs::order and within a tile
+//   kRowsBackwards  1,024 vertices at a time, the rows of 32 of a warp 512 apart;
+//   kPairsForwards  1,024 vertices at a time, two neighbouring ones per lane,
+// which is about the order that frames of this kind have always been added up in:
+// one tile after the other, first or last part of the stream first.  An FP32 sum
+// depends on the order of its additions in its last bit, and where the stored
+// average lies next to the middle of two halves, that bit moves it by a unit of
+// binary16, up to 9.8e-4 of the value, so for these histories a different
+// order is a visible difference: with the creator's contribution first and the
+// rest in any order, a frame of 1.66 M vertices had 33,300 cells with another
+// sum than the insert in one pass gave, in this order 12,000, and 11,400 from
+// one run of that insert to the next; of 61 M vertices (2^26 slots) 364,000,
+// 74,000 and 44,000.  It costs 4 and 340 us there (111.6 and 8,660 us a frame).
+__device__ __forceinline__ void add_ordered(const FusedArgs& a, WarpShared& sh) {
+  constexpr uint32_t kHalf = 1024, kSpan = 2 * kHalf;
+  static_assert(kFusedBlock == 512, "two rows, or one row of pairs, per warp and half tile");
+  __shared__ uint32_t s_next;
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+  const uint32_t ntiles = static_cast<uint32_t>((a.n + kSpan - 1) / kSpan);
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_next = static_cast<uint32_t>(atomicAdd(&a.t.ctrl->tile_next, 1ull));
+    __syncthreads();
+    const uint32_t k = s_next;
+    if (k >= ntiles) return;
+    const bool back = a.order == kRowsBackwards;
+    const size_t t0 = static_cast<size_t>(back ? ntiles - 1u - k : k) * kSpan;
+    for (uint32_t c = 0; c < kSpan; c += kHalf) {
+      if (back) {
+        add_warp_as<false, 2, kFusedBlock>(a.t, a.v, t0 + c + 32 * warp, a.n, a.stash, a.merge, sh);
+        __syncthreads();
+      } else {
+        add_pairs(a.t, a.v, t0 + c + 64 * warp + 2 * lane, a.n, a.stash);
+      }
+    }
+  }
+}
+
 // The persistent kernel.  Every phase is a loop of independent warps:
 //   0   the slot table is emptied (sweep), just before it is filled, so that
 //       the compare-and-swaps meet it in L2;
@@ -1153,7 +1237,7 @@ __device__ __forceinline__ void lookup_warp(const TableDev& t, const VertexPtrs&
 //       balances: its atomics serialize on one address, HD 146 us against 126);
 //       a tile's new cells take ids from the tile's own range, and each
 //       vertex's cell id goes to the stash;
-//   A2  accumulation (128 vertices at a time);
+//   A2  accumulation (128 vertices at a time, or in order: add_ordered);
 //   B   temporal blend of each tile's new cells;
 //   C   one lookup per vertex (128 at a time); a frame that did not sweep
 //       empties its slots,
@@ -1178,6 +1262,7 @@ __global__ void __launch_bounds__(kFusedBlock, W == 4 ? 1 : 2) k_fused(FusedArgs
   {
     WarpInsert<W> s;
     const bool rec = blended || !a.sweep;
+    const uint32_t own = TEMPORAL && a.order ? 0u : kOwnerBit;
     for (uint32_t k = gw; k < ntiles; k += nw) {
       // from the end of the vertex stream: streams are bounce-major, so the
       // secondary-bounce tiles, whose vertices nearly all create cells of
@@ -1190,9 +1275,9 @@ __global__ void __launch_bounds__(kFusedBlock, W == 4 ? 1 : 2) k_fused(FusedArgs
       s.id_base = tile * tile_i;
 #pragma unroll 1
       for (size_t j0 = t0; j0 < end; j0 += 32 * W)
-        insert_warp<W, KV, false>(a.kc, t, a.v, j0, end, s, sh, rec, a.merge, a.stash);
+        insert_warp<W, KV, false>(a.kc, t, a.v, j0, end, s, sh, rec, own, a.merge, a.stash);
       if (k + nw >= ntiles)  // the warp's last tile
-        while (s.queued) queue_step<W>(t, a.v, s, sh, rec, a.stash);
+        while (s.queued) queue_step<W>(t, a.v, s, sh, rec, own, a.stash);
       if (lane == 0) __stcg(t.bcount + tile, s.claims);
     }
     s.retire(t, rec);
@@ -1206,8 +1291,11 @@ __global__ void __launch_bounds__(kFusedBlock, W == 4 ? 1 : 2) k_fused(FusedArgs
     if (blockIdx.x == 0) atomicAdd(&t.ctrl->vertices, static_cast<unsigned long long>(a.n));
   }
 
-  for (size_t j = gw * static_cast<size_t>(128); j < a.n; j += nw * static_cast<size_t>(128))
-    add_warp(t, a.v, j, a.n, a.stash, a.merge, sh);
+  if (TEMPORAL && a.order)
+    add_ordered(a, sh);
+  else
+    for (size_t j = gw * static_cast<size_t>(128); j < a.n; j += nw * static_cast<size_t>(128))
+      add_warp(t, a.v, j, a.n, a.stash, a.merge, sh);
   if (!grid_barrier(t.ctrl, gridDim.x)) return;
 
   if (blended) {
@@ -1238,6 +1326,7 @@ struct MultiArgs {
   uint32_t* stash;  // indexed by tile, tile_v words each
   uint32_t nviews, total_tiles, tile_v;
   float alpha;
+  int ordered;  // a view adds its contributions up in order
 };
 
 // The warp's copy of the descriptor of the view that tile gt belongs to;
@@ -1270,6 +1359,7 @@ __global__ void __launch_bounds__(BLOCK, (W == 4 ? 1 : 2) * (kFusedBlock / BLOCK
 
   if (threadIdx.x == 0)
     for (uint32_t v = blockIdx.x; v < a.nviews; v += gridDim.x) reset_counters(a.views[v].t.ctrl);
+  if (blockIdx.x == 0 && threadIdx.x == 0) reset_counters(a.ctrl);
   // empty the slot tables of the views that are swept
   for (uint32_t v = 0; v < a.nviews; ++v) {
     take_view(&vd, a, __ldg(&a.views[v].tile_base), cur);
@@ -1284,8 +1374,9 @@ __global__ void __launch_bounds__(BLOCK, (W == 4 ? 1 : 2) * (kFusedBlock / BLOCK
     WarpInsert<W> s;
     uint32_t last = 0u;  // the last tile worked on
     auto ids = [&]() { return a.stash + static_cast<size_t>(vd.tile_base) * tile_v; };
+    auto own = [&]() { return TEMPORAL && vd.ordered ? 0u : kOwnerBit; };
     auto flush = [&]() {  // leave the view in vd
-      while (s.queued) queue_step<W>(vd.t, vd.v, s, sh, true, ids());
+      while (s.queued) queue_step<W>(vd.t, vd.v, s, sh, true, own(), ids());
       if (lane == 0) __stcg(vd.t.bcount + last, s.claims);
       unsigned long long o = s.cnt.ovf, c = s.cnt.cells;
       for (int off = 16; off > 0; off >>= 1) {
@@ -1309,7 +1400,7 @@ __global__ void __launch_bounds__(BLOCK, (W == 4 ? 1 : 2) * (kFusedBlock / BLOCK
       s.id_base = last * tile_i;
 #pragma unroll 1
       for (size_t j0 = t0; j0 < end; j0 += 32 * W)
-        insert_warp<W, false, false>(vd.kc, vd.t, vd.v, j0, end, s, sh, true, 2, ids());
+        insert_warp<W, false, false>(vd.kc, vd.t, vd.v, j0, end, s, sh, true, own(), 2, ids());
       if (lane == 0) __stcg(vd.t.bcount + last, s.claims);
     }
     if (cur != kOverflowSlot) flush();
@@ -1319,12 +1410,30 @@ __global__ void __launch_bounds__(BLOCK, (W == 4 ? 1 : 2) * (kFusedBlock / BLOCK
   }
   if (!grid_barrier(a.ctrl, gridDim.x)) return;
 
-  for (uint32_t gt = run0; gt < run1; ++gt) {
+  auto add_tile = [&](uint32_t gt) {
     take_view(&vd, a, gt, cur);
     const size_t t0 = static_cast<size_t>(gt - vd.tile_base) * tile_v;
     const size_t end = min(static_cast<size_t>(vd.n), t0 + tile_v);
-    for (size_t j = t0; j < end; j += 128)
-      add_warp(vd.t, vd.v, j, end, a.stash + static_cast<size_t>(vd.tile_base) * tile_v, 2, sh);
+    const uint32_t* ids = a.stash + static_cast<size_t>(vd.tile_base) * tile_v;
+    if (TEMPORAL && vd.ordered)
+      for (size_t j = t0; j < end; j += 64) add_pairs(vd.t, vd.v, j + 2 * lane, end, ids);
+    else
+      for (size_t j = t0; j < end; j += 128) add_warp(vd.t, vd.v, j, end, ids, 2, sh);
+  };
+  if (TEMPORAL && a.ordered) {
+    // as in add_ordered, forwards, a tile per warp
+    __shared__ uint32_t s_next;
+    for (;;) {
+      __syncthreads();
+      if (threadIdx.x == 0) s_next = static_cast<uint32_t>(atomicAdd(&a.ctrl->tile_next, 1ull));
+      __syncthreads();
+      const uint64_t first = static_cast<uint64_t>(s_next) * (BLOCK / 32);
+      if (first >= a.total_tiles) break;
+      const uint64_t gt = first + (threadIdx.x >> 5);
+      if (gt < a.total_tiles) add_tile(static_cast<uint32_t>(gt));
+    }
+  } else {
+    for (uint32_t gt = run0; gt < run1; ++gt) add_tile(gt);
   }
   if (!grid_barrier(a.ctrl, gridDim.x)) return;
 
@@ -1411,17 +1520,20 @@ cudaError_t launch_insert(const KeyConst& kc, const TableDev& t, const VertexPtr
                           cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   const int grid = split_grid((n + kTile - 1) / kTile * 32);
+  const bool ordered = add_order(t, false) != kAnyOrder;
+  const uint32_t own = ordered ? 0u : kOwnerBit;
   if (t.hist_migrate || t.normal_search) {  // keep each new cell's quantized key
     if (batch == 2)
-      k_insert<2, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, merge);
+      k_insert<2, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, own, merge);
     else
-      k_insert<4, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, merge);
+      k_insert<4, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, own, merge);
   } else if (batch == 2) {
-    k_insert<2, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, merge);
+    k_insert<2, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, own, merge);
   } else {
-    k_insert<4, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, merge);
+    k_insert<4, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, own, merge);
   }
-  k_add<<<split_grid((n + 127) / 128 * 32), kBlock, 0, st>>>(t, v, n, stash, id_out, merge);
+  k_add<<<split_grid((n + 127) / 128 * 32), kBlock, 0, st>>>(t, v, n, stash, id_out, ordered ? 1 : 0,
+                                                            merge);
   return cudaGetLastError();
 }
 
@@ -1593,6 +1705,7 @@ cudaError_t launch_fused(const KeyConst& kc, const TableDev& t, const VertexPtrs
   a.sweep = plan.sweep ? 1 : 0;
   a.nq = nq;
   a.merge = plan.merge;
+  a.order = plan.order;
   void* args[] = {&a};
   cudaError_t e = cudaLaunchCooperativeKernel(fused_kernel(plan), dim3(plan.grid), dim3(plan.block), args,
                                               0, st);
@@ -1604,6 +1717,11 @@ cudaError_t launch_fused(const KeyConst& kc, const TableDev& t, const VertexPtrs
         t, ntiles, tile_ids(plan.tile, plan.batch), 0);
   }
   return cudaGetLastError();
+}
+
+AddOrder add_order(const TableDev& t, bool backwards) {
+  if (t.hist_mode != 2 || t.fixed) return kAnyOrder;
+  return backwards ? kRowsBackwards : kPairsForwards;
 }
 
 bool sweep_pays_host(const TableDev& t, size_t vertices) { return sweep_pays(t, vertices); }
@@ -1630,8 +1748,8 @@ cudaError_t plan_multi(size_t total_tiles, uint32_t tile, bool temporal, int bat
 }
 
 cudaError_t launch_multi(const ViewDesc* views, uint32_t nviews, uint32_t total_tiles, Ctrl* ctrl,
-                         bool temporal, float alpha, const MultiPlan& plan, uint32_t* stash,
-                         cudaStream_t st) {
+                         bool temporal, bool ordered, float alpha, const MultiPlan& plan,
+                         uint32_t* stash, cudaStream_t st) {
   MultiArgs a;
   a.views = views;
   a.ctrl = ctrl;
@@ -1640,6 +1758,7 @@ cudaError_t launch_multi(const ViewDesc* views, uint32_t nviews, uint32_t total_
   a.total_tiles = total_tiles;
   a.tile_v = plan.tile;
   a.alpha = alpha;
+  a.ordered = ordered ? 1 : 0;
   void* args[] = {&a};
   return cudaLaunchCooperativeKernel(multi_kernel(temporal, plan.batch, plan.block), dim3(plan.grid),
                                      dim3(plan.block), args, 0, st);
