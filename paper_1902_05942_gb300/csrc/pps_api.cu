@@ -597,8 +597,9 @@ int pps_filter(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_ve
     // history migration, similar normals: the split kernels; the insert's cell
     // ids (the stash, in place) spare the lookup its keys and probes
     const size_t tiles = (n + pps::tile_size() - 1) / pps::tile_size();
-    if (int rc = ensure_dense(t, tiles * pps::split_tile_ids(), 0, st)) return rc;
     if (int rc = pps_build(t, cam, frame, stream)) return rc;
+    // (only now: emptying the last frame's slots reads its cells' records)
+    if (int rc = ensure_dense(t, tiles * pps::split_tile_ids(), 0, st)) return rc;
     if (int rc = pps_insert(t, v, n, t->stash, stream)) return rc;
     if (blend)
       if (int rc = pps_blend(t, alpha, stream)) return rc;
