@@ -69,9 +69,9 @@ struct pps_table {
   pps_tuning tune{};         // launch shape (batch width 0 = library default)
   size_t D = 0;              // capacity of the dense cell arrays
   uint32_t* stash = nullptr;  // [D] the vertices' cell ids during a call
-  // The slots still hold the last frame of a persistent launch, which empties
-  // them before it uses them: nothing else may read them before empty_slots.
-  bool stale = false;
+  // A launch that leaves its frame in the slots has been made or captured on this
+  // table: whether they hold one now, Ctrl::left says.
+  bool leaves = false;
   uint32_t* neigh_q = nullptr;  // neighborhood search: queue of low-count vertices
   size_t neigh_q_cap = 0;
   void* stage = nullptr;  // pps_filter_host device staging
@@ -200,33 +200,21 @@ int merge_of(const pps_table* t) { return t->tune.merge ? static_cast<int>(t->tu
 // from the end of the stream, the others from its start (add_ordered).
 constexpr uint32_t kBackwards = 1u << 23;
 
-// Empty the slot table: of the split path's frame, or of what a persistent
-// launch left.
-int empty_slots(pps_table* t, cudaStream_t st) {
-  if (t->stale)
-    PPS_CUDA(cudaMemsetAsync(t->dev.slots, 0, t->T * sizeof(unsigned long long), st));
-  else if (t->state != kClean)
-    PPS_CUDA(pps::launch_clear(t->dev, t->frame_tiles, st));
-  t->stale = false;
-  return PPS_OK;
-}
-
-// Begin a frame: unless its launch empties the whole slot table itself
-// (`swept`), empty the slots.
-int reset_slots(pps_table* t, bool swept, cudaStream_t st) {
-  if (!swept) {
-    if (int rc = empty_slots(t, st)) return rc;
-  } else if (t->state != kClean) {
-    t->stale = true;
-  }
+// Empty the slots of the split path's frame.
+int empty_frame(pps_table* t, cudaStream_t st) {
+  if (t->state != kClean) PPS_CUDA(pps::launch_clear(t->dev, t->frame_tiles, st));
   t->frame_tiles = 0;
   t->state = kClean;
   return PPS_OK;
 }
 
-// The frame's counters to zero (a persistent launch does it itself).
-int reset_counters(pps_table* t, cudaStream_t st) {
-  PPS_CUDA(cudaMemsetAsync(t->dev.ctrl, 0, pps::kCtrlFrameBytes, st));
+// Begin a frame that no persistent launch begins: slots and counters emptied.
+int reset_frame(pps_table* t, cudaStream_t st) {
+  if (t->state == kClean && t->leaves)
+    PPS_CUDA(pps::launch_clear(t->dev, 0, st));
+  else if (int rc = empty_frame(t, st))
+    return rc;
+  PPS_CUDA(cudaMemsetAsync(t->dev.ctrl, 0, pps::kCtrlEmptyBytes, st));
   return PPS_OK;
 }
 
@@ -468,8 +456,7 @@ int pps_build(pps_table* t, const pps_camera* cam, uint32_t frame, void* stream)
   if (int rc = check_table(t)) return rc;
   if (!cam) return fail(PPS_EINVAL, "camera is NULL");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (int rc = reset_slots(t, false, st)) return rc;
-  if (int rc = reset_counters(t, st)) return rc;
+  if (int rc = reset_frame(t, st)) return rc;
   set_camera(t, cam, frame);
   t->state = kOpen;
   if (t->coarse) return pps_build(t->coarse, cam, frame, stream);
@@ -550,10 +537,11 @@ int filter_one(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_ve
   plan.neigh = t->dev.neighbors != 0;
   plan.kv = v->dist || v->extra;
   if (blend) plan.order = pps::add_order(t->dev, t->T <= kBackwards && !plan.evict && !plan.neigh && !plan.kv);
-  plan.sweep = n && pps::sweep_pays_host(t->dev, n);
-  if (int rc = reset_slots(t, plan.sweep, st)) return rc;
   set_camera(t, cam, frame);
-  if (n == 0) return reset_counters(t, st);
+  if (n == 0) return reset_frame(t, st);
+  plan.sweep = pps::sweep_pays_host(t->dev, n);
+  if (!plan.sweep)
+    if (int rc = empty_frame(t, st)) return rc;
   auto ready = [&]() -> int {
     PPS_CUDA(pps::plan_fused(n, ~size_t{0}, &plan));
     if (int rc = ensure_dense(t, pps::fused_cells(n, plan.tile, plan.batch), 0, st)) return rc;
@@ -569,14 +557,21 @@ int filter_one(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_ve
     }
     return blend ? next_epoch(t, st) : PPS_OK;
   };
-  if (int rc = ready()) {  // no launch to reset the counters
-    cudaMemsetAsync(t->dev.ctrl, 0, pps::kCtrlFrameBytes, st);
-    return rc;
+  auto launch = [&]() -> int {
+    if (int rc = ready()) return rc;
+    PPS_CUDA(pps::launch_fused(t->kc, t->dev, to_dev(v), n, out, blend != 0, alpha, plan, t->stash,
+                               t->neigh_q, st));
+    return PPS_OK;
+  };
+  const int rc = launch();
+  if (rc) {  // nothing empties the slots and resets the counters
+    cudaMemsetAsync(t->dev.slots, 0, t->T * sizeof(unsigned long long), st);
+    cudaMemsetAsync(t->dev.ctrl, 0, pps::kCtrlEmptyBytes, st);
   }
-  PPS_CUDA(pps::launch_fused(t->kc, t->dev, to_dev(v), n, out, blend != 0, alpha, plan, t->stash,
-                             t->neigh_q, st));
-  t->stale = plan.sweep;
-  return PPS_OK;
+  t->frame_tiles = 0;
+  t->state = kClean;
+  t->leaves = t->leaves || plan.sweep;
+  return rc;
 }
 
 }  // namespace
@@ -787,8 +782,7 @@ int table_for_batch(pps_table* t, size_t n, ViewDesc* vd, int* batch, int* block
                             "migration or normal search");
   // the batch's tile width and batch are not known yet: room for the widest id ranges
   if (int rc = ensure_dense(t, fused_cells(n, 64u, 4), 0, st)) return rc;
-  if (int rc = empty_slots(t, st)) return rc;
-  t->stale = true;  // until something else needs the slots, the batch's launches do as they like
+  t->leaves = true;
   vd->kc = t->kc;
   vd->t = t->dev;
   *batch = batch_of(t);
@@ -865,8 +859,11 @@ int pps_stats(pps_table* t, pps_stats_t* out, void* stream) {
   out->device_error = c.error;
   out->frame = t->kc.frame;
   if (c.error) {
-    // clear the error word and the barrier state so the table stays usable
+    // clear the error word and the barrier state so the table stays usable; the
+    // slots may hold anything
     PPS_CUDA(cudaMemsetAsync(&t->dev.ctrl->error, 0, pps::kCtrlErrorBytes, st));  // + barrier
+    PPS_CUDA(cudaMemsetAsync(&t->dev.ctrl->left, 1, sizeof(t->dev.ctrl->left), st));
+    t->leaves = true;
     PPS_CUDA(cudaStreamSynchronize(st));
     return fail(PPS_EDEVICE, pps::device_error_text(c.error));
   }

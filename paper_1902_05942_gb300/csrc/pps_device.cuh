@@ -60,11 +60,16 @@ struct Ctrl {
   unsigned long long hist_overflow;
   unsigned long long neigh_count;  // persistent kernel: low-count vertices queued for the search
   unsigned long long tile_next;    // ordered additions: next tile to hand out
+  // The slots still hold the frame of a launch that empties them before it uses
+  // them: the next launch that does not do so of itself has to.  It is kept here
+  // and not on the host, which does not see the launches of a replayed graph.
+  unsigned long long left;
   unsigned int error;
   unsigned int bar_count;
   unsigned int pad[2];
 };
-constexpr size_t kCtrlFrameBytes = 6 * sizeof(unsigned long long);  // reset per frame
+constexpr size_t kCtrlFrameBytes = 6 * sizeof(unsigned long long);  // the counters, reset per frame
+constexpr size_t kCtrlEmptyBytes = 7 * sizeof(unsigned long long);  // and `left`, once the slots are empty
 constexpr size_t kCtrlErrorBytes = 2 * sizeof(unsigned int);        // error word and barrier, from `error` on
 
 enum : unsigned int {

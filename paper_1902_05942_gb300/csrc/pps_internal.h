@@ -46,7 +46,7 @@ struct ViewDesc {
   uint32_t tile_base;  // first tile of this view in the batch
   uint32_t ntiles;
   int blended;  // blend this view's cells (temporal table and blending requested)
-  int sweep;    // zero this view's slot table by a sweep at the end
+  int sweep;    // zero this view's slot table by a sweep first
   int ordered;  // add contributions up in the order of kPairsForwards
 };
 
@@ -79,6 +79,8 @@ cudaError_t launch_keys(const KeyConst& kc, const VertexPtrs& v, size_t n, uint3
                         uint32_t* f_out, cudaStream_t st);
 cudaError_t launch_blend(const KeyConst& kc, const TableDev& t, uint32_t ntiles, float alpha,
                          cudaStream_t st);
+// Empty the slots: those of the split path's frame of `ntiles` tiles, or all of
+// them where a launch left its own (Ctrl::left, which the caller resets).
 cudaError_t launch_clear(const TableDev& t, uint32_t ntiles, cudaStream_t st);
 // Evicting history: lower every entry's priority by `by` (epoch rebase).
 cudaError_t launch_hist_age(const TableDev& t, uint32_t by, cudaStream_t st);

@@ -1070,7 +1070,7 @@ __global__ void __launch_bounds__(kBlock) k_neighbors(KeyConst kc, TableDev t, V
 
 __global__ void __launch_bounds__(kBlock) k_clear_sweep(TableDev t, uint32_t ntiles, uint32_t tile_i,
                                                         int sweep) {
-  if (sweep)
+  if (sweep || __ldcg(&t.ctrl->left))
     sweep_slots(t, blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x,
                 static_cast<size_t>(gridDim.x) * blockDim.x);
   else
@@ -1231,7 +1231,7 @@ __device__ __forceinline__ void add_ordered(const FusedArgs& a, WarpShared& sh) 
 
 // The persistent kernel.  Every phase is a loop of independent warps:
 //   0   the slot table is emptied (sweep), just before it is filled, so that
-//       the compare-and-swaps meet it in L2;
+//       the compare-and-swaps meet it in L2; so is what another launch left;
 //   A1  keys, probing insert, in tiles of a.tile_v vertices, every nw-th tile
 //       to one warp (a counter that hands them out costs more than it
 //       balances: its atomics serialize on one address, HD 146 us against 126);
@@ -1252,7 +1252,7 @@ __global__ void __launch_bounds__(kFusedBlock, W == 4 ? 1 : 2) k_fused(FusedArgs
   const uint32_t gw = grid_warp(), nw = grid_warps();
   const bool blended = TEMPORAL && a.blend;
   if (blockIdx.x == 0 && threadIdx.x == 0) reset_counters(t.ctrl);
-  if (a.sweep) {
+  if (a.sweep || __ldcg(&t.ctrl->left)) {  // (the same answer in every CTA: it changes after the next barrier)
     sweep_slots(t, blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x,
                 static_cast<size_t>(gridDim.x) * blockDim.x);
     if (!grid_barrier(t.ctrl, gridDim.x)) return;
@@ -1288,7 +1288,10 @@ __global__ void __launch_bounds__(kFusedBlock, W == 4 ? 1 : 2) k_fused(FusedArgs
   if (threadIdx.x == 0) {
     if (n_ovf) atomicAdd(&t.ctrl->overflow_vertices, n_ovf);
     if (n_cells) atomicAdd(&t.ctrl->frame_cells, n_cells);
-    if (blockIdx.x == 0) atomicAdd(&t.ctrl->vertices, static_cast<unsigned long long>(a.n));
+    if (blockIdx.x == 0) {
+      atomicAdd(&t.ctrl->vertices, static_cast<unsigned long long>(a.n));
+      t.ctrl->left = a.sweep ? 1ull : 0ull;
+    }
   }
 
   if (TEMPORAL && a.order)
@@ -1360,10 +1363,10 @@ __global__ void __launch_bounds__(BLOCK, (W == 4 ? 1 : 2) * (kFusedBlock / BLOCK
   if (threadIdx.x == 0)
     for (uint32_t v = blockIdx.x; v < a.nviews; v += gridDim.x) reset_counters(a.views[v].t.ctrl);
   if (blockIdx.x == 0 && threadIdx.x == 0) reset_counters(a.ctrl);
-  // empty the slot tables of the views that are swept
+  // empty the slot tables of the views that are swept, or were left full
   for (uint32_t v = 0; v < a.nviews; ++v) {
     take_view(&vd, a, __ldg(&a.views[v].tile_base), cur);
-    if (cur == v && vd.sweep)
+    if (cur == v && (vd.sweep || __ldcg(&vd.t.ctrl->left)))
       sweep_slots(vd.t, blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x,
                   static_cast<size_t>(gridDim.x) * blockDim.x);
   }
@@ -1409,6 +1412,9 @@ __global__ void __launch_bounds__(BLOCK, (W == 4 ? 1 : 2) * (kFusedBlock / BLOCK
         atomicAdd(&a.views[v].t.ctrl->vertices, static_cast<unsigned long long>(a.views[v].n));
   }
   if (!grid_barrier(a.ctrl, gridDim.x)) return;
+  if (threadIdx.x == 0)
+    for (uint32_t v = blockIdx.x; v < a.nviews; v += gridDim.x)
+      if (a.views[v].ntiles) a.views[v].t.ctrl->left = a.views[v].sweep ? 1ull : 0ull;
 
   auto add_tile = [&](uint32_t gt) {
     take_view(&vd, a, gt, cur);
@@ -1574,9 +1580,9 @@ static bool sweep_pays(const TableDev& t, size_t vertices) {
 }
 
 cudaError_t launch_clear(const TableDev& t, uint32_t ntiles, cudaStream_t st) {
-  if (ntiles == 0) return cudaSuccess;
   const int sweep = sweep_pays(t, static_cast<size_t>(ntiles) * kTile) ? 1 : 0;
-  const int grid = split_grid(sweep ? ~size_t{0} / 2 : static_cast<size_t>(ntiles) * 32);
+  // (a launch without tiles is there for slots that may have been left)
+  const int grid = split_grid(sweep || !ntiles ? t.mask / 2 + size_t{1} : static_cast<size_t>(ntiles) * 32);
   k_clear_sweep<<<grid, kBlock, 0, st>>>(t, ntiles, kTileIds, sweep);
   return cudaGetLastError();
 }
