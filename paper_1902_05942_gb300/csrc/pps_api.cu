@@ -197,7 +197,8 @@ int batch_of(const pps_table* t) { return t->tune.batch == 4 ? 4 : 2; }
 int merge_of(const pps_table* t) { return t->tune.merge ? static_cast<int>(t->tune.merge) : 2; }
 
 // Plain and temporal frames on tables up to this size have always been inserted
-// from the end of the stream, the others from its start (add_ordered).
+// from the end of the stream, the others from its start: which vertices run out of
+// probes (k_fused) and a sum's last bit (add_ordered) depend on it.
 constexpr uint32_t kBackwards = 1u << 23;
 
 // Empty the slots of the split path's frame.
@@ -536,7 +537,8 @@ int filter_one(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_ve
   plan.evict = t->dev.hist_evict != 0;
   plan.neigh = t->dev.neighbors != 0;
   plan.kv = v->dist || v->extra;
-  if (blend) plan.order = pps::add_order(t->dev, t->T <= kBackwards && !plan.evict && !plan.neigh && !plan.kv);
+  plan.backwards = t->T <= kBackwards && !plan.evict && !plan.neigh && !plan.kv;
+  if (blend) plan.order = pps::add_order(t->dev, plan.backwards);
   set_camera(t, cam, frame);
   if (n == 0) return reset_frame(t, st);
   plan.sweep = pps::sweep_pays_host(t->dev, n);

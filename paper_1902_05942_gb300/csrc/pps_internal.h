@@ -32,6 +32,7 @@ struct FusedPlan {
   bool kv = false;        // ... vertices with key variants
   bool sweep = false;     // zero the whole slot table first, not the frame's slots at the end
   int merge = 2;      // merging of equal keys within a warp (pps_tuning.merge)
+  bool backwards = false;  // insert from the end of the vertex stream
   AddOrder order = kAnyOrder;
 };
 

@@ -92,20 +92,32 @@ struct Counters {
 // 42 against 121 G/s on a 64 MB table).  About one key in seven meets another
 // key there; finishing those on the spot would make the whole warp wait for
 // four or five more memory round trips of a few lanes.  They go into a queue of
-// the warp's own in shared memory instead, and whenever it holds enough of them
-// the warp advances 32 at once, each by one step of its probe sequence.
+// the warp's own in shared memory instead, and while it holds more than a step's
+// worth the warp advances 32 at once, each by one step of its probe sequence.
+//
+// A key that waits there loses its place: later keys fill the slots it would
+// have had, and more keys run out of probes (5.06 M vertices, 2^22 slots, 16
+// probes: 0.178 % of the vertices, 0.128 % where every key is finished at once).
+// So a warp that has seen a key use up a sixth of its probes, which in a table
+// with few collisions hardly ever happens, empties its queue after every step
+// from then on: 0.122 % at 242 us instead of 196; the oldest entries first instead
+// left 0.171 %.  With 8 probes 1.11 % become 0.95 % (at once 0.99 %).  With a quarter
+// of the probes instead of a sixth, 2.94 M vertices in 2^22 slots lost 253 vertices
+// at 64 probes, 225 like this, 219 at once; with an eighth no fewer, but on 9 M
+// vertices with few collisions (2^23 slots, 64 probes) 351 us instead of 337.
 //
 // What bounds pass one now is the keys: without any table access it takes
 // 84 us (about 330 instructions per vertex at 8 warps per scheduler, 64
 // registers), the compare-and-swaps add 20 us, the queue 20 us.
-constexpr int kQueue = 64;  // queue entries per warp
+//
+// Queue entries per warp: a step's worth that may stay, and the keys of two rows.
+constexpr int kQueue = 96;
 
 // Tables far larger than L2 read the home slot before they try to take it: a
 // compare-and-swap that fails still costs the sector's way back to DRAM (random
-// compare-and-swaps 23 G/s on a 1 GB table, loads 43 G/s).  61 M vertices, 2^26
-// slots: 8,890 us without this, 8,725 with it; with 2^24 slots (L2 holds most of
-// them) it makes no difference.
-constexpr uint32_t kLookFirst = (1u << 25) - 1u;  // slots - 1
+// compare-and-swaps 23 G/s on a 1 GB table, loads 43 G/s).  They also empty the
+// queue after every step, whose sectors are then still in L2.  
+constexpr uint32_t kLargeTable = (1u << 25) - 1u;  // slots - 1
 
 // Shared memory of one warp: its queue of keys, and the contributions of a row
 // of 32 vertices while equal cells are merged.
@@ -134,8 +146,9 @@ struct WarpInsert {
   uint32_t claims;   // ids handed out of the current tile's range (the same in every lane)
   uint32_t id_base;  // that range's first id
   uint32_t queued;   // entries in the queue (the same in every lane)
+  uint32_t most;     // entries that may stay in it after a step (the same in every lane)
   Counters cnt;
-  __device__ __forceinline__ WarpInsert() : claims(0u), id_base(0u), queued(0u) {
+  __device__ __forceinline__ WarpInsert() : claims(0u), id_base(0u), queued(0u), most(32u) {
 #pragma unroll
     for (int q = 0; q < W; ++q) my[q] = kOverflowSlot;
   }
@@ -185,10 +198,9 @@ __device__ __forceinline__ void create_cell(const TableDev& t, uint32_t id, floa
 // the first slot of the sequence that holds the fingerprint or is empty
 // decides, and an empty one is taken only by its compare-and-swap.  A step is
 // two or three dependent round trips to L2 whatever it reads, so fewer steps
-// count, most where the table is full or the frame small: two slots at a time
-// and the colours read after the compare-and-swap took 8,140 us on the 61 M
-// vertex frame (load 0.7), this takes 7,855; 117.9 and 114.4 us on a 720p frame.
-// All lanes.
+// count, most where the table is full or the frame small: with two slots at a
+// time and the colours read after the compare-and-swap a 720p frame took 117.9
+// us, like this 114.4.  All lanes.
 template <int W, bool KREC = false>
 __device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& v, WarpInsert<W>& s,
                                            WarpShared& sh, bool rec, uint32_t own, uint32_t* stash,
@@ -264,6 +276,7 @@ __device__ __forceinline__ void queue_step(const TableDev& t, const VertexPtrs& 
     if (KREC) qkw[o] = kr;
   }
   s.queued = at + __popc(again);
+  if (__any_sync(0xFFFFFFFFu, have && 6u * step >= t.max_probes)) s.most = 0u;  // crowded: no key may wait
   __syncwarp();
 }
 
@@ -344,7 +357,7 @@ __device__ __forceinline__ void insert_warp(const KeyConst& kc, const TableDev& 
     s.reserve(q, lead >> q & 1u);
   }
   unsigned long long old[W];
-  const bool look = t.mask >= kLookFirst;
+  const bool look = t.mask >= kLargeTable;
 #pragma unroll
   for (int q = 0; q < W; ++q) {
     old[q] = 0ull;
@@ -400,9 +413,12 @@ __device__ __forceinline__ void insert_warp(const KeyConst& kc, const TableDev& 
       }
       s.queued += __popc(put);
       __syncwarp();
-      while (s.queued > kQueue - 32) queue_step<W, KREC>(t, v, s, sh, rec, own, stash, qkw);
+      if (W > 2)  // (two rows find room)
+        while (s.queued > 2u * s.most) queue_step<W, KREC>(t, v, s, sh, rec, own, stash, qkw);
     }
   }
+  while (s.queued > (t.mask >= kLargeTable ? 0u : s.most))
+    queue_step<W, KREC>(t, v, s, sh, rec, own, stash, qkw);
 }
 
 // Pass two for W rows of 32 vertices from j0 on, STEP apart (those below
@@ -1118,6 +1134,7 @@ struct FusedArgs {
   int sweep;         // zero the whole slot table first, instead of the frame's slots at the end
   uint32_t* nq;      // neighborhood search: the queue of low-count vertices
   int merge;         // merging of equal keys within a warp (insert_warp)
+  int backwards;     // insert from the end of the vertex stream
   int order;         // AddOrder of pass two
 };
 
@@ -1203,7 +1220,8 @@ __device__ __forceinline__ void lookup_warp(const TableDev& t, const VertexPtrs&
 // rest in any order, a frame of 1.66 M vertices had 33,300 cells with another
 // sum than the insert in one pass gave, in this order 12,000, and 11,400 from
 // one run of that insert to the next; of 61 M vertices (2^26 slots) 364,000,
-// 74,000 and 44,000.  It costs 4 and 340 us there (111.6 and 8,660 us a frame).
+// 74,000 and 44,000.  It costs 4 and 340 us there (of 116 and
+// 8,200 us a frame).
 __device__ __forceinline__ void add_ordered(const FusedArgs& a, WarpShared& sh) {
   constexpr uint32_t kHalf = 1024, kSpan = 2 * kHalf;
   static_assert(kFusedBlock == 512, "two rows, or one row of pairs, per warp and half tile");
@@ -1234,7 +1252,15 @@ __device__ __forceinline__ void add_ordered(const FusedArgs& a, WarpShared& sh) 
 //       the compare-and-swaps meet it in L2; so is what another launch left;
 //   A1  keys, probing insert, in tiles of a.tile_v vertices, every nw-th tile
 //       to one warp (a counter that hands them out costs more than it
-//       balances: its atomics serialize on one address, HD 146 us against 126);
+//       balances: its atomics serialize on one address, HD 146 us against 126),
+//       from the end of the vertex stream on frames that have always been
+//       inserted so (backwards: such a stream is bounce-major; its
+//       secondary-bounce tiles, whose vertices nearly all create cells of their
+//       own and cost the most, go first and let the cheap primary-hit tiles
+//       balance the warps at the end) and from its start on the others, above
+//       all on large tables: there the cells with many members, the primary
+//       hits, have to come first, into an empty table, or a quarter more
+//       vertices run out of probes (61 M vertices, 2^26 slots, 32 probes);
 //       a tile's new cells take ids from the tile's own range, and each
 //       vertex's cell id goes to the stash;
 //   A2  accumulation (128 vertices at a time, or in order: add_ordered);
@@ -1264,11 +1290,7 @@ __global__ void __launch_bounds__(kFusedBlock, W == 4 ? 1 : 2) k_fused(FusedArgs
     const bool rec = blended || !a.sweep;
     const uint32_t own = TEMPORAL && a.order ? 0u : kOwnerBit;
     for (uint32_t k = gw; k < ntiles; k += nw) {
-      // from the end of the vertex stream: streams are bounce-major, so the
-      // secondary-bounce tiles, whose vertices nearly all create cells of
-      // their own and cost the most, go first and the cheap primary-hit tiles
-      // balance the warps at the end
-      const uint32_t tile = ntiles - 1u - k;
+      const uint32_t tile = a.backwards ? ntiles - 1u - k : k;
       const size_t t0 = static_cast<size_t>(tile) * tile_v;
       const size_t end = min(a.n, t0 + tile_v);
       s.claims = 0u;
@@ -1391,6 +1413,7 @@ __global__ void __launch_bounds__(BLOCK, (W == 4 ? 1 : 2) * (kFusedBlock / BLOCK
         if (c) atomicAdd(&vd.t.ctrl->frame_cells, c);
       }
       s.cnt = Counters{};
+      s.most = 32u;
       s.retire(vd.t, true);  // reserved ids belong to the view
     };
     for (uint32_t gt = gw; gt < a.total_tiles; gt += nw) {
@@ -1711,6 +1734,7 @@ cudaError_t launch_fused(const KeyConst& kc, const TableDev& t, const VertexPtrs
   a.sweep = plan.sweep ? 1 : 0;
   a.nq = nq;
   a.merge = plan.merge;
+  a.backwards = plan.backwards ? 1 : 0;
   a.order = plan.order;
   void* args[] = {&a};
   cudaError_t e = cudaLaunchCooperativeKernel(fused_kernel(plan), dim3(plan.grid), dim3(plan.block), args,

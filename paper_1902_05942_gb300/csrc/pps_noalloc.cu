@@ -166,6 +166,7 @@ extern "C" int pps_filter_noalloc(const pps_params* p, const pps_camera* cam, ui
   const uint32_t T = 1u << p->log2_slots;
   pps::FusedPlan plan;
   plan.sweep = true;
+  plan.backwards = true;
   cudaError_t e = pps::plan_fused(n, kNoAllocMaxCells, &plan);
   if (e != cudaSuccess)
     return noalloc_fail(PPS_ECUDA, std::string("pps_filter_noalloc: ") + cudaGetErrorString(e));
