@@ -591,6 +591,17 @@ int pps_mlp_gradient(pps_mlp *m, const pps_vertices *v, const float *tr, const f
  */
 int pps_selftest_wait(int kind, uint32_t limit_us, uint32_t *error_word);
 
+/*
+ * pps_selftest_infer: one CTA of the learned fallback's evaluation, `tiles`
+ * (1 .. 3) tiles for each of its four groups of 128 threads, in which one thread
+ * of every group, that of row `row` (0 .. 127), acts as if its wait for the output
+ * layer had run out while the others go on.  The launch has to end, with the
+ * wait-timeout bit (1) in *error_word (host).  Synchronous on the current
+ * device; uses its own device memory.  PPS_EINVAL for a bad row or number of
+ * tiles or NULL error_word (checked before any CUDA call).
+ */
+int pps_selftest_infer(int row, uint32_t tiles, uint32_t *error_word);
+
 #ifdef __cplusplus
 }
 #endif

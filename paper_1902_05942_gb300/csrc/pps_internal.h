@@ -115,6 +115,12 @@ std::string device_error_text(unsigned int word);  // the bits of a device error
 int check_params(const pps_params* p);
 
 // Self-test of the tensor-core kernels' bounded mbarrier wait (pps_mlp.cu).
+// One CTA of the learned fallback's evaluation over `tiles` tiles per group, in
+// which the thread of row `row` gives up its wait for the output layer; `mem`:
+// selftest_infer_bytes() zeroed bytes, 16-byte aligned.
+constexpr uint32_t kSelftestVertices = 3 * 512;
+size_t selftest_infer_bytes();
+cudaError_t launch_selftest_infer(int row, uint32_t tiles, void* mem, unsigned int* err, cudaStream_t st);
 cudaError_t launch_selftest_mbar(unsigned long long limit_ns, unsigned int* err, cudaStream_t st);
 
 }  // namespace pps

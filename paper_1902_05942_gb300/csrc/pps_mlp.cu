@@ -373,8 +373,12 @@ __device__ __forceinline__ bool group_sync(int g, bool pred) {
 
 }  // namespace tc
 
-__global__ void __launch_bounds__(tc::kThreads, 2) k_mlp_infer_tc(Dev d, VertexPtrs v, const int32_t* list,
-                                                      const uint32_t* counter, OutPtrs o, int all) {
+// GIVES_UP (self-test): in every group the thread of row `quitter` acts as if
+// its wait for the output layer had run out, on each of its tiles.
+template <bool GIVES_UP>
+__global__ void __launch_bounds__(tc::kThreads, 2)
+    k_mlp_infer_tc(Dev d, VertexPtrs v, const int32_t* list, const uint32_t* counter, OutPtrs o, int all,
+                   int quitter) {
   extern __shared__ unsigned char smem_raw[];
   tc::Smem& s = *reinterpret_cast<tc::Smem*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
@@ -441,7 +445,9 @@ __global__ void __launch_bounds__(tc::kThreads, 2) k_mlp_infer_tc(Dev d, VertexP
   int32_t j = row_of(tile);
   VertexIn vi = load_vertex(d, v, j);
   int32_t jn = row_of(tile + stride);
-  for (; tile < ntiles && ok; tile += stride) {
+  // A thread whose wait ran out goes on to the group's next barrier, where all
+  // 128 threads vote: none of them leaves the loop alone.
+  for (; tile < ntiles; tile += stride) {
     tc::encode_row(act, row, vi, j >= 0);
     // while this tile goes through the layers: the next tile's vertex (its list
     // entry was read one tile ago, so the loads do not wait for it) and the
@@ -463,6 +469,7 @@ __global__ void __launch_bounds__(tc::kThreads, 2) k_mlp_infer_tc(Dev d, VertexP
       }
       __syncwarp();
       ok = tc::mbar_wait(mbar, parity);
+      if (GIVES_UP && layer == 3 && row == quitter) ok = false;
       parity ^= 1u;
       tc::fence_after();
       if (layer < 3) {
@@ -492,7 +499,10 @@ __global__ void __launch_bounds__(tc::kThreads, 2) k_mlp_infer_tc(Dev d, VertexP
     j = jn;
     jn = jnn;
   }
-  if (!ok && (tid & 31) == 0) atomicOr(d.err, 1u);
+  if (!ok) {
+    atomicOr(d.err, 1u);
+    tc::mbar_wait(mbar, parity ^ 1u);  // (bounded) for a product still under way
+  }
   tc::fence_before();
   __syncthreads();
   if (warp == 0)
@@ -1063,6 +1073,41 @@ cudaError_t launch_selftest_mbar(unsigned long long limit_ns, unsigned int* err,
   mlp::k_selftest_mbar<<<1, 32, 0, st>>>(limit_ns, err);
   return cudaGetLastError();
 }
+
+size_t selftest_infer_bytes() {
+  // zeroed: network (FP32 and BF16), one value per vertex, list and its length
+  return mlp::kP * sizeof(float) + mlp::kWb * sizeof(__nv_bfloat16) + 16 +
+         kSelftestVertices * (2 * sizeof(float) + sizeof(int32_t) + sizeof(uint32_t)) + 16;
+}
+
+cudaError_t launch_selftest_infer(int row, uint32_t tiles, void* mem, unsigned int* err, cudaStream_t st) {
+  unsigned char* p = static_cast<unsigned char*>(mem);
+  auto take = [&](size_t bytes) {
+    void* at = p;
+    p += (bytes + 15) / 16 * 16;
+    return at;
+  };
+  mlp::Dev d{};
+  d.wb = static_cast<__nv_bfloat16*>(take(mlp::kWb * sizeof(__nv_bfloat16)));
+  uint32_t* count = static_cast<uint32_t*>(take(sizeof(uint32_t)));
+  float* in = static_cast<float*>(take(kSelftestVertices * sizeof(float)));
+  float* out = static_cast<float*>(take(kSelftestVertices * sizeof(float)));
+  int32_t* list = static_cast<int32_t*>(take(kSelftestVertices * sizeof(int32_t)));
+  d.master = reinterpret_cast<float*>(p);
+  d.err = err;
+  VertexPtrs v{};
+  v.px = v.py = v.pz = v.nx = v.ny = v.nz = in;
+  OutPtrs o{};
+  o.r = o.g = o.b = out;
+  const uint32_t n = std::min<uint32_t>(tiles * mlp::tc::kThreads, kSelftestVertices);
+  cudaError_t e = cudaMemcpyAsync(count, &n, sizeof(n), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(mlp::k_mlp_infer_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(mlp::tc::kSmemBytes));
+  if (e != cudaSuccess) return e;
+  mlp::k_mlp_infer_tc<true><<<1, mlp::tc::kThreads, mlp::tc::kSmemBytes, st>>>(d, v, list, count, o, 1, row);
+  return cudaGetLastError();
+}
 }  // namespace pps
 
 // ---------------------------------------------------------------- C ABI
@@ -1231,7 +1276,7 @@ int pps_mlp_create(pps_mlp** out, const pps_mlp_params* p, const float* init_hos
   }
   if (e == cudaSuccess) e = cudaMemcpy(m->dev.master, w.data(), P * sizeof(float), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
-    if (cudaFuncSetAttribute(pps::mlp::k_mlp_infer_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(pps::mlp::k_mlp_infer_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(pps::mlp::tc::kSmemBytes)) != cudaSuccess ||
         cudaFuncSetAttribute(pps::mlp::k_mlp_train_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(pps::mlp::tct::kSmemBytes)) != cudaSuccess)
@@ -1380,9 +1425,9 @@ static int launch_infer(pps_mlp* m, const pps_vertices* v, size_t n, const pps::
   cfg.stream = st;
   cfg.attrs = &early;
   cfg.numAttrs = 1;
-  MLP_CUDA(cudaLaunchKernelEx(&cfg, pps::mlp::k_mlp_infer_tc, m->dev, vptrs(v),
+  MLP_CUDA(cudaLaunchKernelEx(&cfg, pps::mlp::k_mlp_infer_tc<false>, m->dev, vptrs(v),
                               static_cast<const int32_t*>(m->list),
-                              static_cast<const uint32_t*>(m->counter), o, all));
+                              static_cast<const uint32_t*>(m->counter), o, all, 0));
   return PPS_OK;
 }
 

@@ -20,6 +20,27 @@ __global__ void k_selftest_barrier(Ctrl* c, unsigned long long limit_ns) {
 }  // namespace
 }  // namespace pps
 
+extern "C" int pps_selftest_infer(int row, uint32_t tiles, uint32_t* error_word) {
+  if (!error_word) return pps::record_error(PPS_EINVAL, "error_word is NULL");
+  if (row < 0 || row > 127) return pps::record_error(PPS_EINVAL, "row must be in [0, 127]");
+  if (tiles < 1 || tiles > 3) return pps::record_error(PPS_EINVAL, "tiles must be 1, 2 or 3");
+  *error_word = 0;
+  unsigned char* mem = nullptr;
+  const size_t bytes = pps::selftest_infer_bytes() + 64;
+  cudaError_t e = cudaMalloc(&mem, bytes);
+  if (e == cudaSuccess) e = cudaMemset(mem, 0, bytes);
+  unsigned int* word = reinterpret_cast<unsigned int*>(mem);
+  if (e == cudaSuccess) e = pps::launch_selftest_infer(row, tiles, mem + 64, word, nullptr);
+  if (e == cudaSuccess) e = cudaMemcpy(error_word, word, sizeof(*word), cudaMemcpyDeviceToHost);
+  cudaFree(mem);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    const std::string msg = std::string("pps_selftest_infer: ") + cudaGetErrorString(e);
+    return pps::record_error(PPS_ECUDA, msg.c_str());
+  }
+  return PPS_OK;
+}
+
 extern "C" int pps_selftest_wait(int kind, uint32_t limit_us, uint32_t* error_word) {
   if (!error_word) return pps::record_error(PPS_EINVAL, "error_word is NULL");
   if (kind != 0 && kind != 1) return pps::record_error(PPS_EINVAL, "kind must be 0 or 1");

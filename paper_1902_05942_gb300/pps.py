@@ -128,6 +128,7 @@ SIGNATURES = {
                          ctypes.c_int),
     "pps_batch_run": ([_vp, ctypes.POINTER(pps_camera), _u32, _vp], ctypes.c_int),
     "pps_batch_destroy": ([_vp], ctypes.c_int),
+    "pps_selftest_infer": ([ctypes.c_int, _u32, ctypes.POINTER(_u32)], ctypes.c_int),
     "pps_selftest_wait": ([ctypes.c_int, _u32, ctypes.POINTER(_u32)], ctypes.c_int),
     "pps_bench_rate": ([ctypes.c_int, ctypes.c_size_t, ctypes.c_size_t, _vp, _vp,
                         ctypes.POINTER(ctypes.c_double)], ctypes.c_int),
@@ -236,6 +237,13 @@ def camera(pos: Sequence[float]) -> pps_camera:
 # ---------------------------------------------------------------- C-named calls
 def pps_version() -> str:
     return lib().pps_version().decode()
+
+
+def pps_selftest_infer(row: int, tiles: int) -> int:
+    """Error word of the fallback's evaluation when the thread of one row gives up."""
+    w = _u32()
+    _check(lib().pps_selftest_infer(int(row), int(tiles), ctypes.byref(w)))
+    return w.value
 
 
 def pps_selftest_wait(kind: int, limit_us: int) -> int:
