@@ -841,8 +841,7 @@ int pps_stats(pps_table* t, pps_stats_t* out, void* stream) {
   if (!out) return fail(PPS_EINVAL, "out is NULL");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   PPS_CUDA(cudaMemsetAsync(t->scratch_u64, 0, 2 * sizeof(unsigned long long), st));
-  if (t->state != kClean)  // between frames the table is empty
-    PPS_CUDA(pps::launch_count_nonzero(t->dev.slots, 8, 0, 8, t->T, t->scratch_u64, st));
+  PPS_CUDA(pps::launch_count_nonzero(t->dev.slots, 8, 0, 8, t->T, t->scratch_u64, st));
   if (t->dev.hcells)
     PPS_CUDA(pps::launch_count_nonzero(t->dev.hcells, t->dev.hstride, t->dev.hfp_off, 4, t->Th,
                                        t->scratch_u64 + 1, st));
@@ -855,7 +854,8 @@ int pps_stats(pps_table* t, pps_stats_t* out, void* stream) {
   out->frame_cells = c.frame_cells;
   out->overflow_vertices = c.overflow_vertices;
   out->vertices = c.vertices;
-  out->occupied_slots = occ[0];
+  // (what a launch left there is no frame's any more)
+  out->occupied_slots = t->state == kClean && c.left ? 0 : occ[0];
   out->hist_occupied = occ[1];
   out->hist_overflow = c.hist_overflow;
   out->device_error = c.error;
@@ -877,11 +877,15 @@ int pps_table_dump(pps_table* t, uint32_t* fp_host, void* acc_host, void* stream
   if (!fp_host) return fail(PPS_EINVAL, "fp_host is NULL");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t acc_b = t->dev.fixed ? 32 : 16;
-  if (t->state == kClean) {  // between frames the table is empty
+  if (t->state == kClean) {
+    unsigned long long left = 0;
+    PPS_CUDA(cudaMemcpyAsync(&left, &t->dev.ctrl->left, sizeof(left), cudaMemcpyDeviceToHost, st));
     PPS_CUDA(cudaStreamSynchronize(st));
-    std::memset(fp_host, 0, t->T * sizeof(uint32_t));
-    if (acc_host) std::memset(acc_host, 0, t->T * acc_b);
-    return PPS_OK;
+    if (left) {  // no frame's any more
+      std::memset(fp_host, 0, t->T * sizeof(uint32_t));
+      if (acc_host) std::memset(acc_host, 0, t->T * acc_b);
+      return PPS_OK;
+    }
   }
   unsigned long long* slots =
       static_cast<unsigned long long*>(std::malloc(t->T * sizeof(unsigned long long)));

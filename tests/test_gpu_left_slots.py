@@ -100,3 +100,27 @@ def test_replayed_graphs_in_any_order():
         split(j)
         tab.filter(vs[1], _cam(7), 7)
     tab.close()
+
+
+def test_occupancy_is_counted_in_the_slots():
+    """Between frames too: a replayed insert, of which the host knows nothing,
+    shows in the statistics and the dump; what a launch left behind does not."""
+    tab = pps.Table(_cfg(16))
+    large, v = _views(30_000, 300)
+    tab.build(_cam(7), 7)
+    tab.insert(v)
+    cells = tab.stats()["occupied_slots"]
+    assert cells == tab.stats()["frame_cells"] > 0
+    graph = torch.cuda.CUDAGraph()
+    tab.build(_cam(7), 7)
+    with torch.cuda.graph(graph):
+        tab.insert(v)
+    tab.filter(v, _cam(7), 7)  # empties its own slots
+    assert tab.stats()["occupied_slots"] == 0 and not tab.dump()[0].any()
+    graph.replay()
+    assert tab.stats()["occupied_slots"] == cells and (tab.dump()[0] != 0).sum() == cells
+    tab.filter(large, _cam(7), 7)  # empties the table first and leaves its own cells
+    assert tab.stats()["occupied_slots"] == 0 and not tab.dump()[0].any()
+    tab.filter(v, _cam(7), 7)
+    assert tab.stats()["occupied_slots"] == 0 and not tab.dump()[0].any()
+    tab.close()
