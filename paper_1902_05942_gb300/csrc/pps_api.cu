@@ -771,19 +771,15 @@ int pps_host_wait(pps_table* t) {
 }  // extern "C"
 
 namespace pps {
-// For batched launches: the device description of a table about to filter n
-// vertices in one persistent launch (cell-id capacity ensured), its batch
-// width, and whether it keeps a history.  The table must be between frames.
-int table_for_batch(pps_table* t, size_t n, ViewDesc* vd, int* batch, int* block,
-                    bool* temporal_out, cudaStream_t st) {
+// For batched launches: the device description of a table, its batch width, and
+// whether it keeps a history.  The table must be between frames.
+int table_for_batch(pps_table* t, ViewDesc* vd, int* batch, int* block, bool* temporal_out) {
   if (int rc = check_table(t)) return rc;
   if (t->state != kClean) return fail(PPS_ESTATE, "a table of a batch is in the middle of a frame");
   if (t->p.fallback != PPS_FALLBACK_NONE || t->p.hist_evict || t->p.hist_migrate ||
       t->p.normal_search)
     return fail(PPS_EINVAL, "batched views take tables without a low-count fallback, eviction, "
                             "migration or normal search");
-  // the batch's tile width and batch are not known yet: room for the widest id ranges
-  if (int rc = ensure_dense(t, fused_cells(n, 64u, 4), 0, st)) return rc;
   t->leaves = true;
   vd->kc = t->kc;
   vd->t = t->dev;
@@ -792,6 +788,11 @@ int table_for_batch(pps_table* t, size_t n, ViewDesc* vd, int* batch, int* block
   *temporal_out = temporal(t);
   return PPS_OK;
 }
+
+// Make room for `cells` cells in a table between frames.
+int table_reserve(pps_table* t, size_t cells, cudaStream_t st) { return ensure_dense(t, cells, 0, st); }
+
+const TableDev& table_dev(const pps_table* t) { return t->dev; }
 }  // namespace pps
 
 extern "C" {

@@ -25,6 +25,7 @@
 struct pps_batch {
   struct OwnView {  // a view with a launch of its own
     uint32_t index;  // of its camera
+    pps_table* table;
     pps::ViewDesc vd;
     pps::FusedPlan plan;
   };
@@ -32,6 +33,7 @@ struct pps_batch {
   std::vector<OwnView> own;
   std::vector<pps::ViewDesc> base;  // views of the shared launch, without camera and frame
   std::vector<uint32_t> index;      // of their cameras
+  std::vector<pps_table*> tables;   // theirs
   uint32_t total_tiles = 0;
   bool temporal = false;
   bool ordered = false;  // a view of the shared launch adds its contributions up in order
@@ -92,7 +94,7 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
     pps::ViewDesc vd{};
     bool tmp = false;
     int bw = 2, blk = 512;
-    if (int rc = pps::table_for_batch(v.table, v.n, &vd, &bw, &blk, &tmp, nullptr)) {
+    if (int rc = pps::table_for_batch(v.table, &vd, &bw, &blk, &tmp)) {
       delete b;
       return rc;
     }
@@ -113,7 +115,7 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
       plan.temporal = vd.blended != 0;
       plan.sweep = vd.sweep != 0;
       if (vd.ordered) plan.order = pps::kPairsForwards;
-      b->own.push_back(pps_batch::OwnView{i, vd, plan});
+      b->own.push_back(pps_batch::OwnView{i, v.table, vd, plan});
       own_words = std::max<size_t>(own_words, v.n);
     } else {
       b->temporal = b->temporal || tmp;
@@ -121,6 +123,7 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
       total += v.n;
       b->base.push_back(vd);
       b->index.push_back(i);
+      b->tables.push_back(v.table);
     }
   }
   if (blend && (!(alpha <= 1.0f) || alpha != alpha)) {
@@ -139,6 +142,16 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
     if (e == cudaSuccess) e = pps::plan_fused(w.vd.n, ~size_t{0}, &w.plan);
   }
   const uint32_t nshared = static_cast<uint32_t>(b->base.size());
+  // room for the cell ids of each view's tiles
+  int rc = PPS_OK;
+  for (size_t i = 0; i < b->own.size() && e == cudaSuccess && !rc; ++i)
+    rc = pps::table_reserve(b->own[i].table, pps::fused_cells(b->own[i].vd.n, b->own[i].plan.tile, batch), nullptr);
+  for (size_t i = 0; i < nshared && e == cudaSuccess && !rc; ++i)
+    rc = pps::table_reserve(b->tables[i], pps::fused_cells(b->base[i].n, tile, batch), nullptr);
+  if (rc) {
+    delete b;
+    return rc;
+  }
   const int graphs = nshared ? 2 : 0;
   if (e == cudaSuccess && nshared)
     e = pps::plan_multi(b->total_tiles, tile, b->temporal, batch, block, &b->plan);
@@ -203,6 +216,7 @@ int pps_batch_run(pps_batch* b, const pps_camera* cams, uint32_t frame, void* st
     if (e == cudaSuccess) {
       for (size_t i = 0; i < b->base.size(); ++i) {
         pps::ViewDesc vd = b->base[i];
+        vd.t = pps::table_dev(b->tables[i]);  // another call on the table may have moved its arrays
         aim(vd.kc, cams[b->index[i]]);
         b->hviews[k][i] = vd;
       }
@@ -214,7 +228,7 @@ int pps_batch_run(pps_batch* b, const pps_camera* cams, uint32_t frame, void* st
     const pps::ViewDesc& vd = b->own[i].vd;
     pps::KeyConst kc = vd.kc;
     aim(kc, cams[b->own[i].index]);
-    e = pps::launch_fused(kc, vd.t, vd.v, vd.n, vd.o, vd.blended != 0, b->alpha, b->own[i].plan, b->gstash,
+    e = pps::launch_fused(kc, pps::table_dev(b->own[i].table), vd.v, vd.n, vd.o, vd.blended != 0, b->alpha, b->own[i].plan, b->gstash,
                           nullptr, st);
   }
   if (e != cudaSuccess) return bfail(PPS_ECUDA, std::string("pps_batch_run: ") + cudaGetErrorString(e));

@@ -128,7 +128,8 @@ cudaError_t launch_selftest_mbar(unsigned long long limit_ns, unsigned int* err,
 struct pps_table;
 
 namespace pps {
-int table_for_batch(pps_table* t, size_t n, ViewDesc* vd, int* batch, int* block, bool* temporal,
-                    cudaStream_t st);
+int table_for_batch(pps_table* t, ViewDesc* vd, int* batch, int* block, bool* temporal);
+int table_reserve(pps_table* t, size_t cells, cudaStream_t st);
+const TableDev& table_dev(const pps_table* t);
 
 }  // namespace pps
