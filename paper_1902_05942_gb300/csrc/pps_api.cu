@@ -65,7 +65,8 @@ struct pps_table {
   pps::TableDev dev{};
   pps::KeyConst kc{};
   int state = kClean;
-  uint32_t frame_tiles = 0;  // split path: tiles (cell-id blocks) used this frame
+  uint32_t frame_tiles = 0;  // split path: units of cell ids used this frame
+  bool wide_ids = false;     // self-test: inserts as if their ids took 32 bits
   pps_tuning tune{};         // launch shape (batch width 0 = library default)
   size_t D = 0;              // capacity of the dense cell arrays
   uint32_t* stash = nullptr;  // [D] the vertices' cell ids during a call
@@ -219,18 +220,25 @@ int reset_frame(pps_table* t, cudaStream_t st) {
   return PPS_OK;
 }
 
+// Cell ids that a word of the stash has room for beside the bit that marks a
+// cell's creator.
+constexpr size_t kMostOwned = 0x7FFFFFF0ull;
+
+// Tile counts beside `cells` cells: one per tile, whose range has 160 ids or more.
+size_t tile_counts(size_t cells) { return cells / 128 + 16; }
+
 // Make the dense cell arrays hold at least `need` cells, keeping the first
 // `keep` cells (accumulators, cell info, tile counts and quantized keys),
 // and the stash as many vertices.
 int ensure_dense(pps_table* t, size_t need, size_t keep, cudaStream_t st) {
   if (need <= t->D) return PPS_OK;
-  constexpr size_t kMost = 0x7FFFFFF0ull;  // the stash words' top bit marks a cell's creator
-  if (need > kMost) return fail(PPS_EINVAL, "more than 2^31 - 16 cells in one frame");
+  constexpr size_t kMost = 0xFFFFFFF0ull;
+  if (need > kMost) return fail(PPS_EINVAL, "more than 2^32 - 16 cell ids in one frame");
   size_t cap = t->D ? t->D : 1;
   while (cap < need) cap *= 2;
   if (cap > kMost) cap = kMost;
   const size_t acc_b = t->dev.fixed ? 32 : 16;
-  const size_t nb = cap / 4 + 16;  // tile counts: one per block of >= 4 cells
+  const size_t nb = tile_counts(cap);
   void *acc = nullptr, *info = nullptr, *bc = nullptr, *kw = nullptr, *hold = nullptr, *ids = nullptr;
   cudaError_t e = cudaMalloc(&acc, cap * acc_b);
   if (e == cudaSuccess) e = cudaMalloc(&info, cap * sizeof(uint4));
@@ -245,7 +253,7 @@ int ensure_dense(pps_table* t, size_t need, size_t keep, cudaStream_t st) {
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(info, t->dev.info, keep * sizeof(uint4), cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(bc, t->dev.bcount, (t->D / 4 + 16) * sizeof(uint32_t),
+      e = cudaMemcpyAsync(bc, t->dev.bcount, tile_counts(t->D) * sizeof(uint32_t),
                           cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess && kw)
       e = cudaMemcpyAsync(kw, t->dev.kw, keep * sizeof(uint4), cudaMemcpyDeviceToDevice, st);
@@ -278,6 +286,12 @@ int ensure_dense(pps_table* t, size_t need, size_t keep, cudaStream_t st) {
   t->dev.bcount = static_cast<uint32_t*>(bc);
   t->D = cap;
   return PPS_OK;
+}
+
+// The same for a persistent launch.
+int reserve_owned(pps_table* t, size_t cells, cudaStream_t st) {
+  if (cells > kMostOwned) return fail(PPS_EINVAL, "more than 2^31 - 16 cell ids in one frame");
+  return ensure_dense(t, cells, 0, st);
 }
 
 void set_camera(pps_table* t, const pps_camera* cam, uint32_t frame) {
@@ -397,8 +411,8 @@ int pps_create(pps_table** out, const pps_params* p) {
   if (e == cudaSuccess) e = alloc(reinterpret_cast<void**>(&t->scratch_u64), 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   // the cells of a frame of min(T, 2^22) vertices on the split path
-  const size_t tiles0 = std::min<size_t>(T, 1u << 22) / pps::tile_size() + 1;
-  if (e == cudaSuccess && ensure_dense(t, tiles0 * pps::split_tile_ids(), 0, nullptr) != PPS_OK)
+  if (e == cudaSuccess &&
+      ensure_dense(t, pps::split_units(std::min<size_t>(T, 1u << 22) + 1) * pps::split_unit_ids(), 0, nullptr) != PPS_OK)
     e = cudaErrorMemoryAllocation;
   if (e != cudaSuccess) {
     free_all(t);
@@ -471,13 +485,12 @@ int pps_insert(pps_table* t, const pps_vertices* v, size_t n, uint32_t* slot_out
   if ((t->dev.hist_migrate || t->dev.normal_search) && v->extra)
     return fail(PPS_EINVAL, "a table with hist_migrate or normal_search takes no extra key word");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const size_t tile = static_cast<size_t>(pps::tile_size());
-  const size_t tiles = (n + tile - 1) / tile;
-  const size_t ids = static_cast<size_t>(pps::split_tile_ids());
-  if (int rc = ensure_dense(t, (t->frame_tiles + tiles) * ids, t->frame_tiles * ids, st)) return rc;
+  const size_t units = pps::split_units(n), ids = static_cast<size_t>(pps::split_unit_ids());
+  const size_t need = (t->frame_tiles + units) * ids;
+  if (int rc = ensure_dense(t, need, t->frame_tiles * ids, st)) return rc;
   PPS_CUDA(pps::launch_insert(t->kc, t->dev, to_dev(v), n, t->stash, slot_out, t->frame_tiles,
-                              batch_of(t), merge_of(t), st));
-  t->frame_tiles += static_cast<uint32_t>(tiles);
+                              t->wide_ids || need > kMostOwned, batch_of(t), merge_of(t), st));
+  t->frame_tiles += static_cast<uint32_t>(units);
   if (t->coarse) return pps_insert(t->coarse, v, n, nullptr, stream);
   return PPS_OK;
 }
@@ -502,7 +515,7 @@ int pps_query(pps_table* t, const pps_vertices* v, size_t n, const uint32_t* slo
   if (int rc = check_output(out, n)) return rc;
   if (t->state == kClean) return fail(PPS_ESTATE, "pps_query needs an open frame");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const uint32_t id_limit = t->frame_tiles * static_cast<uint32_t>(pps::split_tile_ids());
+  const uint32_t id_limit = t->frame_tiles * static_cast<uint32_t>(pps::split_unit_ids());
   if (!t->coarse) {
     PPS_CUDA(pps::launch_query(t->kc, t->dev, to_dev(v), n, slot_in, to_dev(out),
                                t->state == kBlended, id_limit, st));
@@ -518,7 +531,7 @@ int pps_query(pps_table* t, const pps_vertices* v, size_t n, const uint32_t* slo
                              id_limit, st));
   const pps_table* k = t->coarse;
   PPS_CUDA(pps::launch_query(k->kc, k->dev, to_dev(v), n, nullptr, c, k->state == kBlended,
-                             k->frame_tiles * static_cast<uint32_t>(pps::split_tile_ids()), st));
+                             k->frame_tiles * static_cast<uint32_t>(pps::split_unit_ids()), st));
   PPS_CUDA(pps::launch_combine_coarse(n, f.status, c, o, st));
   return PPS_OK;
 }
@@ -546,7 +559,7 @@ int filter_one(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_ve
     if (int rc = empty_frame(t, st)) return rc;
   auto ready = [&]() -> int {
     PPS_CUDA(pps::plan_fused(n, ~size_t{0}, &plan));
-    if (int rc = ensure_dense(t, pps::fused_cells(n, plan.tile, plan.batch), 0, st)) return rc;
+    if (int rc = reserve_owned(t, pps::fused_cells(n, plan.tile, plan.batch), st)) return rc;
     if (t->dev.neighbors && t->neigh_q_cap < n) {
       cudaFree(t->neigh_q);
       t->neigh_q = nullptr;
@@ -593,10 +606,9 @@ int pps_filter(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_ve
   if (t->dev.hist_migrate || t->dev.normal_search) {
     // history migration, similar normals: the split kernels; the insert's cell
     // ids (the stash, in place) spare the lookup its keys and probes
-    const size_t tiles = (n + pps::tile_size() - 1) / pps::tile_size();
     if (int rc = pps_build(t, cam, frame, stream)) return rc;
     // (only now: emptying the last frame's slots reads its cells' records)
-    if (int rc = ensure_dense(t, tiles * pps::split_tile_ids(), 0, st)) return rc;
+    if (int rc = ensure_dense(t, pps::split_units(n) * pps::split_unit_ids(), 0, st)) return rc;
     if (int rc = pps_insert(t, v, n, t->stash, stream)) return rc;
     if (blend)
       if (int rc = pps_blend(t, alpha, stream)) return rc;
@@ -790,7 +802,7 @@ int table_for_batch(pps_table* t, ViewDesc* vd, int* batch, int* block, bool* te
 }
 
 // Make room for `cells` cells in a table between frames.
-int table_reserve(pps_table* t, size_t cells, cudaStream_t st) { return ensure_dense(t, cells, 0, st); }
+int table_reserve(pps_table* t, size_t cells, cudaStream_t st) { return reserve_owned(t, cells, st); }
 
 const TableDev& table_dev(const pps_table* t) { return t->dev; }
 }  // namespace pps
@@ -812,6 +824,13 @@ int pps_set_tuning(pps_table* t, const pps_tuning* tune) {
     if (r) return fail(PPS_EINVAL, "reserved fields must be zero");
   t->tune = *tune;
   if (t->coarse) t->coarse->tune = *tune;
+  return PPS_OK;
+}
+
+int pps_selftest_wide_ids(pps_table* t, int on) {
+  if (int rc = check_table(t)) return rc;
+  t->wide_ids = on != 0;
+  if (t->coarse) t->coarse->wide_ids = t->wide_ids;
   return PPS_OK;
 }
 

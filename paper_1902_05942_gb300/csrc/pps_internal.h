@@ -70,9 +70,11 @@ cudaError_t launch_multi(const ViewDesc* views, uint32_t nviews, uint32_t total_
 AddOrder add_order(const TableDev& t, bool backwards);
 bool sweep_pays_host(const TableDev& t, size_t vertices);
 
+// `wide`: ids of this insert may take all 32 bits, so that the stash has no bit
+// left for a cell's creator.
 cudaError_t launch_insert(const KeyConst& kc, const TableDev& t, const VertexPtrs& v, size_t n,
-                          uint32_t* stash, uint32_t* id_out, uint32_t tile_base, int batch, int merge,
-                          cudaStream_t st);
+                          uint32_t* stash, uint32_t* id_out, uint32_t unit_base, bool wide, int batch,
+                          int merge, cudaStream_t st);
 cudaError_t launch_query(const KeyConst& kc, const TableDev& t, const VertexPtrs& v, size_t n,
                          const uint32_t* id_in, const OutPtrs& o, bool blended, uint32_t id_limit,
                          cudaStream_t st);
@@ -99,8 +101,10 @@ cudaError_t launch_fused(const KeyConst& kc, const TableDev& t, const VertexPtrs
                          const OutPtrs& o, bool blend, float alpha, const FusedPlan& plan, uint32_t* stash, uint32_t* nq, cudaStream_t st);
 
 int sm_count();   // multiprocessors of the device
-int tile_size();  // vertices per warp tile of the split path
-int split_tile_ids();  // cell ids of such a tile's range
+// The split path hands out cell ids in units: ids per unit, and units that one
+// insert of n vertices takes.
+int split_unit_ids();
+size_t split_units(size_t n);
 // ... of the persistent kernels, for a launch over n vertices
 uint32_t fused_tile(size_t n, int batch);
 // Cells that the tiles' id ranges span (tiles of `tile` vertices).

@@ -30,8 +30,8 @@ namespace pps {
 namespace {
 
 constexpr int kBlock = 256;       // split kernels
-constexpr int kTile = 256;        // vertices per warp tile of the split path
-constexpr int kTileIds = kTile + 32 * 5;  // cell ids of its range (tile_ids, widest batch)
+constexpr int kTile = 256;        // vertices per warp tile of the split path, at least
+constexpr int kTileIds = kTile + 32 * 5;  // cell ids of a unit, such a tile's range (tile_ids, widest batch)
 constexpr int kFusedBlock = 512;  // persistent kernels
 constexpr int kFusedTile = 256;   // vertices per warp tile, large frames
 
@@ -131,7 +131,7 @@ struct WarpShared {
   float row[96];
 };
 
-constexpr uint32_t kDeferred = 0x7FFFFFFFu;  // cell id not known yet
+constexpr uint32_t kDeferred = 0xFFFFFFFEu;  // cell id not known yet
 
 // The most cell ids that a warp draws from the range of one tile of `v`
 // vertices, W vertices per lane and step: one for each new cell made while it
@@ -496,7 +496,9 @@ __device__ __forceinline__ void add_warp(const TableDev& t, const VertexPtrs& v,
 }
 
 // Pass two for two neighbouring vertices per lane, j and j + 1 (those below
-// `end`), FP32: equal cells' contributions are added up first.
+// `end`), on frames where nobody owns a cell (so that ids may take 32 bits):
+// equal cells' contributions are added up first.
+template <bool FIXED>
 __device__ __forceinline__ void add_pairs(const TableDev& t, const VertexPtrs& v, size_t j, size_t end,
                                           const uint32_t* stash) {
   uint32_t id[2];
@@ -505,19 +507,34 @@ __device__ __forceinline__ void add_pairs(const TableDev& t, const VertexPtrs& v
   for (int q = 0; q < 2; ++q) id[q] = j + q < end ? __ldcg(stash + j + q) : kOverflowSlot;
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
-    if (id[q] & kOwnerBit) continue;  // overflowed
+    if (id[q] == kOverflowSlot) continue;
     r[q] = __ldcs(v.r + j + q);
     g[q] = __ldcs(v.g + j + q);
     b[q] = __ldcs(v.b + j + q);
   }
-  const bool both = !(id[0] & kOwnerBit) && id[0] == id[1];
+  const bool both = id[0] != kOverflowSlot && id[0] == id[1];
+  long long fr[2] = {0, 0}, fg[2] = {0, 0}, fb[2] = {0, 0};
+  if (FIXED) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      if (id[q] != kOverflowSlot) {
+        fr[q] = to_fixed(r[q]);
+        fg[q] = to_fixed(g[q]);
+        fb[q] = to_fixed(b[q]);
+      }
+  }
   if (both) {
     r[0] = __fadd_rn(r[0], r[1]);
     g[0] = __fadd_rn(g[0], g[1]);
     b[0] = __fadd_rn(b[0], b[1]);
+    fr[0] += fr[1];
+    fg[0] += fg[1];
+    fb[0] += fb[1];
   }
-  if (!(id[0] & kOwnerBit)) accumulate<false>(t, id[0], r[0], g[0], b[0], 0, 0, 0, both ? 2u : 1u);
-  if (!(id[1] & kOwnerBit) && !both) accumulate<false>(t, id[1], r[1], g[1], b[1], 0, 0, 0, 1u);
+  if (id[0] != kOverflowSlot)
+    accumulate<FIXED>(t, id[0], r[0], g[0], b[0], fr[0], fg[0], fb[0], both ? 2u : 1u);
+  if (id[1] != kOverflowSlot && !both)
+    accumulate<FIXED>(t, id[1], r[1], g[1], b[1], fr[1], fg[1], fb[1], 1u);
 }
 
 // The cell id of a stash word (kOverflowSlot: probe overflow).
@@ -842,29 +859,32 @@ __device__ __forceinline__ void sweep_slots(const TableDev& t, size_t gid, size_
 }
 
 // ------------------------------------------------------------------ split path
-// Pass one of the insert, one warp per tile of kTile vertices; a tile's new
-// cells get ids from the tile's own range.
+// Pass one of the insert, one warp per tile of tile_v vertices; a tile's new
+// cells get ids from the tile's own range, `units` ranges of kTileIds ids from
+// unit_base on, whose counts (t.bcount) the later passes go by.
 template <int W, bool KREC>
 __global__ void __launch_bounds__(kBlock) k_insert(KeyConst kc, TableDev t, VertexPtrs v,
-                                                   size_t n, uint32_t* stash, uint32_t tile_base,
-                                                   uint32_t own, int merge) {
+                                                   size_t n, uint32_t* stash, uint32_t unit_base,
+                                                   uint32_t tile_v, uint32_t units, uint32_t own,
+                                                   int merge) {
   __shared__ WarpShared s_warp[kBlock / 32];
   __shared__ uint4 s_kw[KREC ? kBlock / 32 : 1][kQueue];
   WarpShared& sh = s_warp[threadIdx.x >> 5];
   uint4* qkw = s_kw[KREC ? threadIdx.x >> 5 : 0];
   WarpInsert<W> s;
-  const uint32_t tiles = static_cast<uint32_t>((n + kTile - 1) / kTile);
+  const uint32_t tiles = static_cast<uint32_t>((n + tile_v - 1) / tile_v);
   for (uint32_t tile = grid_warp(); tile < tiles; tile += grid_warps()) {
-    const uint32_t tix = tile_base + tile;
-    const size_t t0 = static_cast<size_t>(tile) * kTile, end = min(n, t0 + kTile);
+    const uint32_t unit = unit_base + tile * units;
+    const size_t t0 = static_cast<size_t>(tile) * tile_v, end = min(n, t0 + tile_v);
     s.claims = 0u;
-    s.id_base = tix * kTileIds;
+    s.id_base = unit * kTileIds;
 #pragma unroll 1
     for (size_t j0 = t0; j0 < end; j0 += 32 * W)
       insert_warp<W, true, KREC>(kc, t, v, j0, end, s, sh, true, own, merge, stash, qkw);
     if (tile + grid_warps() >= tiles)  // the warp's last
       while (s.queued) queue_step<W, KREC>(t, v, s, sh, true, own, stash, qkw);
-    if ((threadIdx.x & 31u) == 0u) t.bcount[tix] = s.claims;
+    for (uint32_t u = threadIdx.x & 31u; u < units; u += 32)
+      t.bcount[unit + u] = s.claims > u * kTileIds ? min(s.claims - u * kTileIds, static_cast<uint32_t>(kTileIds)) : 0u;
   }
   s.retire(t, true);
   const unsigned long long a = block_sum(static_cast<unsigned long long>(s.cnt.ovf));
@@ -877,8 +897,8 @@ __global__ void __launch_bounds__(kBlock) k_insert(KeyConst kc, TableDev t, Vert
 }
 
 // Pass two; id_out (nullable): the vertices' cell ids for the caller.
-// `ordered`: all contributions in the order of kPairsForwards, in tiles of 1,024
-// vertices, four to a thread.
+// `ordered`: nobody owns a cell, all contributions in the order of
+// kPairsForwards, in tiles of 1,024 vertices, four to a thread.
 __global__ void __launch_bounds__(kBlock) k_add(TableDev t, VertexPtrs v, size_t n, const uint32_t* stash,
                                                 uint32_t* id_out, int ordered, int merge) {
   __shared__ WarpShared s_warp[kBlock / 32];
@@ -886,10 +906,14 @@ __global__ void __launch_bounds__(kBlock) k_add(TableDev t, VertexPtrs v, size_t
   if (ordered) {
     for (size_t t0 = blockIdx.x * static_cast<size_t>(4 * kBlock); t0 < n; t0 += gridDim.x * static_cast<size_t>(4 * kBlock)) {
       const size_t j0 = t0 + 4 * threadIdx.x;
-      add_pairs(t, v, j0, n, stash);
-      add_pairs(t, v, j0 + 2, n, stash);
+      for (size_t j = j0; j < j0 + 4; j += 2) {
+        if (t.fixed)
+          add_pairs<true>(t, v, j, n, stash);
+        else
+          add_pairs<false>(t, v, j, n, stash);
+      }
       if (id_out)
-        for (size_t j = j0; j < min(n, j0 + 4); ++j) id_out[j] = stash_id(stash[j]);
+        for (size_t j = j0; j < min(n, j0 + 4); ++j) id_out[j] = stash[j];
     }
     return;
   }
@@ -1241,7 +1265,7 @@ __device__ __forceinline__ void add_ordered(const FusedArgs& a, WarpShared& sh) 
         add_warp_as<false, 2, kFusedBlock>(a.t, a.v, t0 + c + 32 * warp, a.n, a.stash, a.merge, sh);
         __syncthreads();
       } else {
-        add_pairs(a.t, a.v, t0 + c + 64 * warp + 2 * lane, a.n, a.stash);
+        add_pairs<false>(a.t, a.v, t0 + c + 64 * warp + 2 * lane, a.n, a.stash);
       }
     }
   }
@@ -1445,7 +1469,7 @@ __global__ void __launch_bounds__(BLOCK, (W == 4 ? 1 : 2) * (kFusedBlock / BLOCK
     const size_t end = min(static_cast<size_t>(vd.n), t0 + tile_v);
     const uint32_t* ids = a.stash + static_cast<size_t>(vd.tile_base) * tile_v;
     if (TEMPORAL && vd.ordered)
-      for (size_t j = t0; j < end; j += 64) add_pairs(vd.t, vd.v, j + 2 * lane, end, ids);
+      for (size_t j = t0; j < end; j += 64) add_pairs<false>(vd.t, vd.v, j + 2 * lane, end, ids);
     else
       for (size_t j = t0; j < end; j += 128) add_warp(vd.t, vd.v, j, end, ids, 2, sh);
   };
@@ -1516,8 +1540,23 @@ int sm_count() {
   return cached;
 }
 
-int tile_size() { return kTile; }
-int split_tile_ids() { return kTileIds; }
+int split_unit_ids() { return kTileIds; }
+
+// Vertices per warp tile of the split path: 256, or more on frames so large that
+// every warp still gets tiles enough; a larger tile wastes fewer ids on those its
+// warp keeps in reserve (1.63 ids a vertex for 256 vertices, 1.22 for 1,024, 1.12 for
+// 4,096, 1.02 for 16,384).
+static uint32_t split_tile(size_t n) {
+  uint32_t v = kTile;
+  while (v < 16384u && n >= static_cast<size_t>(v) * 4 * 16384) v *= 4;
+  return v;
+}
+static uint32_t tile_units(uint32_t tile_v) { return (tile_ids(tile_v, 4) + kTileIds - 1) / kTileIds; }
+
+size_t split_units(size_t n) {
+  const uint32_t v = split_tile(n);
+  return (n + v - 1) / v * tile_units(v);
+}
 size_t fused_cells(size_t n, uint32_t tile, int batch) {
   return (n + tile - 1) / tile * tile_ids(tile, batch);
 }
@@ -1545,21 +1584,22 @@ static bool vec_outputs(const OutPtrs& o) {
 }
 
 cudaError_t launch_insert(const KeyConst& kc, const TableDev& t, const VertexPtrs& v, size_t n,
-                          uint32_t* stash, uint32_t* id_out, uint32_t tile_base, int batch, int merge,
-                          cudaStream_t st) {
+                          uint32_t* stash, uint32_t* id_out, uint32_t unit_base, bool wide, int batch,
+                          int merge, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  const int grid = split_grid((n + kTile - 1) / kTile * 32);
-  const bool ordered = add_order(t, false) != kAnyOrder;
+  const uint32_t tile_v = split_tile(n), units = tile_units(tile_v);
+  const int grid = split_grid((n + tile_v - 1) / tile_v * 32);
+  const bool ordered = wide || add_order(t, false) != kAnyOrder;
   const uint32_t own = ordered ? 0u : kOwnerBit;
   if (t.hist_migrate || t.normal_search) {  // keep each new cell's quantized key
     if (batch == 2)
-      k_insert<2, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, own, merge);
+      k_insert<2, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, unit_base, tile_v, units, own, merge);
     else
-      k_insert<4, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, own, merge);
+      k_insert<4, true><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, unit_base, tile_v, units, own, merge);
   } else if (batch == 2) {
-    k_insert<2, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, own, merge);
+    k_insert<2, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, unit_base, tile_v, units, own, merge);
   } else {
-    k_insert<4, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, tile_base, own, merge);
+    k_insert<4, false><<<grid, kBlock, 0, st>>>(kc, t, v, n, stash, unit_base, tile_v, units, own, merge);
   }
   k_add<<<split_grid((n + 127) / 128 * 32), kBlock, 0, st>>>(t, v, n, stash, id_out, ordered ? 1 : 0,
                                                             merge);

@@ -129,6 +129,7 @@ SIGNATURES = {
     "pps_batch_run": ([_vp, ctypes.POINTER(pps_camera), _u32, _vp], ctypes.c_int),
     "pps_batch_destroy": ([_vp], ctypes.c_int),
     "pps_selftest_infer": ([ctypes.c_int, _u32, ctypes.POINTER(_u32)], ctypes.c_int),
+    "pps_selftest_wide_ids": ([_vp, ctypes.c_int], ctypes.c_int),
     "pps_selftest_wait": ([ctypes.c_int, _u32, ctypes.POINTER(_u32)], ctypes.c_int),
     "pps_bench_rate": ([ctypes.c_int, ctypes.c_size_t, ctypes.c_size_t, _vp, _vp,
                         ctypes.POINTER(ctypes.c_double)], ctypes.c_int),
@@ -237,6 +238,10 @@ def camera(pos: Sequence[float]) -> pps_camera:
 # ---------------------------------------------------------------- C-named calls
 def pps_version() -> str:
     return lib().pps_version().decode()
+
+
+def pps_selftest_wide_ids(handle: int, on: bool) -> None:
+    _check(lib().pps_selftest_wide_ids(handle, int(on)))
 
 
 def pps_selftest_infer(row: int, tiles: int) -> int:
