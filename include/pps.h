@@ -419,7 +419,7 @@ int pps_keys(pps_table *t, const pps_vertices *v, size_t n, uint32_t *h_out, uin
  * pps_filter on a table created from `p` (FP32 atomics: equal up to
  * summation order).
  *  - Working memory is one static device array inside the library (about
- *    33 MB), held by every GPU that loads the library until the process exits.
+ *    22 MB), held by every GPU that loads the library until the process exits.
  *    Limits: log2_slots <= 20 and n <= 524,288; larger requests, another
  *    accum_mode, or a history return PPS_EINVAL.
  *  - The first call in a CUDA context (the device's primary context, that

@@ -555,6 +555,7 @@ int filter_one(pps_table* t, const pps_camera* cam, uint32_t frame, const pps_ve
   set_camera(t, cam, frame);
   if (n == 0) return reset_frame(t, st);
   plan.sweep = pps::sweep_pays_host(t->dev, n);
+  if (plan.sweep || t->leaves) plan.swept = t->T;
   if (!plan.sweep)
     if (int rc = empty_frame(t, st)) return rc;
   auto ready = [&]() -> int {

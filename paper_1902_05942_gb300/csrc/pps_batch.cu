@@ -79,7 +79,7 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
   cudaGetDevice(&b->device);
   b->alpha = alpha;
   int batch = 2, block = 512;
-  size_t total = 0, own_words = 0;
+  size_t total = 0, own_words = 0, swept = 0;
   for (uint32_t i = 0; i < nviews; ++i) {
     const pps_view& v = views[i];
     if (!v.table || !v.out.r || !v.out.g || !v.out.b || (v.n && (!v.v.px || !v.v.py || !v.v.pz ||
@@ -114,6 +114,7 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
       plan.merge = 2;
       plan.temporal = vd.blended != 0;
       plan.sweep = vd.sweep != 0;
+      plan.swept = static_cast<size_t>(vd.t.mask) + 1;
       if (vd.ordered) plan.order = pps::kPairsForwards;
       b->own.push_back(pps_batch::OwnView{i, v.table, vd, plan});
       own_words = std::max<size_t>(own_words, v.n);
@@ -121,6 +122,7 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
       b->temporal = b->temporal || tmp;
       b->ordered = b->ordered || vd.ordered;
       total += v.n;
+      swept += static_cast<size_t>(vd.t.mask) + 1;
       b->base.push_back(vd);
       b->index.push_back(i);
       b->tables.push_back(v.table);
@@ -154,7 +156,7 @@ int pps_batch_create(pps_batch** out, const pps_view* views, uint32_t nviews, in
   }
   const int graphs = nshared ? 2 : 0;
   if (e == cudaSuccess && nshared)
-    e = pps::plan_multi(b->total_tiles, tile, b->temporal, batch, block, &b->plan);
+    e = pps::plan_multi(b->total_tiles, tile, swept, b->temporal, batch, block, &b->plan);
   const size_t bytes = nshared * sizeof(pps::ViewDesc);
   for (int k = 0; k < graphs && e == cudaSuccess; ++k) {
     e = cudaMalloc(&b->dviews[k], bytes);

@@ -31,6 +31,7 @@ struct FusedPlan {
   bool neigh = false;     // ... the neighborhood search
   bool kv = false;        // ... vertices with key variants
   bool sweep = false;     // zero the whole slot table first, not the frame's slots at the end
+  size_t swept = 0;       // slots the launch zeroes, or may find left over and have to zero
   int merge = 2;      // merging of equal keys within a warp (pps_tuning.merge)
   bool backwards = false;  // insert from the end of the vertex stream
   AddOrder order = kAnyOrder;
@@ -57,11 +58,11 @@ struct MultiPlan {
 };
 
 // Plan / launch the batched persistent kernel over `total_tiles` warp tiles of
-// `tile` vertices of the views in device memory (`views`, nviews entries);
+// `tile` vertices (`swept`: slots of all tables) of the views in device memory (`views`, nviews entries);
 // `ctrl` carries the grid barrier, `stash` (total_tiles
 // tiles) the vertices' cell ids.
-cudaError_t plan_multi(size_t total_tiles, uint32_t tile, bool temporal, int batch, int block,
-                       MultiPlan* plan);
+cudaError_t plan_multi(size_t total_tiles, uint32_t tile, size_t swept, bool temporal, int batch,
+                       int block, MultiPlan* plan);
 cudaError_t launch_multi(const ViewDesc* views, uint32_t nviews, uint32_t total_tiles, Ctrl* ctrl,
                          bool temporal, bool ordered, float alpha, const MultiPlan& plan,
                          uint32_t* stash, cudaStream_t st);

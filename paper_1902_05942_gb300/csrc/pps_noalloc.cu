@@ -44,20 +44,20 @@ constexpr uint32_t kNoAllocMaxLog2Slots = 20;                // up to 2^20 slots
 constexpr size_t kNoAllocMaxVertices = size_t{1} << 19;      // up to 524,288 vertices
 
 constexpr size_t kSlotBytes = (size_t{1} << kNoAllocMaxLog2Slots) * sizeof(unsigned long long);
-// Cells the id ranges of the warp tiles may span (pps::fused_cells): 64
-// vertices per tile up to 131,072 vertices, 128 up to 262,144, 256 beyond.
-constexpr size_t kNoAllocMaxCells = (size_t{1} << 19) / 256 * (256 + 96);
+// Cells the id ranges of the warp tiles may span: those of the largest call in
+// tiles of 256 vertices.  Smaller calls take tiles of 64 or 128 vertices, whose
+// ranges are wider for their size, as long as they fit (pps::plan_fused).  The
+// launch sweeps and does not blend, so it keeps no records of the cells.
+constexpr size_t kNoAllocMaxCells = kNoAllocMaxVertices / 256 * (256 + 96);
 constexpr size_t kAccBytes = kNoAllocMaxCells * sizeof(float4);
-constexpr size_t kInfoBytes = kNoAllocMaxCells * sizeof(uint4);
 constexpr size_t kStashBytes = kNoAllocMaxVertices * sizeof(uint32_t);
 constexpr size_t kCountBytes = kNoAllocMaxVertices / 64 * sizeof(uint32_t);  // cells per warp tile
 constexpr size_t kCtrlBytes = 256;
 constexpr size_t kOffAcc = kSlotBytes;
-constexpr size_t kOffInfo = kOffAcc + kAccBytes;
-constexpr size_t kOffStash = kOffInfo + kInfoBytes;
+constexpr size_t kOffStash = kOffAcc + kAccBytes;
 constexpr size_t kOffCount = kOffStash + kStashBytes;
 constexpr size_t kOffCtrl = kOffCount + kCountBytes;
-constexpr size_t kScratchBytes = kOffCtrl + kCtrlBytes;  // about 33 MB
+constexpr size_t kScratchBytes = kOffCtrl + kCtrlBytes;  // about 22 MB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -166,6 +166,7 @@ extern "C" int pps_filter_noalloc(const pps_params* p, const pps_camera* cam, ui
   const uint32_t T = 1u << p->log2_slots;
   pps::FusedPlan plan;
   plan.sweep = true;
+  plan.swept = size_t{1} << p->log2_slots;
   plan.backwards = true;
   cudaError_t e = pps::plan_fused(n, kNoAllocMaxCells, &plan);
   if (e != cudaSuccess)
@@ -174,7 +175,6 @@ extern "C" int pps_filter_noalloc(const pps_params* p, const pps_camera* cam, ui
   pps::TableDev t{};
   t.slots = reinterpret_cast<unsigned long long*>(base);
   t.acc = reinterpret_cast<float4*>(base + kOffAcc);
-  t.info = reinterpret_cast<uint4*>(base + kOffInfo);
   t.bcount = reinterpret_cast<uint32_t*>(base + kOffCount);
   t.ctrl = reinterpret_cast<pps::Ctrl*>(base + kOffCtrl);
   t.mask = T - 1;
