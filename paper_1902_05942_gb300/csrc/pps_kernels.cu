@@ -113,10 +113,19 @@ struct Counters {
 // Queue entries per warp: a step's worth that may stay, and the keys of two rows.
 constexpr int kQueue = 96;
 
-// Tables far larger than L2 read the home slot before they try to take it: a
-// compare-and-swap that fails still costs the sector's way back to DRAM (random
-// compare-and-swaps 23 G/s on a 1 GB table, loads 43 G/s).  They also empty the
-// queue after every step, whose sectors are then still in L2.  
+// Tables of 2^24 and 2^25 slots, larger than L2 but not by much, read the home
+// slot before they try to take it: a compare-and-swap that fails still costs the
+// sector's way back to DRAM (random compare-and-swaps 23 G/s on a 1 GB table, loads
+// 43 G/s).  Frames without history, without and with the read, us: 2^23 slots 328
+// and 341 (9.0 M vertices); 2^24 362 and 354 (9.0 M), 594 and 580 (14.9 M), 1,022 and
+// 967 (17.2 M, load 0.8); 2^25 413 and 400, 656 and 640, 2,260 and 2,124 (34.4 M, load
+// 0.8); 2^26 1,874 and 2,037 (34.4 M), 3,840 and 4,050 (61 M).
+constexpr uint32_t kLookFrom = (1u << 24) - 1u, kLookTo = (1u << 25) - 1u;  // slots - 1
+
+// Tables from 2^25 slots on empty the queue after every step, while the sectors of
+// the keys' home slots are still in L2.  Without and with that, us: 2^24 slots 362
+// and 378 (9.0 M vertices), 594 and 627 (14.9 M); 2^25 414 and 413, 654 and 656, 2,322
+// and 2,260 (34.4 M); 2^26 2,037 and 1,874 (34.4 M), 4,066 and 3,841 (61 M).
 constexpr uint32_t kLargeTable = (1u << 25) - 1u;  // slots - 1
 
 // Shared memory of one warp: its queue of keys, and the contributions of a row
@@ -357,7 +366,7 @@ __device__ __forceinline__ void insert_warp(const KeyConst& kc, const TableDev& 
     s.reserve(q, lead >> q & 1u);
   }
   unsigned long long old[W];
-  const bool look = t.mask >= kLargeTable;
+  const bool look = t.mask >= kLookFrom && t.mask <= kLookTo;
 #pragma unroll
   for (int q = 0; q < W; ++q) {
     old[q] = 0ull;
