@@ -396,7 +396,8 @@ int pps_filter_host_async(pps_table *t, const pps_camera *cam, uint32_t frame,
 int pps_host_wait(pps_table *t);
 
 /* pps_set_tuning / pps_get_tuning: set or read the launch shape (pps_tuning).
- * Results do not depend on it.  Errors: PPS_EINVAL. */
+ * Results do not depend on it.  batch, block and merge read as the values in
+ * effect, the other fields as they were set.  Errors: PPS_EINVAL. */
 int pps_set_tuning(pps_table *t, const pps_tuning *tune);
 int pps_get_tuning(pps_table *t, pps_tuning *tune);
 

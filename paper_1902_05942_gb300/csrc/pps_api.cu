@@ -840,9 +840,7 @@ int pps_get_tuning(pps_table* t, pps_tuning* tune) {
   if (!tune) return fail(PPS_EINVAL, "tuning is NULL");
   *tune = t->tune;
   tune->batch = static_cast<uint32_t>(batch_of(t));
-  // one insert serves every table; the fields read as they always did
-  tune->insert = t->tune.insert ? t->tune.insert : t->T > (1u << 23) ? 1u : 2u;
-  tune->key_warps = t->tune.key_warps ? t->tune.key_warps : 8u;
+  // (insert and key_warps have no effect: what was set, or 0)
   tune->block = t->tune.block ? t->tune.block : 512u;
   tune->merge = static_cast<uint32_t>(merge_of(t));
   return PPS_OK;
