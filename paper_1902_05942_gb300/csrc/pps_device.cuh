@@ -291,8 +291,8 @@ __device__ __forceinline__ KeyWords key_words(const KeyConst& kc, float px, floa
   if (kc.jitter) {
     // jitter(n): a point of the tangent plane, (u, w) uniform in [-0.5, 0.5)
     const uint2 rnd = philox_first2_rk(id, stream_id, kc);
-    // (products with powers of two, and with s = +-1, are exact: the fused
-    // forms below round once, like the separate operations)
+    // (products of 24-bit integers with 2^-24, and with s = +-1, are exact: the
+    // fused forms round once, like the separate operations)
     const float u = __fmaf_rn(__uint2float_rn(rnd.x >> 8), 0x1p-24f, -0.5f);
     const float w = __fmaf_rn(__uint2float_rn(rnd.y >> 8), 0x1p-24f, -0.5f);
     // tangent frame after Duff et al. (JCGT 2017)
@@ -306,9 +306,10 @@ __device__ __forceinline__ KeyWords key_words(const KeyConst& kc, float px, floa
     const float by = __fadd_rn(s, __fmul_rn(__fmul_rn(ny, ny), a));
     const float bz = -ny;
     const float E = pow2_int(l0);  // voxel edge at the pre-jitter level
-    xj = __fmaf_rn(__fadd_rn(__fmul_rn(u, tx), __fmul_rn(w, bx)), E, px);
-    yj = __fmaf_rn(__fadd_rn(__fmul_rn(u, ty), __fmul_rn(w, by)), E, py);
-    zj = __fmaf_rn(__fadd_rn(__fmul_rn(u, tz), __fmul_rn(w, bz)), E, pz);
+    // (not fused: the product with E is exact only between underflow and overflow)
+    xj = __fadd_rn(px, __fmul_rn(__fadd_rn(__fmul_rn(u, tx), __fmul_rn(w, bx)), E));
+    yj = __fadd_rn(py, __fmul_rn(__fadd_rn(__fmul_rn(u, ty), __fmul_rn(w, by)), E));
+    zj = __fadd_rn(pz, __fmul_rn(__fadd_rn(__fmul_rn(u, tz), __fmul_rn(w, bz)), E));
     l1 = ke.dist ? level_at(kc, __fadd_rn(__fsub_rn(__ldg(ke.dist + ke.j),
                                                     camera_distance(kc, px, py, pz)),
                                           camera_distance(kc, xj, yj, zj)))
