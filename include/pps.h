@@ -216,8 +216,9 @@ typedef struct pps_camera {
  *             choice for every call on a table in a frame.
  * pps_batch_create, pps_filter_noalloc and the host-buffer calls reject dist
  * and extra.
- * All nine float arrays are required.  16-byte-aligned arrays are read with
- * 128-bit loads; other alignments take a scalar path.
+ * All nine float arrays are required.  They are read 32 bits a vertex, a warp's
+ * loads of an array adjoining; pps_query without slot_in reads 16-byte-aligned
+ * arrays with 128-bit loads, others by a scalar path.
  */
 typedef struct pps_vertices {
   const float *px, *py, *pz;

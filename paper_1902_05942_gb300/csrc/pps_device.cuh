@@ -68,8 +68,7 @@ struct Ctrl {
   unsigned int bar_count;
   unsigned int pad[2];
 };
-constexpr size_t kCtrlFrameBytes = 6 * sizeof(unsigned long long);  // the counters, reset per frame
-constexpr size_t kCtrlEmptyBytes = 7 * sizeof(unsigned long long);  // and `left`, once the slots are empty
+constexpr size_t kCtrlEmptyBytes = 7 * sizeof(unsigned long long);  // counters and `left`: zero once the slots are empty
 constexpr size_t kCtrlErrorBytes = 2 * sizeof(unsigned int);        // error word and barrier, from `error` on
 
 enum : unsigned int {
@@ -742,36 +741,25 @@ struct Result {
   uint8_t status;
 };
 
-template <int W>
+// The results of the four vertices from j on (those below `end`).
 __device__ __forceinline__ void store_batch(const OutPtrs& o, size_t j, size_t end, bool vec,
-                                            const Result (&res)[W]) {
-  if (vec && j + W <= end) {
-    if constexpr (W == 4) {
-      __stcs(reinterpret_cast<float4*>(o.r + j), make_float4(res[0].r, res[1].r, res[2].r, res[3].r));
-      __stcs(reinterpret_cast<float4*>(o.g + j), make_float4(res[0].g, res[1].g, res[2].g, res[3].g));
-      __stcs(reinterpret_cast<float4*>(o.b + j), make_float4(res[0].b, res[1].b, res[2].b, res[3].b));
-      if (o.count)
-        __stcs(reinterpret_cast<uint4*>(o.count + j),
-               make_uint4(res[0].n, res[1].n, res[2].n, res[3].n));
-      if (o.status) {
-        const uint32_t w = res[0].status | (res[1].status << 8) | (res[2].status << 16) |
-                           (static_cast<uint32_t>(res[3].status) << 24);
-        __stcs(reinterpret_cast<unsigned int*>(o.status + j), w);
-      }
-    } else {
-      __stcs(reinterpret_cast<float2*>(o.r + j), make_float2(res[0].r, res[1].r));
-      __stcs(reinterpret_cast<float2*>(o.g + j), make_float2(res[0].g, res[1].g));
-      __stcs(reinterpret_cast<float2*>(o.b + j), make_float2(res[0].b, res[1].b));
-      if (o.count) __stcs(reinterpret_cast<uint2*>(o.count + j), make_uint2(res[0].n, res[1].n));
-      if (o.status) {
-        const unsigned short w = static_cast<unsigned short>(res[0].status | (res[1].status << 8));
-        __stcs(reinterpret_cast<unsigned short*>(o.status + j), w);
-      }
+                                            const Result (&res)[4]) {
+  if (vec && j + 4 <= end) {
+    __stcs(reinterpret_cast<float4*>(o.r + j), make_float4(res[0].r, res[1].r, res[2].r, res[3].r));
+    __stcs(reinterpret_cast<float4*>(o.g + j), make_float4(res[0].g, res[1].g, res[2].g, res[3].g));
+    __stcs(reinterpret_cast<float4*>(o.b + j), make_float4(res[0].b, res[1].b, res[2].b, res[3].b));
+    if (o.count)
+      __stcs(reinterpret_cast<uint4*>(o.count + j),
+             make_uint4(res[0].n, res[1].n, res[2].n, res[3].n));
+    if (o.status) {
+      const uint32_t w = res[0].status | (res[1].status << 8) | (res[2].status << 16) |
+                         (static_cast<uint32_t>(res[3].status) << 24);
+      __stcs(reinterpret_cast<unsigned int*>(o.status + j), w);
     }
     return;
   }
 #pragma unroll
-  for (int q = 0; q < W; ++q) {
+  for (int q = 0; q < 4; ++q) {
     if (j + q < end) {
       o.r[j + q] = res[q].r;
       o.g[j + q] = res[q].g;

@@ -974,7 +974,7 @@ __global__ void __launch_bounds__(kBlock) k_query(KeyConst kc, TableDev t, Verte
       for (int q = 0; q < 4; ++q)
         if (j + q < n && id[q] != kOverflowSlot) res[q] = similar_pool(t, id[q], blended != 0);
     }
-    store_batch<4>(o, j, n, ovec != 0, res);
+    store_batch(o, j, n, ovec != 0, res);
     if (t.neighbors) {
 #pragma unroll
       for (int q = 0; q < 4; ++q)
