@@ -98,13 +98,15 @@ struct Counters {
 // A key that waits there loses its place: later keys fill the slots it would
 // have had, and more keys run out of probes (5.06 M vertices, 2^22 slots, 16
 // probes: 0.178 % of the vertices, 0.128 % where every key is finished at once).
-// So a warp that has seen a key use up a sixth of its probes, which in a table
-// with few collisions hardly ever happens, empties its queue after every step
-// from then on: 0.122 % at 242 us instead of 196; the oldest entries first instead
-// left 0.171 %.  With 8 probes 1.11 % become 0.95 % (at once 0.99 %).  With a quarter
-// of the probes instead of a sixth, 2.94 M vertices in 2^22 slots lost 253 vertices
-// at 64 probes, 225 like this, 219 at once; with an eighth no fewer, but on 9 M
-// vertices with few collisions (2^23 slots, 64 probes) 351 us instead of 337.
+// So a warp that has seen a key use up a sixth of its probes empties its queue
+// after every step from then on: 0.122 % at 242 us instead of 196; the oldest
+// entries first instead left 0.171 %.  With 8 probes 1.11 % become 0.95 % (at once
+// 0.99 %).  With a quarter of the probes instead of a sixth, 2.94 M vertices in 2^22
+// slots lost 253 vertices at 64 probes, 225 like this, 219 at once; with an eighth
+// no fewer, but on 9 M vertices with few collisions (2^23 slots, 64 probes) 351 us
+// instead of 337.  Where the limit is short such keys are common and the time is
+// spent on tables that lose next to nothing, too: 2^23 slots, 16 probes 191 -> 216
+// us, temporal 354 -> 372; with 64 probes 190 -> 193 and 354 -> 350.
 //
 // What bounds pass one now is the keys: without any table access it takes
 // 84 us (about 330 instructions per vertex at 8 warps per scheduler, 64
