@@ -69,7 +69,8 @@ def _overflow_at_once(home, fp, log2_slots, probes, chunk=16384):
 def test_no_more_overflow_than_with_every_key_finished_at_once(probes):
     """2^22 slots filled to 0.7.  The share is a sum over long runs of slots:
     four standard deviations of a count, and 4 % for the different order of
-    keys that are in flight together."""
+    keys that are in flight together.  The order is another in every run, and
+    with it the count (by 5 of 230, by 16 of 3,700): the median of five."""
     log2_slots, n = 22, int(0.7 * (1 << 22))
     v = _stream(n)
     tab = pps.Table(_cfg(log2_slots, probes))
@@ -79,9 +80,12 @@ def test_no_more_overflow_than_with_every_key_finished_at_once(probes):
     got = []
     for batch in (2, 4):
         tab.tune(batch)
-        out = tab.filter(v, EYE, 0)
-        got.append(tab.stats()["overflow_vertices"])
-        assert got[-1] == int((out["status"] == 2).sum())
+        lost = []
+        for _ in range(5):
+            out = tab.filter(v, EYE, 0)
+            lost.append(tab.stats()["overflow_vertices"])
+            assert lost[-1] == int((out["status"] == 2).sum())
+        got.append(sorted(lost)[2])
     tab.close()
     assert max(got) <= 1.04 * want + 4 * want ** 0.5, (got, want)
 
